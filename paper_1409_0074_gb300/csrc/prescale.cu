@@ -13,12 +13,24 @@
 // One evaluation: the gathered subset rows -> K (n x n, binary64) -> K^{-1}
 // in place by Gauss-Jordan elimination without pivoting (K is symmetric
 // positive definite; the pivots are the successive Schur complements, so
-// their logs sum to log|K|), one launch per pivot with the pivot's row,
-// column and reciprocal double-buffered so that no launch reads what it
-// writes -> alpha ->
+// their logs sum to log|K|), in panels of 32 pivots (below) -> alpha ->
 // per-row partial sums of the trace and quadratic-form terms (one warp per
 // row, fixed order) -> the likelihood and its gradient in eta = log theta on
-// one thread, which also advances the maximiser.
+// one warp, whose first lane also advances the maximiser.
+//
+// Panels.  Step k of the elimination is, with m_i = -A_ik / A_kk and r_j = A_kj
+// as they are before the step,
+//   A_ij <- m_i r_j + A_ij,  A_ik <- m_i,  A_kj <- r_j / A_kk,  A_kk <- 1 / A_kk.
+// The 32 steps of a panel run first on its diagonal block (gj_diag_block: one
+// CTA), then on the panel's columns and rows (gj_panels: a warp per row or
+// column, every m_i^(k) and r_j^(k) kept), and then all at once, in the same
+// order, on the rest (gj_rest: a rank-32 update from registers and shared
+// memory).  Every element sees the operations of the one-pivot-per-launch form
+// in the same order, so K^{-1} has the same bits; it is read and written once
+// per panel instead of once per pivot, in 2 launches instead of 32.  The rest
+// is bound by the FP64 pipe (n^3 multiply-adds, two per SM and cycle); the
+// next panel's diagonal block, a chain of 32 dependent divisions, runs beside
+// it on an SM of its own (block 0 of gj_rest).
 //
 // Maximiser: BFGS on eta from eta0 = log theta0 (inverse curvature H = I at
 // the start), ascent direction d = H grad scaled so that no coordinate moves
@@ -41,6 +53,8 @@ namespace lagp {
 #define SEP_MAX_N 1024
 #define SEP_MAX_P 16
 #define SEP_TOL 1e-9
+#define GJ_NB 32             // pivots per panel
+#define GJ_THREADS 512       // gj_rest: one 32 x 32 tile at a time, two elements per thread
 
 enum { SEP_INIT = 0, SEP_TRIAL = 1 };
 
@@ -58,8 +72,10 @@ struct SepWork {
   double* S;       // [n][p] subset rows
   double* ys;      // [n]
   double* A;       // [n][n] K, then K^{-1}
-  double* snap;    // [2][2][n] pivot column / row of the current and next step, then
-                   // [2] the reciprocal pivot of the current and next step
+  double* dm;      // [32][32] m_i^(k) of the panel's diagonal block (the reciprocal pivot at i = k)
+  double* dr;      // [32][32] r_j^(k) of the diagonal block, row k
+  double* pm;      // [n][32] m_i^(k) of the rows outside the panel
+  double* pr;      // [n][32] r_j^(k) of the columns outside the panel
   double* piv;     // [n]
   double* alpha;   // [n]
   double* part;    // [n][2p] per-row partial sums
@@ -79,7 +95,10 @@ static size_t sep_layout(int n, int p, char* base, SepWork* w) {
   t.S = reinterpret_cast<double*>(take(sizeof(double) * n * p));
   t.ys = reinterpret_cast<double*>(take(sizeof(double) * n));
   t.A = reinterpret_cast<double*>(take(sizeof(double) * n * n));
-  t.snap = reinterpret_cast<double*>(take(sizeof(double) * (4 * n + 2)));
+  t.dm = reinterpret_cast<double*>(take(sizeof(double) * GJ_NB * GJ_NB));
+  t.dr = reinterpret_cast<double*>(take(sizeof(double) * GJ_NB * GJ_NB));
+  t.pm = reinterpret_cast<double*>(take(sizeof(double) * n * GJ_NB));
+  t.pr = reinterpret_cast<double*>(take(sizeof(double) * n * GJ_NB));
   t.piv = reinterpret_cast<double*>(take(sizeof(double) * n));
   t.alpha = reinterpret_cast<double*>(take(sizeof(double) * n));
   t.part = reinterpret_cast<double*>(take(sizeof(double) * n * 2 * p));
@@ -120,7 +139,7 @@ __device__ __forceinline__ double sep_corr(const double* a, const double* b, int
   return exp(-s);
 }
 
-// K at theta = exp(eta_t), and the first pivot row / column
+// K at theta = exp(eta_t)
 __global__ void sep_build(int n, int p, double g, SepWork w) {
   if (w.st->done) return;
   double ith[SEP_MAX_P];
@@ -129,40 +148,151 @@ __global__ void sep_build(int n, int p, double g, SepWork w) {
   if (a >= n || b >= n) return;
   const double v = (a == b) ? 1.0 + g : sep_corr(w.S + (int64_t)a * p, w.S + (int64_t)b * p, p, ith);
   w.A[(int64_t)a * n + b] = v;
-  if (b == 0) w.snap[a] = v;            // column 0
-  if (a == 0) w.snap[n + b] = v;        // row 0
-  if (a == 0 && b == 0) w.snap[4 * n] = 1.0 / v;
 }
 
-// Gauss-Jordan step k: every element from its own value and the pivot's
-// column (cin) and row (rin) as they were before the step, with the pivot's
-// reciprocal computed once by the previous step; the new column and row
-// k + 1 go to cout / rout, and the thread that forms the next pivot also
-// forms its reciprocal, for the next step.
-__global__ void gj_step(int n, int k, SepWork w) {
-  if (w.st->done) return;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= n || j >= n) return;
-  const double* cin = w.snap + (k & 1) * 2 * n;
-  const double* rin = cin + n;
-  double* cout = w.snap + ((k + 1) & 1) * 2 * n;
-  double* rout = cout + n;
-  const double pi = w.snap[4 * n + (k & 1)];
-  double v;
-  if (i == k && j == k) {
-    v = pi;
-    w.piv[k] = rin[k];
-  } else if (j == k) {
-    v = -cin[i] * pi;
-  } else if (i == k) {
-    v = rin[j] * pi;
-  } else {
-    v = fma(-cin[i] * pi, rin[j], w.A[(int64_t)i * n + j]);
+__device__ __forceinline__ double shfl_d(double v, int src) {
+  return __shfl_sync(0xffffffffu, v, src);
+}
+
+// The panel's steps on its diagonal block at pivot K0: warp g of 16 holds rows
+// g and g + 16, lane c column c (elements past n unused).  The steps' m and r
+// go to w.dm and w.dr, the pivots to w.piv, and the block to A.
+__device__ void gj_diag_block(int n, int K0, double d0, double d1, SepWork w) {
+  __shared__ double rowbuf[2][GJ_NB], pibuf[2];
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int nb = min(GJ_NB, n - K0);
+  for (int k = 0; k < nb; ++k) {
+    const int f = k & 1;
+    if ((k & 15) == g) {            // the pivot row's warp
+      const double v = k < 16 ? d0 : d1;
+      const double p = 1.0 / shfl_d(v, k);
+      rowbuf[f][lane] = v;
+      w.dr[k * GJ_NB + lane] = v;
+      if (lane == k) { pibuf[f] = p; w.piv[K0 + k] = v; }
+    }
+    __syncthreads();
+    const double r = rowbuf[f][lane], pi = pibuf[f];
+    const double c0 = shfl_d(d0, k), c1 = shfl_d(d1, k);
+    const double m = -((lane & 1) ? c1 : c0) * pi;
+    const double m0 = g == k ? pi : shfl_d(m, 0), m1 = g + 16 == k ? pi : shfl_d(m, 1);
+    // the pivot row is r pi = r pi - 0
+    d0 = lane == k ? m0 : fma(m0, r, g == k ? -0.0 : d0);
+    d1 = lane == k ? m1 : fma(m1, r, g + 16 == k ? -0.0 : d1);
+    if (lane < 2) w.dm[(g + 16 * lane) * GJ_NB + k] = lane ? m1 : m0;
   }
-  w.A[(int64_t)i * n + j] = v;
-  if (j == k + 1) cout[i] = v;
-  if (i == k + 1) rout[j] = v;
-  if (i == k + 1 && j == k + 1) w.snap[4 * n + ((k + 1) & 1)] = 1.0 / v;
+  if (lane < nb && g < nb) w.A[(int64_t)(K0 + g) * n + K0 + lane] = d0;
+  if (lane < nb && g + 16 < nb) w.A[(int64_t)(K0 + g + 16) * n + K0 + lane] = d1;
+}
+
+// The first panel's diagonal block (one CTA of GJ_THREADS).
+__global__ void __launch_bounds__(GJ_THREADS) gj_first(int n, SepWork w) {
+  if (w.st->done) return;
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const double d0 = lane < n && g < n ? w.A[(int64_t)g * n + lane] : 0.0;
+  const double d1 = lane < n && g + 16 < n ? w.A[(int64_t)(g + 16) * n + lane] : 0.0;
+  gj_diag_block(n, 0, d0, d1, w);
+}
+
+// The panel's steps on the rows and columns outside its block: one warp per
+// row i (lane: panel column; elements A_i,K0..) or column j (lane: panel row).
+__global__ void __launch_bounds__(256) gj_panels(int n, int K0, SepWork w) {
+  if (w.st->done) return;
+  __shared__ double dm[GJ_NB][GJ_NB + 1], dr[GJ_NB][GJ_NB + 1];
+  for (int e = threadIdx.x; e < GJ_NB * GJ_NB; e += blockDim.x) {
+    dm[e / GJ_NB][e % GJ_NB] = w.dm[e];
+    dr[e / GJ_NB][e % GJ_NB] = w.dr[e];
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, nb = min(GJ_NB, n - K0);
+  const int item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int out = n - nb;                            // rows, then columns, outside the block
+  if (item >= 2 * out) return;
+  const bool col = item >= out;
+  int x = col ? item - out : item;
+  if (x >= K0) x += nb;
+  const bool in = lane < nb;
+  double* el = col ? w.A + (int64_t)(K0 + lane) * n + x : w.A + (int64_t)x * n + K0 + lane;
+  double v = in ? *el : 0.0, kept = 0.0;
+  if (col) {
+    for (int k = 0; k < nb; ++k) {
+      const double r = shfl_d(v, k);
+      if (lane == k) kept = r;
+      v = fma(dm[lane][k], r, lane == k ? -0.0 : v);
+    }
+  } else {
+    for (int k = 0; k < nb; ++k) {
+      const double m = -shfl_d(v, k) * dm[k][k];
+      if (lane == k) kept = m;
+      v = lane == k ? m : fma(m, dr[k][lane], v);
+    }
+  }
+  if (!in) return;
+  *el = v;
+  (col ? w.pr : w.pm)[(int64_t)x * GJ_NB + lane] = kept;
+}
+
+// The panel's steps on everything else, 32 x 32 tiles: block 0 takes the next
+// panel's diagonal tile and then runs its steps; the other blocks stride over
+// the remaining tiles, the next tile's operands loaded while one is updated.
+__global__ void __launch_bounds__(GJ_THREADS) gj_rest(int n, int b, SepWork w) {
+  if (w.st->done) return;
+  __shared__ double M[2][GJ_NB][GJ_NB + 1], R[2][GJ_NB][GJ_NB + 1];
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int nt = (n + GJ_NB - 1) / GJ_NB, side = nt - 1;      // tile rows outside the panel
+  const int nb = min(GJ_NB, n - b * GJ_NB);
+  const int next = b + 1 < nt ? b * side + b : -1;             // the next diagonal tile's index
+  const int tiles = side * side;
+  // block 0: only the next diagonal tile (none after the last panel)
+  int t = blockIdx.x == 0 ? next : (int)blockIdx.x - 1;
+  const int stride = blockIdx.x == 0 ? tiles : (int)gridDim.x - 1;
+  if (blockIdx.x > 0 && t == next) t += stride;
+  if (t < 0 || t >= tiles) return;
+  double m0, m1, r0, r1, a0, a1;
+  auto load = [&](int t) {
+    int ti = t / side, tj = t - ti * side;
+    ti += ti >= b; tj += tj >= b;
+    const int i0 = ti * GJ_NB + g, j = tj * GJ_NB + lane, jr = tj * GJ_NB + g;
+    m0 = i0 < n ? w.pm[(int64_t)i0 * GJ_NB + lane] : 0.0;
+    m1 = i0 + 16 < n ? w.pm[(int64_t)(i0 + 16) * GJ_NB + lane] : 0.0;
+    r0 = jr < n ? w.pr[(int64_t)jr * GJ_NB + lane] : 0.0;
+    r1 = jr + 16 < n ? w.pr[(int64_t)(jr + 16) * GJ_NB + lane] : 0.0;
+    a0 = i0 < n && j < n ? w.A[(int64_t)i0 * n + j] : 0.0;
+    a1 = i0 + 16 < n && j < n ? w.A[(int64_t)(i0 + 16) * n + j] : 0.0;
+  };
+  load(t);
+  for (int f = 0; t < tiles; f ^= 1) {
+    M[f][g][lane] = m0; M[f][g + 16][lane] = m1;
+    R[f][g][lane] = r0; R[f][g + 16][lane] = r1;
+    double x0 = a0, x1 = a1;
+    const int cur = t;
+    t += stride;
+    if (t == next && blockIdx.x > 0) t += stride;
+    __syncthreads();
+    if (t < tiles) load(t);
+    if (nb == GJ_NB) {
+#pragma unroll 8
+      for (int k = 0; k < GJ_NB; ++k) {
+        const double r = R[f][lane][k];
+        x0 = fma(M[f][g][k], r, x0);
+        x1 = fma(M[f][g + 16][k], r, x1);
+      }
+    } else {
+      for (int k = 0; k < nb; ++k) {
+        const double r = R[f][lane][k];
+        x0 = fma(M[f][g][k], r, x0);
+        x1 = fma(M[f][g + 16][k], r, x1);
+      }
+    }
+    int ti = cur / side, tj = cur - ti * side;
+    ti += ti >= b; tj += tj >= b;
+    const int i0 = ti * GJ_NB + g, j = tj * GJ_NB + lane;
+    if (blockIdx.x == 0) {
+      gj_diag_block(n, (b + 1) * GJ_NB, x0, x1, w);
+      return;
+    }
+    if (i0 < n && j < n) w.A[(int64_t)i0 * n + j] = x0;
+    if (i0 + 16 < n && j < n) w.A[(int64_t)(i0 + 16) * n + j] = x1;
+  }
 }
 
 __device__ __forceinline__ double warp_sum_d(double v) {
@@ -245,7 +375,7 @@ __device__ void sep_propose(SepState* s, int p, double lo, double hi, int maxit,
 __global__ void sep_finish(int n, int p, double lo, double hi, int maxit, SepWork w) {
   SepState* s = w.st;
   if (s->done) return;
-  __shared__ double red[2];
+  __shared__ double red[2], sums[2 * SEP_MAX_P];
   const int lane = threadIdx.x;
   double ps = 0.0, ld = 0.0;
   for (int a = lane; a < n; a += 32) {
@@ -255,6 +385,18 @@ __global__ void sep_finish(int n, int p, double lo, double hi, int maxit, SepWor
   ps = warp_sum_d(ps);
   ld = warp_sum_d(ld);
   if (lane == 0) { red[0] = ps; red[1] = ld; }
+  // the rows' partial sums in row order, one lane per sum (2p of them)
+  if (lane < 2 * p) {
+    double t = 0.0;
+    if (lane < p) {
+#pragma unroll 8
+      for (int a = 0; a < n; ++a) t += w.part[(int64_t)a * 2 * p + lane];
+    } else {
+#pragma unroll 8
+      for (int a = 0; a < n; ++a) t += w.alpha[a] * w.part[(int64_t)a * 2 * p + lane];
+    }
+    sums[lane] = t;
+  }
   __syncwarp();
   if (lane != 0) return;
   const double psi = red[0], logdet = red[1], hn = 0.5 * n;
@@ -262,11 +404,7 @@ __global__ void sep_finish(int n, int p, double lo, double hi, int maxit, SepWor
   if (!(psi > 0.0)) l = NAN;
   double gt[SEP_MAX_P];
   for (int k = 0; k < p; ++k) {
-    double tr = 0.0, q = 0.0;
-    for (int a = 0; a < n; ++a) {
-      tr += w.part[(int64_t)a * 2 * p + k];
-      q += w.alpha[a] * w.part[(int64_t)a * 2 * p + p + k];
-    }
+    const double tr = sums[k], q = sums[p + k];
     const double th = exp(s->eta_t[k]);
     // dl/dtheta_k times theta_k (the gradient in eta)
     gt[k] = (-0.5 * tr + hn * q / psi) / th;
@@ -366,11 +504,23 @@ extern "C" int laGP_sep_mle(const double* design, const double* y, int64_t N, in
   if (cudaGetLastError() != cudaSuccess) return LAGP_ERR_CUDA;
   const dim3 blk(32, 8), grd((n + 31) / 32, (n + 7) / 8);
   const int rows_grid = (n + 7) / 8;
+  // Gauss-Jordan panels: block 0 of gj_rest is the next panel's, the others one per SM
+  const int nt = (n + GJ_NB - 1) / GJ_NB, rest_tiles = (nt - 1) * (nt - 1);
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return LAGP_ERR_CUDA;
+  const int rest_grid = 1 + (rest_tiles < sms - 1 ? rest_tiles : (sms > 1 ? sms - 1 : 1));
   // at most maxit iterations of at most 41 trials each, plus the first evaluation
   const int64_t max_evals = (int64_t)maxit * 41 + 1;
   for (int64_t e = 0; e < max_evals; ++e) {
     sep_build<<<grd, blk, 0, s>>>(n, p, g, w);
-    for (int k = 0; k < n; ++k) gj_step<<<grd, blk, 0, s>>>(n, k, w);
+    gj_first<<<1, GJ_THREADS, 0, s>>>(n, w);
+    for (int b = 0; b < nt && rest_tiles > 0; ++b) {
+      const int out = n - (n - b * GJ_NB < GJ_NB ? n - b * GJ_NB : GJ_NB);
+      gj_panels<<<(2 * out + 7) / 8, 256, 0, s>>>(n, b * GJ_NB, w);
+      gj_rest<<<rest_grid, GJ_THREADS, 0, s>>>(n, b, w);
+    }
     sep_alpha<<<rows_grid, 256, 0, s>>>(n, w);
     sep_rows<<<rows_grid, 256, 0, s>>>(n, p, w);
     sep_finish<<<1, 32, 0, s>>>(n, p, lo, hi, maxit, w);

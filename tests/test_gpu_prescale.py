@@ -80,3 +80,21 @@ def test_local_path_on_prescaled_inputs(lagp, w4, search):
     o = oracle_run(s, search, nrays=4)
     ident, _ = assert_fp64_parity(g, o, s.n0, s.M)
     assert ident >= s.M - 1
+
+
+@pytest.mark.parametrize("n_sub", [2, 31, 32, 33, 64, 65, 97, 1024])
+def test_panel_edges_of_the_inverse(lagp, w4, n_sub):
+    """One maximiser iteration from theta0 at subset sizes around the 32-pivot
+    panels of the Gauss-Jordan inverse: theta moves by the (scaled) gradient at
+    theta0, which the oracle forms from a Cholesky factor.  With g = 1e-2 the
+    condition number is at most n / g, so the inverse's relative error is below
+    n^2 / g * eps, about 1e-8 at the largest size; 1e-7 leaves room for the
+    gradient's own sums."""
+    sub = W.subset(w4.N, n_sub, seed=2)
+    g = 1e-2
+    th, (it, ev, st) = lagp.sep_mle(to_dev(w4.X), to_dev(w4.Y), to_dev(sub), g, 0.5, TMIN, TMAX,
+                                    maxit=1)
+    assert st == 0 and it == 1
+    S, y = w4.X[sub], w4.Y[sub]
+    to, _, _, _ = SM.sep_mle(S, y, g, 0.5, TMIN, TMAX, maxit=1)
+    np.testing.assert_allclose(th.cpu().numpy(), to, rtol=1e-7)
