@@ -24,6 +24,13 @@
 // The factor itself grows in FP64 (the partitioned update in factored form,
 // Sec 2.2) in global memory, packed lower-triangular.
 //
+// Code size.  The kernel's warps are at different places of a long loop body,
+// so instruction fetches are a cost of their own: with one call site of the
+// point append and of Brent's step, loops left rolled unless their trip hides
+// a latency, and the k-d walk in an instantiation of its own (FULL), the
+// kernel's stalls for instructions fell from 1.3 to 0.6 per issue and its time
+// at the sizes above from 157 to 121.7 ms (143 ms before the register-held kz).
+//
 // Scheduling.  The kernel is persistent: each warp takes the next location
 // from a device work counter until the queue is empty, optionally through a
 // permutation (largest local designs first, so that uneven n does not leave a
@@ -151,10 +158,97 @@ __device__ __forceinline__ double warp_sum64(double v) {
   return v;
 }
 
+// One lane's share of an ALC evaluation: rows i = q, q + G, ... of
+// w = L^{-1} kz, with |w|^2 and w . z summed over them in ascending order.
+// A row is two FMA chains over k (elements 0, 2 and 1, 3 of each quad, one
+// paired FMA per element pair).  Shared loads return 128 bytes per cycle to
+// the registers however many lanes read the same word, and that return path
+// is the kernel's busiest unit, so a lane runs two rows side by side on one
+// load of the ray's kz, whose first KZ_QUADS quads stay in registers for all
+// rows; the row blocks that need no others are unrolled.  That leaves about
+// one 128-bit load per quad of a row (two, with kz loaded per row), and two
+// independent chains to cover each other's latency.  Eight quads is what fits
+// in 96 registers, which 20 resident warps leave each thread: sixteen quads and
+// 16 warps were slower (156.8 against 141.5 ms per 100,000 locations at 8-d,
+// n = 50, N' = 1000), and so were all rows of a lane side by side, column quad
+// by column quad (156.2 ms).
+#define KZ_QUADS 8
+__device__ __forceinline__ void fma_quad(const float4& l4, const float4& k4, float2& acc) {
+  acc = __ffma2_rn(make_float2(l4.x, l4.y), make_float2(k4.x, k4.y), acc);
+  acc = __ffma2_rn(make_float2(l4.z, l4.w), make_float2(k4.z, k4.w), acc);
+}
+template <int G>
+__device__ __forceinline__ void ray_product(const float* __restrict__ Lf,
+                                            const float* __restrict__ kzr,
+                                            const float* __restrict__ zf, int q, int j, int n_max,
+                                            float* vs_out, float* ns_out) {
+  float4 kz[KZ_QUADS];
+  float vs = 0.f, ns = 0.f;
+  constexpr int T = 4 * KZ_QUADS / G;        // unrolled blocks of G rows, in pairs
+  const int sub = q >> 2;                    // G > 4: the lane's four-row block within one of G
+  auto take = [&](int i, bool in, const float2& acc) {
+    if (!in) return;
+    const float w = acc.x + acc.y;
+    vs = fmaf(w, w, vs);
+    ns = fmaf(w, zf[i], ns);
+  };
+#pragma unroll
+  for (int t = 0; t < T; t += 2) {
+    if (G * t >= j) break;
+    const int k_lo = t == 0 ? 0 : ((G * t - 1) >> 2) + 1;      // first quad not yet held
+    const int k_hi0 = (G * t + G - 1) >> 2, k_hi1 = (G * t + 2 * G - 1) >> 2;
+#pragma unroll
+    for (int k = k_lo; k <= k_hi1; ++k) kz[k] = *reinterpret_cast<const float4*>(kzr + 4 * k);
+    // a row past j reads row 0's place and is not taken
+    const int i0 = G * t + q, i1 = i0 + G;
+    const bool in0 = i0 < j, in1 = i1 < j;
+    const float* L0 = Lf + (in0 ? lf_block(i0 >> 2) + 4 * (i0 & 3) : 0);
+    const float* L1 = Lf + (in1 ? lf_block(i1 >> 2) + 4 * (i1 & 3) : 0);
+    float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+#pragma unroll
+    for (int k = 0; k <= k_hi1; ++k) {
+      // a block of more than four rows ends in quads that only its later rows have
+      if (k <= k_hi0 && (G <= 4 || k <= ((G * t) >> 2) + sub))
+        fma_quad(*reinterpret_cast<const float4*>(L0 + 16 * k), kz[k], a0);
+      if (G <= 4 || k <= ((G * t + G) >> 2) + sub)
+        fma_quad(*reinterpret_cast<const float4*>(L1 + 16 * k), kz[k], a1);
+    }
+    take(i0, in0, a0);
+    take(i1, in1, a1);
+  }
+  for (int i0 = 4 * KZ_QUADS + q; i0 < j; i0 += 2 * G) {
+    const bool in1 = i0 + G < j;
+    const int i1 = in1 ? i0 + G : i0;
+    const int u0 = i0 >> 2, u1 = i1 >> 2;
+    const int ld0 = lf_stride(u0, n_max), ld1 = lf_stride(u1, n_max);
+    const float* L0 = Lf + lf_block(u0) + 4 * (i0 & 3);
+    const float* L1 = Lf + lf_block(u1) + 4 * (i1 & 3);
+    float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+#pragma unroll
+    for (int k = 0; k < KZ_QUADS; ++k, L0 += ld0, L1 += ld1) {
+      fma_quad(*reinterpret_cast<const float4*>(L0), kz[k], a0);
+      fma_quad(*reinterpret_cast<const float4*>(L1), kz[k], a1);
+    }
+    int k = KZ_QUADS;
+#pragma unroll 2
+    for (; k <= u0; ++k, L0 += ld0, L1 += ld1) {
+      const float4 k4 = *reinterpret_cast<const float4*>(kzr + 4 * k);
+      fma_quad(*reinterpret_cast<const float4*>(L0), k4, a0);
+      fma_quad(*reinterpret_cast<const float4*>(L1), k4, a1);
+    }
+    for (; k <= u1; ++k, L1 += ld1)
+      fma_quad(*reinterpret_cast<const float4*>(L1), *reinterpret_cast<const float4*>(kzr + 4 * k), a1);
+    take(i0, true, a0);
+    take(i1, in1, a1);
+  }
+  *vs_out = vs;
+  *ns_out = ns;
+}
+
 enum { PH_ALC0 = 0, PH_FIRST = 1, PH_ITER = 2, PH_DONE = 3 };
 
 // One location, by one warp, in the warp's shared-memory region and FP64 slot.
-template <int RP, int PP>
+template <int RP, int PP, bool FULL>
 __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t loc, float* base,
                                                double* Lg) {
   constexpr int G = 32 / RP;
@@ -193,8 +287,11 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
   const double nit64 = -1.0 / theta;
   const float onepg = (float)(1.0 + P.g);
 
-  for (int i = lane; i < roff(ldn); i += 32) Lf[i] = 0.f;
+#pragma unroll 1
+  for (int i = lane; i < lf_words(ldn); i += 32) Lf[i] = 0.f;
+#pragma unroll 1
   for (int i = lane; i < RP * KP; i += 32) kzb[i] = 0.f;
+#pragma unroll 1
   for (int i = lane; i < (P.nc_max + 31) / 32; i += 32) { mask[i] = 0u; smask[i] = 0u; }
   if (lane < PP) {
     const bool in = lane < p;
@@ -202,8 +299,14 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
     lof[lane] = in ? (float)(P.lo[lane] - P.center[lane]) : 0.f;
     hif[lane] = in ? (float)(P.hi[lane] - P.center[lane]) : 0.f;
   }
-  if (P.tie_gap) for (int i = lane; i < ldn; i += 32) P.tie_gap[loc * ldn + i] = 0.0;
-  if (P.nevals) for (int i = lane; i < ldn; i += 32) P.nevals[loc * ldn + i] = 0;
+  if (P.tie_gap) {
+#pragma unroll 1
+    for (int i = lane; i < ldn; i += 32) P.tie_gap[loc * ldn + i] = 0.0;
+  }
+  if (P.nevals) {
+#pragma unroll 1
+    for (int i = lane; i < ldn; i += 32) P.nevals[loc * ldn + i] = 0;
+  }
   __syncwarp();
 
   int j = 0;
@@ -218,9 +321,11 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
   auto add_point = [&](int gi, int rr) -> bool {
     const double* c64 = P.X + (int64_t)gi * p;
     double kxj = 0.0;   // K(x_new, x), on lane j mod 32
+#pragma unroll 1
     for (int i = lane; i <= j; i += 32) {
-      if (i < j) kvs[i] = corr64_fast(P.X + (int64_t)gsel[i] * p, c64, p, nit64);
-      else kxj = corr64_fast(c64, xq, p, nit64);
+      const double c = corr64_fast(i < j ? P.X + (int64_t)gsel[i] * p : xq, c64, p, nit64);
+      if (i < j) kvs[i] = c;
+      else kxj = c;
     }
     kxj = __shfl_sync(0xffffffffu, kxj, j & 31);
     __syncwarp();
@@ -230,6 +335,7 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
     // instruction costs the same whatever its active lanes, so every lane
     // evaluates the scalar tail.
     double vv = 0.0, lz = 0.0, lzy = 0.0;
+#pragma unroll 1
     for (int i = lane; i < j; i += 32) {
       const double acc = dot64_ilp(Lg + tri(i), kvs, i + 1);
       ls[i] = acc;
@@ -246,7 +352,9 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
     if (!(v > 0.0)) return false;
     const double inv_d = rsqrt(v);
     double* Lj = Lg + tri(j);
-    float* Lfj = Lf + roff(j);
+    float* Lfj = Lf + lf_at(j, 0, ldn);
+    const int lds = lf_stride(j >> 2, ldn);
+#pragma unroll 1
     for (int k = lane; k < j; k += 32) {
       double a0 = 0.0, a1 = 0.0;
       int i = k;
@@ -257,11 +365,11 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
       if (i < j) a0 = fma(ls[i], Lg[tri(i) + k], a0);
       const double rk = -(a0 + a1) * inv_d;
       Lj[k] = rk;
-      Lfj[k] = (float)rk;
+      Lfj[lds * (k >> 2) + (k & 3)] = (float)rk;
     }
     if (lane == 0) {
       Lj[j] = inv_d;
-      Lfj[j] = (float)inv_d;
+      Lfj[lds * (j >> 2) + (j & 3)] = (float)inv_d;
       gsel[j] = gi;
       if (rr >= 0) mask[rr >> 5] |= 1u << (rr & 31);
       const double zj = (kxj - lz) * inv_d;
@@ -274,18 +382,22 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
     return true;
   };
 
-  for (int rr = 0; rr < P.n0 && ok; ++rr) ok = add_point(cl[rr], rr);
-
   const int r = lane / G, q = lane % G;
-  for (int step = P.n0; step < n && ok; ++step) {
+#pragma unroll 1
+  for (int step = 0; step < n && ok; ++step) {
+    int pick = step, pick_g = -1;     // rank among the candidates (or -1) and design index
+    if (step < P.n0) {
+      pick_g = cl[step];
+    } else {
     // ---- ray starts: unselected candidates of rank k0, k0+1, ... (mod |U|) ----
     // lane l owns mask words l, l + 32, ...; a warp scan of their unselected
     // counts locates the word holding each target rank
     {
       const int nU = nc - j;
-      const int k0 = ray_offset(j, P.n0);
+      const int k0 = ray_offset(j, P.n0) % nU;
       const int nw = (nc + 31) >> 5;
       int seen = 0;
+#pragma unroll 1
       for (int w0 = 0; w0 < nw; w0 += 32) {
         const int wd = w0 + lane;
         uint32_t un = 0u;
@@ -301,10 +413,13 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
           if (lane >= o) incl += y;
         }
         const int first = seen + incl - c;
+#pragma unroll 1
         for (int t = 0; t < R; ++t) {
-          const int target = (k0 + t) % nU;
+          int target = k0 + t;
+          if (target >= nU) target %= nU;      // (round the end: rare)
           if (target >= first && target < first + c) {
             uint32_t u = un;
+#pragma unroll 1
             for (int q2 = target - first; q2 > 0; --q2) u &= u - 1u;   // drop lower bits
             const int rr = wd * 32 + __ffs(u) - 1;
             starts[t] = rr;
@@ -321,6 +436,7 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
     if (ray_live) {
       const float* a = P.Xf + (int64_t)cl[starts[r]] * PP;
       float tau = 1.f;
+#pragma unroll 1
       for (int k = 0; k < p; ++k) {
         const float dk = 10.f * (a[k] - xf[k]);
         if (dk > 0.f) tau = fminf(tau, (hif[k] - a[k]) / dk);
@@ -348,6 +464,7 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
       bx = 2.f * nit2 * bxs;
       float* cr = Cb + r * KP;
       float* br = Bb + r * KP;
+#pragma unroll 1
       for (int k4 = q; 4 * k4 < j; k4 += G) {
         float cq[4], bq[4];
 #pragma unroll
@@ -385,6 +502,7 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
     Brent st;
     st.a = 0.f; st.b = 1.f; st.x = st.w = st.v = 0.f; st.fx = st.fw = st.fv = 0.f;
     st.d = 0.f; st.e = 0.f;
+#pragma unroll 1
     for (int round = 0; round < RAY_MAX_ROUNDS; ++round) {
       const bool active = phase != PH_DONE;
       if (!__any_sync(0xffffffffu, active)) break;
@@ -394,6 +512,7 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
         const float* cr = Cb + r * KP;
         const float* br = Bb + r * KP;
         const float2 s2v = make_float2(s_eval, s_eval), g2 = make_float2(gam, gam);
+#pragma unroll 1
         for (int k4 = q; 4 * k4 < j; k4 += G) {
           const float4 c4 = *reinterpret_cast<const float4*>(cr + 4 * k4);
           const float4 b4 = *reinterpret_cast<const float4*>(br + 4 * k4);
@@ -407,25 +526,7 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
       }
       __syncwarp();
       float vs = 0.f, ns = 0.f;
-      if (active) {
-        for (int i = q; i < j; i += G) {
-          const float* Li = Lf + roff(i);
-          const int len = (i + 4) & ~3;
-          // two accumulators (elements 0, 2 and 1, 3 of each quad) in one
-          // paired FMA per element pair
-          float2 acc = make_float2(0.f, 0.f);
-#pragma unroll 2
-          for (int k = 0; k < len; k += 4) {
-            const float4 l4 = *reinterpret_cast<const float4*>(Li + k);
-            const float4 k4 = *reinterpret_cast<const float4*>(kzr + k);
-            acc = __ffma2_rn(make_float2(l4.x, l4.y), make_float2(k4.x, k4.y), acc);
-            acc = __ffma2_rn(make_float2(l4.z, l4.w), make_float2(k4.z, k4.w), acc);
-          }
-          const float w = acc.x + acc.y;
-          vs = fmaf(w, w, vs);
-          ns = fmaf(w, zf[i], ns);
-        }
-      }
+      if (active) ray_product<G>(Lf, kzr, zf, q, j, ldn, &vs, &ns);
 #pragma unroll
       for (int o = G / 2; o > 0; o >>= 1) {
         vs += __shfl_xor_sync(0xffffffffu, vs, o);
@@ -440,32 +541,35 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
       __syncwarp();
       if (active) {
         ++evals;
-        bool more = false;
-        float u = 0.f;
+        bool more;
+        float u = 0.381966011250105151795f;   // the first golden-section point
         if (phase == PH_ALC0) {
           alc0 = val;
-          if (len2 > 0.f) { phase = PH_FIRST; s_eval = 0.381966011250105151795f; more = true; }
-        } else if (phase == PH_FIRST) {
-          st.x = st.w = st.v = s_eval;
-          st.fx = st.fw = st.fv = -val;
-          more = brent_next(st, &u);
-          if (more) { s_eval = u; phase = PH_ITER; }
+          more = len2 > 0.f;
         } else {
-          brent_take(st, s_eval, -val);
+          if (phase == PH_FIRST) {
+            st.x = st.w = st.v = s_eval;
+            st.fx = st.fw = st.fv = -val;
+          } else {
+            brent_take(st, s_eval, -val);
+          }
           more = brent_next(st, &u);
-          if (more) s_eval = u;
         }
         if (more && evals > 1000) more = false;
         if (!more) {
           if (phase == PH_ALC0 || alc0 >= -st.fx) { s_star = 0.f; alc_star = alc0; }
           else { s_star = st.x; alc_star = -st.fx; }
           phase = PH_DONE;
+        } else {
+          s_eval = u;
+          phase = phase == PH_ALC0 ? PH_FIRST : PH_ITER;
         }
       }
     }
     // ---- best ray, its continuous point x* ----
     float best = -1.f, second = -1.f;
     int ib = 0, ev = 0;
+#pragma unroll 1
     for (int rr = 0; rr < R; ++rr) {
       const float a_r = __shfl_sync(0xffffffffu, alc_star, rr * G);
       ev += __shfl_sync(0xffffffffu, evals, rr * G);
@@ -488,16 +592,18 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
     for (int k = 0; k < PP; k += 2) nx[k / 2] = make_float2(-xs[k], -xs[k + 1]);
     float bd0 = __int_as_float(0x7f800000), bd1 = bd0;
     int bi0 = 0x7fffffff, bi1 = 0x7fffffff;
-    int pick_g = -1;                  // the full scope's pick (design index)
-    if (P.full) {
+    if (FULL) {
       // nearest point of X_N outside the design; the step's starts are
       // forbidden unless they equal x*
       const KdView<float>& V = P.kd;
       auto excluded = [&](int32_t gi, int64_t pos, bool allow_starts) -> bool {
+#pragma unroll 1
         for (int i = 0; i < j; ++i) if (gsel[i] == gi) return true;
         if (allow_starts) return false;
+#pragma unroll 1
         for (int t = 0; t < R; ++t) {
           if (cl[starts[t]] != gi) continue;
+#pragma unroll 1
           for (int k = 0; k < p; ++k) if (V.pts[pos * PP + k] != xs[k]) return true;
         }
         return false;
@@ -518,6 +624,7 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
       auto distx = [&](int64_t pos, int32_t) -> float {
         const float* c = V.pts + pos * PP;
         float d = 0.f;
+#pragma unroll 1
         for (int k = 0; k < PP; ++k) { const float t = c[k] - xf[k]; d = fmaf(t, t, d); }
         return d;
       };
@@ -530,18 +637,16 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
       const int lim = (sb == 0.f) ? starts[ib] + 1 : nc;
       const int nw = (lim + 31) >> 5;
       const uint32_t bit = 1u << lane;
-#pragma unroll 1
-      for (int wd = 0; wd < nw; ++wd) {
+      auto consider = [&](int wd, const float4 (&cv)[PP / 4]) {
         const int rr = wd * 32 + lane;
         if (rr < lim && !(mask[wd] & bit)) {
-          const float* c = P.Xf + (int64_t)cl[rr] * PP;
           float2 d2 = make_float2(0.f, 0.f);
           bool same = true;                   // every coordinate equal to x*'s
 #pragma unroll
           for (int k = 0; k < PP; k += 4) {
-            const float4 cv = *reinterpret_cast<const float4*>(c + k);
-            const float2 t01 = __fadd2_rn(make_float2(cv.x, cv.y), nx[k / 2]);
-            const float2 t23 = __fadd2_rn(make_float2(cv.z, cv.w), nx[k / 2 + 1]);
+            const float4 v = cv[k / 4];
+            const float2 t01 = __fadd2_rn(make_float2(v.x, v.y), nx[k / 2]);
+            const float2 t23 = __fadd2_rn(make_float2(v.z, v.w), nx[k / 2 + 1]);
             same &= (t01.x == 0.f) & (t01.y == 0.f) & (t23.x == 0.f) & (t23.y == 0.f);
             d2 = __ffma2_rn(t01, t01, d2);
             d2 = __ffma2_rn(t23, t23, d2);
@@ -550,6 +655,23 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
           if (d < bd1) { bd1 = d; bi1 = rr; }
           if ((same || !(smask[wd] & bit)) && d < bd0) { bd0 = d; bi0 = rr; }
         }
+      };
+      // two candidates per lane at a time, and the next two's indices loaded
+      // while their rows arrive from L2
+      int g0 = cl[min(lane, lim - 1)], g1 = cl[min(32 + lane, lim - 1)];
+#pragma unroll 1
+      for (int wd = 0; wd < nw; wd += 2) {
+        const float4* c0 = reinterpret_cast<const float4*>(P.Xf + (int64_t)g0 * PP);
+        const float4* c1 = reinterpret_cast<const float4*>(P.Xf + (int64_t)g1 * PP);
+        float4 v0[PP / 4], v1[PP / 4];
+#pragma unroll
+        for (int k = 0; k < PP / 4; ++k) v0[k] = c0[k];
+#pragma unroll
+        for (int k = 0; k < PP / 4; ++k) v1[k] = c1[k];
+        g0 = cl[min((wd + 2) * 32 + lane, lim - 1)];
+        g1 = cl[min((wd + 3) * 32 + lane, lim - 1)];
+        consider(wd, v0);
+        consider(wd + 1, v1);
       }
     }
 #pragma unroll
@@ -561,13 +683,14 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
       if (od0 < bd0 || (od0 == bd0 && oi0 < bi0)) { bd0 = od0; bi0 = oi0; }
       if (od1 < bd1 || (od1 == bd1 && oi1 < bi1)) { bd1 = od1; bi1 = oi1; }
     }
-    int pick = -1;
-    if (!P.full) {
+    pick = -1;
+    if (!FULL) {
       pick = bi0 != 0x7fffffff ? bi0 : (bi1 != 0x7fffffff ? bi1 : -1);
       pick_g = pick >= 0 ? cl[pick] : -1;
     } else if (pick_g >= 0) {
       // its candidate rank, when it is one
       int rk = 0x7fffffff;
+#pragma unroll 1
       for (int rr = lane; rr < nc; rr += 32) if (cl[rr] == pick_g) rk = min(rk, rr);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) rk = min(rk, __shfl_xor_sync(0xffffffffu, rk, o));
@@ -580,11 +703,13 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
           (best > 0.f && R > 1) ? (double)((best - second) / best) : 0.0;
       if (P.nevals) P.nevals[loc * ldn + (step - P.n0)] = ev;
     }
+    }
     ok = (pick_g >= 0) && add_point(pick_g, pick);
   }
 
   if (ok) {
     double a = 0.0, b = 0.0, c = 0.0;
+#pragma unroll 1
     for (int i = lane; i < j; i += 32) {
       a = fma(z64[i], zy64[i], a);
       b = fma(zy64[i], zy64[i], b);
@@ -603,25 +728,27 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
     atomicOr(P.status, LAGP_DEV_BAD_UPDATE);
   }
   if (P.selected)
+#pragma unroll 1
     for (int i = lane; i < ldn; i += 32) P.selected[loc * ldn + i] = (i < j) ? gsel[i] : -1;
   if (lane == 0) promote_location(P.promote, P.promote_count, loc, *vmin);
 }
 
-// at least 20 resident warps per SM (at most 102 registers per thread)
-template <int RP, int PP, int RW>
-__global__ void __launch_bounds__(RW * 32, 20 / RW) ray32_kernel(RayParams P) {
+// 20 resident warps per SM (at most 96 registers per thread, 32 of them the
+// ray's kz quads); the block holds 1, 2 or 4 warps
+template <int RP, int PP, bool FULL>
+__global__ void __launch_bounds__(128, 5) ray32_kernel(RayParams P) {
   extern __shared__ __align__(16) float sm[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WarpLayout lay = warp_layout(P.n_max, PP, RP, P.nc_max);
   float* base = sm + (size_t)warp * (lay.bytes / 4);
-  double* Lg = P.g64 + ((int64_t)blockIdx.x * RW + warp) * P.g64_stride;
+  double* Lg = P.g64 + ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * P.g64_stride;
   const unsigned items = P.count ? *P.count : (unsigned)P.M;
   for (;;) {
     unsigned it = 0;
     if (lane == 0) it = atomicAdd(P.queue, 1u);
     it = __shfl_sync(0xffffffffu, it, 0);
     if (it >= items) break;
-    ray32_location<RP, PP>(P, P.order ? (int64_t)P.order[it] : (int64_t)it, base, Lg);
+    ray32_location<RP, PP, FULL>(P, P.order ? (int64_t)P.order[it] : (int64_t)it, base, Lg);
     __syncwarp();
   }
 }
@@ -654,9 +781,9 @@ int ray32_slots(int64_t chunk) {
   return (int)((s + 3) / 4 * 4);
 }
 
-template <int RP, int PP, int RW>
-static cudaError_t ray32_go(const RayParams& P, size_t sm, int slots, cudaStream_t s) {
-  auto k = ray32_kernel<RP, PP, RW>;
+template <int RP, int PP>
+static cudaError_t ray32_go(const RayParams& P, int RW, size_t sm, int slots, cudaStream_t s) {
+  auto k = P.full ? ray32_kernel<RP, PP, true> : ray32_kernel<RP, PP, false>;
   cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (err != cudaSuccess) return err;
   const int64_t grid = persistent_grid(k, RW * 32, sm, P.M, slots, RW);
@@ -693,17 +820,13 @@ cudaError_t launch_ray32(const DesignArgs& a, cudaStream_t s) {
   const int RW = a.tune.ray_warps;
   const size_t sm = (size_t)lay.bytes * RW;
   const int slots = ray32_slots(a.ws->chunk);
-  const int key = (RW * 100 + RP) * 100 + a.PP;
-  switch (key) {
-#define RAY_CASE(RWV, RPV, PPV) \
-  case (RWV * 100 + RPV) * 100 + PPV: return ray32_go<RPV, PPV, RWV>(P, sm, slots, s);
-#define RAY_CASES(RWV)                                                                   \
-    RAY_CASE(RWV, 2, 4) RAY_CASE(RWV, 2, 8) RAY_CASE(RWV, 2, 12) RAY_CASE(RWV, 2, 16)     \
-    RAY_CASE(RWV, 4, 4) RAY_CASE(RWV, 4, 8) RAY_CASE(RWV, 4, 12) RAY_CASE(RWV, 4, 16)     \
-    RAY_CASE(RWV, 8, 4) RAY_CASE(RWV, 8, 8) RAY_CASE(RWV, 8, 12) RAY_CASE(RWV, 8, 16)     \
-    RAY_CASE(RWV, 16, 4) RAY_CASE(RWV, 16, 8) RAY_CASE(RWV, 16, 12) RAY_CASE(RWV, 16, 16)
-    RAY_CASES(1) RAY_CASES(2) RAY_CASES(4)
-#undef RAY_CASES
+  switch (RP * 100 + a.PP) {
+#define RAY_CASE(RPV, PPV) \
+  case RPV * 100 + PPV: return ray32_go<RPV, PPV>(P, RW, sm, slots, s);
+    RAY_CASE(2, 4) RAY_CASE(2, 8) RAY_CASE(2, 12) RAY_CASE(2, 16)
+    RAY_CASE(4, 4) RAY_CASE(4, 8) RAY_CASE(4, 12) RAY_CASE(4, 16)
+    RAY_CASE(8, 4) RAY_CASE(8, 8) RAY_CASE(8, 12) RAY_CASE(8, 16)
+    RAY_CASE(16, 4) RAY_CASE(16, 8) RAY_CASE(16, 12) RAY_CASE(16, 16)
 #undef RAY_CASE
     default:
       return cudaErrorInvalidValue;

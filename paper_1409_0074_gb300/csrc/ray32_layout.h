@@ -25,6 +25,22 @@ LAGP_HD int roff(int i) {
   return 4 * (i + 2 * a * (a - 1) + a * b);
 }
 LAGP_HD int tri(int i) { return i * (i + 1) / 2; }
+// The inverse factor's FP32 rows as the scoring product reads them: four rows
+// 4u .. 4u+3 form a block of u + 1 quads per row, with the rows' k-th quads
+// side by side, so that the four lanes of a ray read 64 contiguous bytes.  A
+// ragged last block past row 32 holds only the rows it has (a design of 50
+// points then takes what plain rows would).  lf_stride(u, n) is the words from
+// one quad of a row to its next, lf_at(i, k, n) the word of element (i, k) and
+// lf_words(n) the words of n rows.
+LAGP_HD int lf_block(int u) { return 8 * u * (u + 1); }
+LAGP_HD int lf_stride(int u, int n) { return (u >= 8 && 4 * u + 4 > n) ? 4 * (n - 4 * u) : 16; }
+LAGP_HD int lf_at(int i, int k, int n) {
+  return lf_block(i >> 2) + lf_stride(i >> 2, n) * (k >> 2) + 4 * (i & 3) + (k & 3);
+}
+LAGP_HD int lf_words(int n) {
+  const int u = (n - 1) >> 2;
+  return lf_block(u) + lf_stride(u, n) * (u + 1);
+}
 // row length of the kz buffer: a multiple of 4 whose quarter is odd, so that
 // the rays' float4 reads fall on different banks
 LAGP_HD int kz_ld(int n) {
@@ -41,7 +57,7 @@ LAGP_HDI WarpLayout warp_layout(int n, int PP, int RP, int nc) {
   WarpLayout w;
   int off = 0;   // in 4-byte words, float region first (16-byte aligned pieces)
   auto take = [&](int words) { int o = off; off += (words + 3) & ~3; return o; };
-  w.lf = take(roff(n));
+  w.lf = take(lf_words(n));
   w.kz = take(RP * kz_ld(n));
   // per-ray exponent coefficients c_k then b_k (rows of kz_ld(n)); the k-d
   // tree walk of the full-scope snap (nodes, then their box distances) and
