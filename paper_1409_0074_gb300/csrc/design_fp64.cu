@@ -518,7 +518,7 @@ __device__ int search_ray(const D64Params& P, Loc& L, const int32_t* cl, int nc,
       };
       auto dist = [&](int64_t, int32_t gi) { return sqdist64(P.X + (int64_t)gi * p, L.xs, p); };
       auto distx = [&](int64_t, int32_t gi) { return sqdist64(P.X + (int64_t)gi * p, L.xq, p); };
-      const KdTop<double> b = kd_nearest<double>(V, L.xs, 1e-12, L.stk, L.bnd, excluded, dist, distx);
+      const KdTop<double> b = kd_nearest<true>(V, L.xs, 1e-12, L.stk, L.bnd, excluded, dist, distx);
       if (lane == 0) {
         L.iscal[1] = b.i1;
         L.iscal[2] = 0x7fffffff;

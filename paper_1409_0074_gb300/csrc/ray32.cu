@@ -628,7 +628,7 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
         for (int k = 0; k < PP; ++k) { const float t = c[k] - xf[k]; d = fmaf(t, t, d); }
         return d;
       };
-      const KdTop<float> b = kd_nearest<float>(V, xs, 1e-5f, stk, bnd, excluded, dist, distx);
+      const KdTop<float> b = kd_nearest<false>(V, xs, 1e-5f, stk, bnd, excluded, dist, distx);
       pick_g = b.i1;
     } else {
       // When the best ray kept s = 0, x* is its start, an allowed candidate at
