@@ -245,6 +245,24 @@ __device__ __forceinline__ void ray_product(const float* __restrict__ Lf,
   *ns_out = ns;
 }
 
+// Three sums over the warp (each the value of warp_sum64, to the bit: the same
+// tree of pairs) in 7 binary64 additions instead of 15: from the step where
+// half the lanes hold one sum's partials, other lanes hold another's.
+__device__ __forceinline__ void warp_sum64_3(double& a, double& b, double& c) {
+  const int lane = threadIdx.x & 31;
+  const double keep = lane < 16 ? a : b, send = lane < 16 ? b : a;
+  double s = keep + __shfl_xor_sync(0xffffffffu, send, 16);   // a below lane 16, b above
+  c += __shfl_xor_sync(0xffffffffu, c, 16);
+  s += __shfl_xor_sync(0xffffffffu, s, 8);
+  c += __shfl_xor_sync(0xffffffffu, c, 8);
+  if (lane & 8) s = c;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  a = __shfl_sync(0xffffffffu, s, 0);
+  b = __shfl_sync(0xffffffffu, s, 16);
+  c = __shfl_sync(0xffffffffu, s, 8);
+}
+
 enum { PH_ALC0 = 0, PH_FIRST = 1, PH_ITER = 2, PH_DONE = 3 };
 
 // One location, by one warp, in the warp's shared-memory region and FP64 slot.
@@ -343,9 +361,7 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
       lz = fma(acc, z64[i], lz);
       lzy = fma(acc, zy64[i], lzy);
     }
-    vv = warp_sum64(vv);
-    lz = warp_sum64(lz);
-    lzy = warp_sum64(lzy);
+    warp_sum64_3(vv, lz, lzy);
     __syncwarp();
     const double v = (1.0 + P.g) - vv;
     if (lane == 0) *vmin = v > 0.0 ? fmin(*vmin, v) : -1.0;
@@ -355,14 +371,30 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
     float* Lfj = Lf + lf_at(j, 0, ldn);
     const int lds = lf_stride(j >> 2, ldn);
 #pragma unroll 1
-    for (int k = lane; k < j; k += 32) {
+    for (int k = lane; k < ((j + 31) & ~31); k += 32) {
+      // sum_i l_i L_ik over i >= k: the even and the odd offsets i - k apart, as
+      // the even and the odd i (adding the two is commutative).  All lanes take
+      // the same row i, so its elements are contiguous over them.  (The other
+      // product, by rows, stays as it is: a second copy of the factor by
+      // columns made it contiguous too, but doubled the scratch the slots cycle
+      // through L2 and was slower, 124.0 against 117.2 ms per 100,000
+      // locations.)
+      const int i0 = k & ~31;
+      const double* Lk = Lg + k;
+      auto at = [&](int i) { return i >= k && i < j ? Lk[tri(i)] : 0.0; };
       double a0 = 0.0, a1 = 0.0;
-      int i = k;
-      for (; i + 1 < j; i += 2) {
-        a0 = fma(ls[i], Lg[tri(i) + k], a0);
-        a1 = fma(ls[i + 1], Lg[tri(i + 1) + k], a1);
+      double n0 = at(i0), n1 = at(i0 + 1), n2 = at(i0 + 2), n3 = at(i0 + 3);
+#pragma unroll 1
+      for (int i = i0; i < j; i += 4) {
+        // the next rows' loads are in flight during this step's FP64
+        const double m0 = n0, m1 = n1, m2 = n2, m3 = n3;
+        n0 = at(i + 4); n1 = at(i + 5); n2 = at(i + 6); n3 = at(i + 7);
+        a0 = fma(ls[i], m0, a0);
+        if (i + 1 < j) a1 = fma(ls[i + 1], m1, a1);
+        if (i + 2 < j) a0 = fma(ls[i + 2], m2, a0);
+        if (i + 3 < j) a1 = fma(ls[i + 3], m3, a1);
       }
-      if (i < j) a0 = fma(ls[i], Lg[tri(i) + k], a0);
+      if (k >= j) break;
       const double rk = -(a0 + a1) * inv_d;
       Lj[k] = rk;
       Lfj[lds * (k >> 2) + (k & 3)] = (float)rk;
@@ -469,25 +501,22 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
         float cq[4], bq[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
+          // a quad's rows are loaded without a branch, all in flight together
           const int k = 4 * k4 + u;
-          cq[u] = -__int_as_float(0x7f800000);
-          bq[u] = 0.f;
-          if (k < j) {
-            const float* sk = P.Xf + (int64_t)gsel[k] * PP;
-            float cs = 0.f, bs = 0.f;
+          const float* sk = P.Xf + (int64_t)gsel[min(k, j - 1)] * PP;
+          float cs = 0.f, bs = 0.f;
 #pragma unroll
-            for (int c = 0; c < PP; c += 4) {
-              const float4 s4 = *reinterpret_cast<const float4*>(sk + c);
-              const float t0 = av[c] - s4.x, t1 = av[c + 1] - s4.y;
-              const float t2 = av[c + 2] - s4.z, t3 = av[c + 3] - s4.w;
-              cs = fmaf(t0, t0, cs); cs = fmaf(t1, t1, cs);
-              cs = fmaf(t2, t2, cs); cs = fmaf(t3, t3, cs);
-              bs = fmaf(dv[c], t0, bs); bs = fmaf(dv[c + 1], t1, bs);
-              bs = fmaf(dv[c + 2], t2, bs); bs = fmaf(dv[c + 3], t3, bs);
-            }
-            cq[u] = nit2 * cs;
-            bq[u] = 2.f * nit2 * bs;
+          for (int c = 0; c < PP; c += 4) {
+            const float4 s4 = *reinterpret_cast<const float4*>(sk + c);
+            const float t0 = av[c] - s4.x, t1 = av[c + 1] - s4.y;
+            const float t2 = av[c + 2] - s4.z, t3 = av[c + 3] - s4.w;
+            cs = fmaf(t0, t0, cs); cs = fmaf(t1, t1, cs);
+            cs = fmaf(t2, t2, cs); cs = fmaf(t3, t3, cs);
+            bs = fmaf(dv[c], t0, bs); bs = fmaf(dv[c + 1], t1, bs);
+            bs = fmaf(dv[c + 2], t2, bs); bs = fmaf(dv[c + 3], t3, bs);
           }
+          cq[u] = k < j ? nit2 * cs : -__int_as_float(0x7f800000);
+          bq[u] = k < j ? 2.f * nit2 * bs : 0.f;
         }
         *reinterpret_cast<float4*>(cr + 4 * k4) = make_float4(cq[0], cq[1], cq[2], cq[3]);
         *reinterpret_cast<float4*>(br + 4 * k4) = make_float4(bq[0], bq[1], bq[2], bq[3]);
@@ -512,16 +541,25 @@ __device__ __forceinline__ void ray32_location(const RayParams& P, const int64_t
         const float* cr = Cb + r * KP;
         const float* br = Bb + r * KP;
         const float2 s2v = make_float2(s_eval, s_eval), g2 = make_float2(gam, gam);
-#pragma unroll 1
-        for (int k4 = q; 4 * k4 < j; k4 += G) {
-          const float4 c4 = *reinterpret_cast<const float4*>(cr + 4 * k4);
-          const float4 b4 = *reinterpret_cast<const float4*>(br + 4 * k4);
+        auto quad = [&](const float4& c4, const float4& b4) {
           const float2 t01 = __ffma2_rn(s2v, g2, make_float2(b4.x, b4.y));
           const float2 t23 = __ffma2_rn(s2v, g2, make_float2(b4.z, b4.w));
           const float2 e01 = __ffma2_rn(s2v, t01, make_float2(c4.x, c4.y));
           const float2 e23 = __ffma2_rn(s2v, t23, make_float2(c4.z, c4.w));
-          *reinterpret_cast<float4*>(kzr + 4 * k4) =
-              make_float4(ex2_approx(e01.x), ex2_approx(e01.y), ex2_approx(e23.x), ex2_approx(e23.y));
+          return make_float4(ex2_approx(e01.x), ex2_approx(e01.y), ex2_approx(e23.x),
+                             ex2_approx(e23.y));
+        };
+        // two quads per trip, so that their loads and exponentials overlap
+#pragma unroll 1
+        for (int k4 = q; 4 * k4 < j; k4 += 2 * G) {
+          const bool two = 4 * (k4 + G) < j;
+          const int k5 = two ? k4 + G : k4;
+          const float4 c4 = *reinterpret_cast<const float4*>(cr + 4 * k4);
+          const float4 b4 = *reinterpret_cast<const float4*>(br + 4 * k4);
+          const float4 c5 = *reinterpret_cast<const float4*>(cr + 4 * k5);
+          const float4 b5 = *reinterpret_cast<const float4*>(br + 4 * k5);
+          *reinterpret_cast<float4*>(kzr + 4 * k4) = quad(c4, b4);
+          if (two) *reinterpret_cast<float4*>(kzr + 4 * k5) = quad(c5, b5);
         }
       }
       __syncwarp();
