@@ -244,6 +244,76 @@ knn_pilot(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N,
   }
 }
 
+// The same thresholds for a small batch: one block per location instead of one
+// per 32 locations, whose two passes over the sample a lone location waits for
+// (0.65 ms at S = 32768).  Every thread keeps its at most 32 distances in
+// registers; the bin of the m-th smallest comes from 16 halvings of the 16-bit
+// bin number by counting: 0.062 ms for one location.  A block per location
+// reads the sample once per location, so the batch where the shared form's
+// 0.65 ms wins back is about ten waves of two blocks per SM; the line is drawn
+// at a third of that.
+#define KNN_PILOT1_THREADS 1024
+#define KNN_PILOT1_MAX_M 1024
+template <int PP>
+__global__ void __launch_bounds__(KNN_PILOT1_THREADS)
+knn_pilot1(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N, int64_t S, int p,
+           const double* __restrict__ xref, int64_t M, const double* __restrict__ center,
+           int nc_max, const int32_t* __restrict__ nc_loc, int cap, float* __restrict__ thr_out) {
+  constexpr int T = 32768 / KNN_PILOT1_THREADS;    // S <= 32768
+  __shared__ int cnt[2][KNN_PILOT1_THREADS / 32];
+  const int64_t q = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t stride = N / S;
+  float qf[PP], nq = 0.f;
+#pragma unroll
+  for (int k = 0; k < PP; ++k) {
+    qf[k] = k < p ? (float)(xref[q * p + k] - center[k]) : 0.f;
+    nq = fmaf(qf[k], qf[k], nq);
+  }
+  uint32_t bin[T];
+#pragma unroll
+  for (int u = 0; u < T; ++u) {
+    const int64_t i = (int64_t)u * KNN_PILOT1_THREADS + tid;
+    bin[u] = 0xffffffffu;
+    if (i < S) {
+      const float* x = Xf + i * stride * PP;
+      float dot = 0.f;
+#pragma unroll
+      for (int k = 0; k < PP; k += 4) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(x + k));
+        dot = fmaf(qf[k], v.x, dot);
+        dot = fmaf(qf[k + 1], v.y, dot);
+        dot = fmaf(qf[k + 2], v.z, dot);
+        dot = fmaf(qf[k + 3], v.w, dot);
+      }
+      const float d = fmaf(-2.f, dot, nq + __ldg(nx + i * stride));
+      bin[u] = __float_as_uint(fmaxf(d, 0.f)) >> 15;
+    }
+  }
+  const int nc = nc_loc ? nc_loc[q] : nc_max;
+  const float lam = (float)S * (float)nc / (float)N;
+  int m = (int)ceilf(lam + 4.5f * sqrtf(lam) + 4.f);
+  // expected admitted points m N / S must leave two tiles of room
+  if (m > S || (double)m * (double)N / (double)S > (double)(cap - 2 * LAGP_KNN_TILE)) m = 0;
+  uint32_t b = 0;      // the smallest bin with at least m distances in bins <= it
+  for (int bit = 15; bit >= 0; --bit) {
+    const uint32_t mid = b | ((1u << bit) - 1u);
+    int c = 0;
+#pragma unroll
+    for (int u = 0; u < T; ++u) c += bin[u] <= mid ? 1 : 0;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0) cnt[bit & 1][warp] = c;
+    __syncthreads();
+    c = __reduce_add_sync(0xffffffffu, cnt[bit & 1][lane]);
+    if (c < m) b = mid + 1u;
+  }
+  if (tid == 0) {
+    const float inf = __int_as_float(0x7f800000);
+    const float thr = __uint_as_float((b << 15) | 0x7fffu);
+    thr_out[q] = (m == 0 || !(thr < inf)) ? inf : thr;
+  }
+}
+
 template <int PP>
 __global__ void __launch_bounds__(KNN_WARPS * 32, 3)
 knn_stream(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N, int64_t ntiles,
@@ -608,6 +678,8 @@ cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
   const bool pilot = N >= (int64_t)32 * nc_max;
   const int64_t S = N / 16 < 32768 ? N / 16 : 32768;
   KnnEntry* kbuf = reinterpret_cast<KnnEntry*>(ws.knn_buf);
+  // a batch of a few locations per SM: one pilot block each
+  const bool small = M <= KNN_PILOT1_MAX_M;
   cudaError_t err;
   switch (PP) {
 #define KNN_CASE(V)                                                                          \
@@ -617,8 +689,13 @@ cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
     if (err != cudaSuccess) return err;                                                      \
     if (pilot) {                                                                             \
       prof_begin("knn_pilot", s);                                                            \
-      knn_pilot<V><<<grid, KNN_WARPS * 32, 0, s>>>(ws.Xf, ws.nx, N, S, p, xref, M, ws.center, \
-                                                   nc_max, nc_loc, cap, ws.knn_thr);         \
+      if (small)                                                                             \
+        knn_pilot1<V><<<(unsigned)M, KNN_PILOT1_THREADS, 0, s>>>(                            \
+            ws.Xf, ws.nx, N, S, p, xref, M, ws.center, nc_max, nc_loc, cap, ws.knn_thr);     \
+      else                                                                                   \
+        knn_pilot<V><<<grid, KNN_WARPS * 32, 0, s>>>(ws.Xf, ws.nx, N, S, p, xref, M,         \
+                                                     ws.center, nc_max, nc_loc, cap,         \
+                                                     ws.knn_thr);                            \
       prof_end(s);                                                                           \
     }                                                                                        \
     if (pilot) {                                                                             \
