@@ -28,6 +28,17 @@
 // costs O(N' j) instead of the O(N' j^2) of re-forming every w, and a full
 // design O(N' n^2) instead of O(N' n^3); the sums see the same FP32 operations
 // in the same order as a from-scratch evaluation would.
+// Each step is a chain (new point -> correlations -> new row -> every
+// candidate's entry -> argmax) that waits on binary64 latency, barriers and
+// the cache in L2, so the chain is kept short: the packed factor lies in shared
+// memory (n <= 64), a row's product with the new correlations takes four lanes
+// and a column sum two (one per accumulator), the new row's terms of z and
+// L^{-1} y come from the threads that formed it, and a thread reads the cached
+// rows of four neighbouring candidates in 128-bit loads, eight rows at a time.
+// 25.7 against 35.0 ms per 20,000 locations (8-d, n = 50, N' = 1000) with the
+// factor in global memory, one lane per row and column and 32-bit loads.  Four
+// CTAs of 256 threads per SM keep the slots' caches near the size of L2: five
+// ran 26.8 ms, five or seven of 128 threads 26.8 and 34.1 ms.
 // Scoring coordinates are FP32 and centred on the design's bounding box.
 #include <cstdint>
 
@@ -38,6 +49,9 @@ namespace lagp {
 
 #define D32_THREADS 256
 #define D32_WARPS (D32_THREADS / 32)
+// row stride of the correlation cache and of the per-candidate arrays: four
+// candidates at a time
+#define D32_LDC(nc) (((nc) + 3) & ~3)
 
 struct D32Params {
   const double* X;
@@ -83,6 +97,9 @@ struct L32 {
   double* xq;      // [p]
   double* kvec;    // [n_max]
   double* l;       // [n_max]
+  double* ys;      // [n_max] y of the selected points
+  double* tz;      // [n_max] the new row's terms of z_j
+  double* ty;      // [n_max] and of (L^{-1} y)_j
   double* z;       // [n_max]
   double* zy;      // [n_max]
   double* kx;      // [n_max]
@@ -94,8 +111,13 @@ struct L32 {
   float neg_inv_theta, onepg;
 };
 
-// lengthscale of the CTA's current location (kept out of the registers)
-static __shared__ double d32_theta;
+// -1 / lengthscale of the CTA's current location (kept out of the registers,
+// and divided once per location: a binary64 division by every warp of every
+// step was more than a third of the kernel's binary64 work)
+static __shared__ double d32_nit64;
+
+// start of row i of the packed inverse factor
+__device__ __host__ __forceinline__ int d32_tri(int i) { return i * (i + 1) / 2; }
 
 __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -105,41 +127,25 @@ __device__ __forceinline__ double warp_sumd(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-// Sum over the block of FP64 terms held only by threads below `active`, to
-// thread 0 (the other threads' a, b are left as their warp sums or unchanged).
-// Only the warps holding terms shuffle, and thread 0 adds the warp totals in
-// warp order, so the result is bit-identical to a full block sum (the idle
-// warps' totals are exact zeros) at a fraction of its FP64 instructions,
-// which are scarce on this part.  Every thread must call it.
-__device__ __forceinline__ void sum_to_thread0(double& a, double& b, int active, double* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int aw = min((active + 31) >> 5, D32_WARPS);
-  if (warp < aw) {
-    a = warp_sumd(a);
-    b = warp_sumd(b);
-    if (lane == 0) { red[2 * warp] = a; red[2 * warp + 1] = b; }
+// Sums over the warp's first `active` values of a shared vector pair, each
+// added up as blocks of 32 (a butterfly per block, the block totals in order):
+// the sums sum_i a_i^2 (one vector) or sum_i a_i, sum_i b_i of two vectors.
+// Every lane of the calling warp returns them.
+__device__ __forceinline__ double sum_squares32(const double* a, int active) {
+  const int lane = threadIdx.x & 31;
+  double t = 0.0;
+  for (int i0 = 0; i0 < active; i0 += 32) {
+    const double x = i0 + lane < active ? a[i0 + lane] : 0.0;
+    t += warp_sumd(__dmul_rn(x, x));     // (not contracted into the first addition)
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double ta = 0.0, tb = 0.0;
-    for (int w = 0; w < aw; ++w) { ta += red[2 * w]; tb += red[2 * w + 1]; }
-    a = ta;
-    b = tb;
-  }
+  return t;
 }
-__device__ __forceinline__ void sum_to_thread0(double& a, int active, double* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int aw = min((active + 31) >> 5, D32_WARPS);
-  if (warp < aw) {
-    a = warp_sumd(a);
-    if (lane == 0) red[warp] = a;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double ta = 0.0;
-    for (int w = 0; w < aw; ++w) ta += red[w];
-    a = ta;
-  }
+__device__ __forceinline__ double sum_vector32(const double* a, int active) {
+  const int lane = threadIdx.x & 31;
+  double t = 0.0;
+  for (int i0 = 0; i0 < active; i0 += 32)
+    t += warp_sumd(i0 + lane < active ? a[i0 + lane] : 0.0);
+  return t;
 }
 
 // best (value, index) over the block: larger value wins, ties to the lower index
@@ -185,108 +191,161 @@ __device__ __forceinline__ const float* cand_f(const D32Params& P, const float* 
 // written (the same arithmetic and candidate order as a separate pass).
 __device__ bool add_point32(const D32Params& P, L32& L, const int32_t* cl, const float* crow,
                             int nc, int r, double* Lg, float* Kc_loc, VI* best) {
-  const int tid = threadIdx.x, p = P.p, j = L.j, ld = P.n_max;
+  const int tid = threadIdx.x, p = P.p, j = L.j, warp = tid >> 5;
   const double* c = P.X + (int64_t)cl[r] * p;
   if (tid < p) L.S64[j * p + tid] = c[tid];
   if (tid < P.PP) L.Sf[j * P.PP + tid] = cand_f(P, crow, r)[tid];
-  __syncthreads();
-  const double nit64 = -1.0 / d32_theta;
-  // correlations of the new point with the design, and with x (thread j)
-  for (int i = tid; i <= j; i += blockDim.x) {
-    if (i < j) L.kvec[i] = corr64_fast(L.S64 + i * p, L.S64 + j * p, p, nit64);
-    else L.kx[j] = corr64_fast(L.S64 + j * p, L.xq, p, nit64);
-  }
-  __syncthreads();
-  // l = L_j^{-1} k_j(x_new); thread 0 forms the pivot v = 1 + g - |l|^2, 1/sqrt(v)
-  double vv = 0.0;
-  for (int i = tid; i < j; i += blockDim.x) {
-    const double acc = dot64_ilp(Lg + (int64_t)i * ld, L.kvec, i + 1);
-    L.l[i] = acc;
-    vv = fma(acc, acc, vv);
-  }
-  sum_to_thread0(vv, j, L.dred);
-  double* piv = L.dred + 2 * D32_WARPS;
-  if (tid == 0) {
-    const double v = (1.0 + P.g) - vv;
-    piv[0] = v;
-    piv[1] = v > 0.0 ? 1.0 / sqrt(v) : 0.0;
-  }
-  __syncthreads();
-  if (!(piv[0] > 0.0)) return false;
-  const double inv_d = piv[1];
-  for (int k = tid; k < j; k += blockDim.x) {
-    double a0 = 0.0, a1 = 0.0;
-    int i = k;
-    for (; i + 1 < j; i += 2) {
-      a0 = fma(L.l[i], Lg[(int64_t)i * ld + k], a0);
-      a1 = fma(L.l[i + 1], Lg[(int64_t)(i + 1) * ld + k], a1);
-    }
-    if (i < j) a0 = fma(L.l[i], Lg[(int64_t)i * ld + k], a0);
-    const double rk = -(a0 + a1) * inv_d;
-    Lg[(int64_t)j * ld + k] = rk;
-    L.Lf[k] = (float)rk;
-  }
-  if (tid == 0) {
-    Lg[(int64_t)j * ld + j] = inv_d;
-    L.Lf[j] = (float)inv_d;
+  if (tid == D32_THREADS - 1) {
+    L.ys[j] = P.Y[cl[r]];
     L.sel[j] = r;
     L.used[r] = 1;
   }
   __syncthreads();
-  // z_j = row_j . k(x), (L^{-1} y)_j = row_j . y_S
-  double zz = 0.0, zyy = 0.0;
-  for (int k = tid; k <= j; k += blockDim.x) {
-    const double rk = Lg[(int64_t)j * ld + k];
-    zz = fma(rk, L.kx[k], zz);
-    zyy = fma(rk, P.Y[cl[L.sel[k]]], zyy);
+  const double nit64 = d32_nit64;
+  // correlations of the new point with the design, and with x (thread j)
+  for (int i = tid; i <= j; i += blockDim.x) {
+    const double kv = corr64_fast(i < j ? L.S64 + i * p : L.xq, L.S64 + j * p, p, nit64);
+    if (i < j) L.kvec[i] = kv;
+    else L.kx[j] = kv;
   }
-  sum_to_thread0(zz, zyy, j + 1, L.dred);
-  if (tid == 0) {
-    L.z[j] = zz;
-    L.zy[j] = zyy;
-    L.zf[j] = (float)zz;
+  __syncthreads();
+  // l = L_j^{-1} k_j(x_new): four lanes per row, one for each of dot64_ilp's
+  // accumulators (the first also takes the remainder)
+  for (int i = tid >> 2; i < ((j + 7) & ~7); i += D32_THREADS / 4) {
+    const int t = tid & 3, len = i + 1, len4 = len & ~3;
+    const double* Li = Lg + d32_tri(i);
+    double acc = 0.0;
+    if (i < j) {
+      for (int k = t; k < len4; k += 4) acc = fma(Li[k], L.kvec[k], acc);
+      if (t == 0)
+        for (int k = len4; k < len; ++k) acc = fma(Li[k], L.kvec[k], acc);
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    if (t == 0 && i < j) L.l[i] = acc;
+  }
+  __syncthreads();
+  // the pivot v = 1 + g - |l|^2 and 1 / sqrt(v), on one warp
+  double* piv = L.dred + 2 * D32_WARPS;
+  if (warp == 0) {
+    const double v = (1.0 + P.g) - sum_squares32(L.l, j);
+    if (tid == 0) {
+      piv[1] = v > 0.0 ? 1.0 / sqrt(v) : 0.0;
+      L.ired[2 * D32_WARPS] = v > 0.0 ? 1 : 0;   // an integer for the other warps to test
+    }
+  }
+  __syncthreads();
+  if (!L.ired[2 * D32_WARPS]) return false;
+  const double inv_d = piv[1];
+  // the new row, and its terms of z_j = row_j . k(x) and (L^{-1} y)_j =
+  // row_j . y_S: two lanes per column, one for its even rows and one for its
+  // odd ones (the sum's two accumulators, in either order)
+  double* Lj = Lg + d32_tri(j);
+  for (int k = tid >> 1; k < ((j + 16) & ~15); k += D32_THREADS / 2) {
+    const int h = tid & 1;
+    double acc = 0.0;
+    if (k < j) {
+      const double* Lk = Lg + k;
+      for (int i = k + ((k ^ h) & 1); i < j; i += 2) acc = fma(L.l[i], Lk[d32_tri(i)], acc);
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    if (k <= j && h == 0) {
+      const double rk = k < j ? -acc * inv_d : inv_d;
+      Lj[k] = rk;
+      L.Lf[k] = (float)rk;
+      L.tz[k] = __dmul_rn(rk, L.kx[k]);
+      L.ty[k] = __dmul_rn(rk, L.ys[k]);
+    }
+  }
+  __syncthreads();
+  // both sums side by side on two warps
+  if (warp < 2) {
+    const double t = sum_vector32(warp == 0 ? L.tz : L.ty, j + 1);
+    if (tid == 0) {
+      L.z[j] = t;
+      L.zf[j] = (float)t;
+    }
+    if (tid == 32) L.zy[j] = t;
   }
   __syncthreads();
   // Row j of L^{-1} is final once written, so w_c = L^{-1} k_j(c) only gains
   // the entry w_cj = row_j . K(S_{0..j}, c); |w_c|^2 and w_c . z are running
   // sums in the order i = 0, 1, ..., the same FP32 operations a from-scratch
-  // evaluation at every step would perform.  Thread q owns candidates
-  // q, q + blockDim, ..., and takes the newest entry from the register that
-  // computed it.  Even terms go to a0 and odd terms to a1, in ascending order.
-  const int64_t ldc = P.nc_max;
+  // evaluation at every step would perform.  A thread owns four neighbouring
+  // candidates, so that a row of their cached correlations is one 128-bit load
+  // and eight rows' loads are in flight, and takes the newest entries from the
+  // registers that computed them.  Even terms go to a0 and odd terms to a1, in
+  // ascending order.
+  const int64_t ldc = D32_LDC(P.nc_max);
   float* row = Kc_loc + (int64_t)j * ldc;
   const float* sj = L.Sf + j * P.PP;
   const float* Lfj = L.Lf;
   const float zj = L.zf[j];
   VI b;
   b.v = -1.f; b.v2 = -1.f; b.i = -1;
-  for (int q = tid; q < nc; q += blockDim.x) {
-    const float kv = __expf(sqdist_row32(cand_f(P, crow, q), sj, P.PP) * L.neg_inv_theta);
-    row[q] = kv;
-    if (L.used[q]) continue;
+  for (int q = 4 * tid; q < nc; q += 4 * blockDim.x) {
+    float kv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      kv[u] = __expf(sqdist_row32(cand_f(P, crow, min(q + u, nc - 1)), sj, P.PP) * L.neg_inv_theta);
+    *reinterpret_cast<float4*>(row + q) = make_float4(kv[0], kv[1], kv[2], kv[3]);
     const float* kc = Kc_loc + q;
-    float a0 = 0.f, a1 = 0.f;
+    float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
     int k = 0;
-#pragma unroll 4
-    for (; k + 2 <= j; k += 2) {
-      a0 = fmaf(Lfj[k], kc[k * ldc], a0);
-      a1 = fmaf(Lfj[k + 1], kc[(k + 1) * ldc], a1);
+#pragma unroll 1
+    for (; k + 8 <= j; k += 8) {
+      float4 c[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) c[t] = *reinterpret_cast<const float4*>(kc + (k + t) * ldc);
+#pragma unroll
+      for (int t = 0; t < 8; t += 2) {
+        const float l0 = Lfj[k + t], l1 = Lfj[k + t + 1];
+        a0[0] = fmaf(l0, c[t].x, a0[0]); a1[0] = fmaf(l1, c[t + 1].x, a1[0]);
+        a0[1] = fmaf(l0, c[t].y, a0[1]); a1[1] = fmaf(l1, c[t + 1].y, a1[1]);
+        a0[2] = fmaf(l0, c[t].z, a0[2]); a1[2] = fmaf(l1, c[t + 1].z, a1[2]);
+        a0[3] = fmaf(l0, c[t].w, a0[3]); a1[3] = fmaf(l1, c[t + 1].w, a1[3]);
+      }
     }
-    if (k == j) {
-      a0 = fmaf(Lfj[j], kv, a0);
-    } else {
-      a0 = fmaf(Lfj[k], kc[k * ldc], a0);
-      a1 = fmaf(Lfj[j], kv, a1);
+    if (k < j) {
+      // the last rows (at most seven), loaded together; a missing one is zero
+      float4 c[7];
+#pragma unroll
+      for (int t = 0; t < 7; ++t)
+        c[t] = k + t < j ? *reinterpret_cast<const float4*>(kc + (k + t) * ldc)
+                         : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int t = 0; t < 7; ++t) {
+        if (k + t < j) {
+          const float l = Lfj[k + t];
+          float (&a)[4] = (t & 1) ? a1 : a0;
+          a[0] = fmaf(l, c[t].x, a[0]); a[1] = fmaf(l, c[t].y, a[1]);
+          a[2] = fmaf(l, c[t].z, a[2]); a[3] = fmaf(l, c[t].w, a[3]);
+        }
+      }
     }
-    const float w = a0 + a1;
-    const float nvs = fmaf(w, w, L.vs[q]), nns = fmaf(w, zj, L.ns[q]);
-    L.vs[q] = nvs;
-    L.ns[q] = nns;
-    const float v = L.onepg - nvs;
-    const float num = nns - L.kxc[q];
-    const float alc = v > 0.f ? num * num / v : 0.f;
-    if (alc > b.v) { b.v2 = b.v; b.v = alc; b.i = q; }
-    else if (alc > b.v2) b.v2 = alc;
+    const float lj = Lfj[j];
+    const bool odd = j & 1;
+    float4 vs = *reinterpret_cast<const float4*>(L.vs + q);
+    float4 ns = *reinterpret_cast<const float4*>(L.ns + q);
+    const float4 kx = *reinterpret_cast<const float4*>(L.kxc + q);
+    const uchar4 us = *reinterpret_cast<const uchar4*>(L.used + q);
+    auto finish = [&](int u, float& v_, float& n_, float kx_, unsigned char used) {
+      const float w = odd ? a0[u] + fmaf(lj, kv[u], a1[u]) : fmaf(lj, kv[u], a0[u]) + a1[u];
+      v_ = fmaf(w, w, v_);
+      n_ = fmaf(w, zj, n_);
+      if (used || q + u >= nc) return;
+      const float v = L.onepg - v_;
+      const float num = n_ - kx_;
+      const float alc = v > 0.f ? num * num / v : 0.f;
+      if (alc > b.v) { b.v2 = b.v; b.v = alc; b.i = q + u; }
+      else if (alc > b.v2) b.v2 = alc;
+    };
+    finish(0, vs.x, ns.x, kx.x, us.x);
+    finish(1, vs.y, ns.y, kx.y, us.y);
+    finish(2, vs.z, ns.z, kx.z, us.z);
+    finish(3, vs.w, ns.w, kx.w, us.w);
+    *reinterpret_cast<float4*>(L.vs + q) = vs;
+    *reinterpret_cast<float4*>(L.ns + q) = ns;
   }
   *best = b;
   __syncthreads();
@@ -306,14 +365,16 @@ __device__ int search_exh32(const L32& L, VI best, double* gap_out) {
 
 // PROMOTE: with precision promotion (a separate instantiation, so that the
 // default one carries none of its code)
-template <bool PROMOTE>
-__global__ void __launch_bounds__(D32_THREADS, 6) design32(D32Params P) {
+// SFACTOR: the packed factor in shared memory (d32_smem_factor), else in the
+// slot's global scratch
+template <bool PROMOTE, bool SFACTOR>
+__global__ void __launch_bounds__(D32_THREADS, 4) design32(D32Params P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned s_item;
   const int tid = threadIdx.x, p = P.p, PP = P.PP, ld = P.n_max;
   // scratch of this CTA slot
-  double* Lg = P.Linv + (int64_t)blockIdx.x * ld * ld;
-  float* Kc_loc = P.Kc + (int64_t)blockIdx.x * ld * P.nc_max;
+  const int ncp = D32_LDC(P.nc_max);
+  float* Kc_loc = P.Kc + (int64_t)blockIdx.x * ld * ncp;
   float* crow = P.crow + (int64_t)blockIdx.x * P.nc_max * PP;
 
   L32 L;
@@ -322,26 +383,32 @@ __global__ void __launch_bounds__(D32_THREADS, 6) design32(D32Params P) {
   L.xq = dp; dp += p;
   L.kvec = dp; dp += ld;
   L.l = dp; dp += ld;
+  L.ys = dp; dp += ld;
+  L.tz = dp; dp += ld;
+  L.ty = dp; dp += ld;
   L.z = dp; dp += ld;
   L.zy = dp; dp += ld;
   L.kx = dp; dp += ld;
   L.dred = dp; dp += 4 * D32_WARPS;
-  float* fp = reinterpret_cast<float*>(dp);
+  double* Lg = SFACTOR ? dp : P.Linv + (int64_t)blockIdx.x * ld * ld;
+  if (SFACTOR) dp += d32_tri(ld);
+  // float4 arrays first, on a 16-byte boundary
+  float* fp = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(dp) + 15) & ~(uintptr_t)15);
+  L.vs = fp; fp += ncp;
+  L.ns = fp; fp += ncp;
+  L.kxc = fp; fp += ncp;
+  L.used = reinterpret_cast<unsigned char*>(fp); fp += ncp / 4;
   L.Lf = fp; fp += ld;
   L.zf = fp; fp += ld;
   L.Sf = fp; fp += ld * PP;
   L.xf = fp; fp += PP;
-  L.vs = fp; fp += P.nc_max;
-  L.ns = fp; fp += P.nc_max;
-  L.kxc = fp; fp += P.nc_max;
   L.red = fp; fp += 4 * D32_WARPS;
   int* ip = reinterpret_cast<int*>(fp);
   L.sel = ip; ip += ld;
-  L.ired = ip; ip += 2 * D32_WARPS + 2;
-  L.used = reinterpret_cast<unsigned char*>(ip);
+  L.ired = ip;
   L.onepg = (float)(1.0 + P.g);
   L.neg_inv_theta = (float)(-1.0 / P.theta);
-  if (threadIdx.x == 0) d32_theta = P.theta;
+  if (threadIdx.x == 0) d32_nit64 = -1.0 / P.theta;
   const unsigned items = P.count ? *P.count : (unsigned)P.M;
   for (;;) {
     if (tid == 0) s_item = atomicAdd(P.queue, 1u);
@@ -356,7 +423,7 @@ __global__ void __launch_bounds__(D32_THREADS, 6) design32(D32Params P) {
     L.j = 0;
     if (P.theta_loc) {
       const double th = P.theta_loc[loc];
-      if (tid == 0) d32_theta = th;
+      if (tid == 0) d32_nit64 = -1.0 / th;
       L.neg_inv_theta = (float)(-1.0 / th);
     }
 
@@ -393,17 +460,15 @@ __global__ void __launch_bounds__(D32_THREADS, 6) design32(D32Params P) {
       ok = (r >= 0) && add_point32(P, L, cl, crow, nc, r, Lg, Kc_loc, &part);
     }
     if (ok) {
-      double a = 0.0, b = 0.0, c = 0.0;
-      for (int i = tid; i < L.j; i += blockDim.x) {
-        a = fma(L.z[i], L.zy[i], a);
-        b = fma(L.zy[i], L.zy[i], b);
-        c = fma(L.z[i], L.z[i], c);
-      }
-      sum_to_thread0(a, b, L.j, L.dred);
-      sum_to_thread0(c, L.j, L.dred + 2 * D32_WARPS);
-      if (tid == 0) {
-        P.mean[loc] = a;
-        P.s2[loc] = b * ((1.0 + P.g) - c) / (double)L.j;
+      for (int i = tid; i < L.j; i += blockDim.x) L.tz[i] = __dmul_rn(L.z[i], L.zy[i]);
+      __syncthreads();
+      if (tid < 32) {
+        const double a = sum_vector32(L.tz, L.j), b = sum_squares32(L.zy, L.j);
+        const double c = sum_squares32(L.z, L.j);
+        if (tid == 0) {
+          P.mean[loc] = a;
+          P.s2[loc] = b * ((1.0 + P.g) - c) / (double)L.j;
+        }
       }
     } else if (tid == 0) {
       P.mean[loc] = __longlong_as_double(0x7ff8000000000000ll);
@@ -418,7 +483,7 @@ __global__ void __launch_bounds__(D32_THREADS, 6) design32(D32Params P) {
       // 1 / sqrt(v); a failed update promotes the location
       double vm = ok ? INFINITY : -1.0;
       for (int i = 0; i < L.j; ++i) {
-        const double dg = Lg[(int64_t)i * ld + i];
+        const double dg = Lg[d32_tri(i) + i];
         vm = fmin(vm, 1.0 / (dg * dg));
       }
       promote_location(P.promote, P.promote_count, loc, vm);
@@ -426,11 +491,16 @@ __global__ void __launch_bounds__(D32_THREADS, 6) design32(D32Params P) {
   }
 }
 
+// The packed factor in shared memory while it leaves room for the CTAs that the
+// registers allow; a larger one (up to 66 KB) would halve them.
+static bool d32_smem_factor(int n_max) { return n_max <= 64; }
+
 static size_t smem_design32(int n_max, int p, int PP, int nc_max) {
-  size_t d = (size_t)n_max * p + p + 5 * n_max + 4 * D32_WARPS;
-  size_t f = 2 * (size_t)n_max + (size_t)n_max * PP + PP + 3 * (size_t)nc_max + 4 * D32_WARPS;
+  size_t d = (size_t)n_max * p + p + 8 * n_max + 4 * D32_WARPS + (d32_smem_factor(n_max) ? d32_tri(n_max) : 0);
+  const size_t ncp = D32_LDC(nc_max);
+  size_t f = 2 * (size_t)n_max + (size_t)n_max * PP + PP + 3 * ncp + ncp / 4 + 4 * D32_WARPS;
   size_t i = (size_t)n_max + 2 * D32_WARPS + 2;
-  return d * 8 + f * 4 + i * 4 + nc_max + 16;
+  return d * 8 + f * 4 + i * 4 + 16;
 }
 
 cudaError_t launch_exh32(const DesignArgs& a, cudaStream_t s) {
@@ -445,7 +515,9 @@ cudaError_t launch_exh32(const DesignArgs& a, cudaStream_t s) {
   P.promote = a.promote ? a.ws->promote : nullptr;
   P.promote_count = a.ws->status + 1;
   size_t sm = smem_design32(a.n_max, a.p, a.PP, a.nc_max);
-  auto k = P.promote ? design32<true> : design32<false>;
+  const bool sf = d32_smem_factor(a.n_max);
+  auto k = P.promote ? (sf ? design32<true, true> : design32<true, false>)
+                     : (sf ? design32<false, true> : design32<false, false>);
   cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (err != cudaSuccess) return err;
   const int64_t grid = persistent_grid(k, D32_THREADS, sm, a.M, exh_slots(a.ws->chunk), 1,
