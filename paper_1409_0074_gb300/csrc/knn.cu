@@ -248,12 +248,8 @@ knn_pilot(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N,
 // per 32 locations, whose two passes over the sample a lone location waits for
 // (0.65 ms at S = 32768).  Every thread keeps its at most 32 distances in
 // registers; the bin of the m-th smallest comes from 16 halvings of the 16-bit
-// bin number by counting: 0.062 ms for one location.  A block per location
-// reads the sample once per location, so the batch where the shared form's
-// 0.65 ms wins back is about ten waves of two blocks per SM; the line is drawn
-// at a third of that.
+// bin number by counting: 0.058 ms for one location, 0.36 ms for 1,024.
 #define KNN_PILOT1_THREADS 1024
-#define KNN_PILOT1_MAX_M 1024
 template <int PP>
 __global__ void __launch_bounds__(KNN_PILOT1_THREADS)
 knn_pilot1(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N, int64_t S, int p,
@@ -678,8 +674,11 @@ cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
   const bool pilot = N >= (int64_t)32 * nc_max;
   const int64_t S = N / 16 < 32768 ? N / 16 : 32768;
   KnnEntry* kbuf = reinterpret_cast<KnnEntry*>(ws.knn_buf);
-  // a batch of a few locations per SM: one pilot block each
-  const bool small = M <= KNN_PILOT1_MAX_M;
+  // a batch of a few locations per SM: one pilot block each (per wave of two
+  // blocks per SM about 0.025 ms, 0.05 at S = 32768; the shared form takes its
+  // two passes over the sample whatever the batch: 0.06 ms at S = 2500, 0.61
+  // at S = 32768, p = 8)
+  const bool small = M <= 304 || (M <= 1024 && S >= 16384);
   cudaError_t err;
   switch (PP) {
 #define KNN_CASE(V)                                                                          \
