@@ -44,6 +44,11 @@
 // (2^-23 of the running sum each) and FP32 input rounding, all bounded by
 // multiples of (|a| + |b|)^2; (K + 16) 2^-21 (|a| + |b|)^2, with a 25% margin.
 // Every wait is bounded; a timeout sets LAGP_DEV_TIMEOUT and all roles stop.
+//
+// What bounds it: first the issue of the MMAs (six per design tile at p = 8,
+// 260 cycles each from one lane's branch: 30.5 ms per 100,000 locations against
+// N = 1e6), then, with the issue in uniform code, the epilogue's chain of
+// minimum, vote and branch per four distances (24.0 ms).
 #include <cstdint>
 
 #include "common.cuh"
@@ -113,19 +118,25 @@ __device__ __forceinline__ uint64_t kt_desc(uint32_t addr, uint32_t sbo) {
          ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
 }
 
+// Issued by one elected lane in code that the whole warp runs: descriptors then
+// stay in uniform registers and an MMA issues every 75 cycles (its own time at
+// N = 128), where one lane's branch took 160 to 260 to move them there each time.
 __device__ __forceinline__ void kt_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
                                        uint32_t acc) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "{\n\t.reg .pred p, e;\n\tsetp.ne.u32 p, %4, 0;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
       "l"(a), "l"(b), "r"(idesc), "r"(acc)
       : "memory");
 }
 
+// by the lane that issues the MMAs
 __device__ __forceinline__ void kt_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
+          smem_u32(bar))
+      : "memory");
 }
 
 __device__ __forceinline__ void kt_arrive(uint64_t* bar) {
@@ -136,8 +147,8 @@ __device__ __forceinline__ void kt_epi_barrier() {
   asm volatile("bar.sync %0, %1;" ::"n"(KT_EPI_BAR), "n"(KT_EPI_WARPS * 32) : "memory");
 }
 
-// 64 columns of this thread's TMEM lane: two 32-column loads, one wait
-__device__ __forceinline__ void kt_ld32x2(uint32_t addr, uint32_t (&v)[64]) {
+// 32 columns of this thread's TMEM lane
+__device__ __forceinline__ void kt_ld32(uint32_t addr, uint32_t (&v)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
       "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
@@ -147,16 +158,6 @@ __device__ __forceinline__ void kt_ld32x2(uint32_t addr, uint32_t (&v)[64]) {
         "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]),
         "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
       : "r"(addr));
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-      "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(v[32]), "=r"(v[33]), "=r"(v[34]), "=r"(v[35]), "=r"(v[36]), "=r"(v[37]),
-        "=r"(v[38]), "=r"(v[39]), "=r"(v[40]), "=r"(v[41]), "=r"(v[42]), "=r"(v[43]),
-        "=r"(v[44]), "=r"(v[45]), "=r"(v[46]), "=r"(v[47]), "=r"(v[48]), "=r"(v[49]),
-        "=r"(v[50]), "=r"(v[51]), "=r"(v[52]), "=r"(v[53]), "=r"(v[54]), "=r"(v[55]),
-        "=r"(v[56]), "=r"(v[57]), "=r"(v[58]), "=r"(v[59]), "=r"(v[60]), "=r"(v[61]),
-        "=r"(v[62]), "=r"(v[63])
-      : "r"(addr + 32));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
@@ -178,6 +179,38 @@ struct KtSmem {
   static constexpr int BYTES = (MISC_OFF + 16 + 1024) > 120 * 1024 ? (MISC_OFF + 16 + 1024)
                                                                    : 120 * 1024;
 };
+
+// Appends a point to a location's buffer (entries past its room are counted
+// but not kept): slot n of the thread's quarter or, of a split launch, the next
+// slot of the buffer that the location's segments share.
+template <bool SPLIT>
+__device__ __forceinline__ void kt_put(float d, int32_t idx, KnnEntry* qb, int room,
+                                       int32_t* counter, int n) {
+  KnnEntry e;
+  e.d = fmaxf(d, 0.f);
+  e.idx = idx;
+  const int slot = SPLIT ? atomicAdd(counter, 1) : n;
+  if (slot < room) qb[slot] = e;
+}
+
+// The passes among four neighbouring distances; how many, and how many lie at
+// or below the pilot value.  Rare (some lane has two), and kept out of line: in
+// line it made the unrolled epilogue 40 KB of code.
+template <bool SPLIT>
+__device__ __forceinline__ int2 kt_put4(float4 d, float keep, float thr, int32_t idx, KnnEntry* qb,
+                                     int room, int32_t* counter, int n) {
+  const float v[4] = {d.x, d.y, d.z, d.w};
+  int2 add = make_int2(0, 0);
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    if (v[u] <= keep) {
+      kt_put<SPLIT>(v[u], idx + u, qb, room, counter, n + add.x);
+      ++add.x;
+      add.y += (v[u] <= thr) ? 1 : 0;
+    }
+  }
+  return add;
+}
 
 template <int KA, bool SPLIT>
 __global__ void __launch_bounds__(KT_THREADS, 1)
@@ -203,7 +236,8 @@ knn_tc(const float* __restrict__ Btiles, int64_t ntiles, int p, const double* __
   uint32_t* tmem_base = reinterpret_cast<uint32_t*>(smem + L::MISC_OFF);
   int* abort_flag = reinterpret_cast<int*>(smem + L::MISC_OFF + 4);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // (the warp's number from lane 0, so that branches on it are uniform)
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int64_t q0 = (tile0 + (int64_t)blockIdx.x) * KT_M;
   // design segment of this CTA: tiles [t_lo, t_lo + nt) (the whole design
   // unless the launch splits it over gridDim.y CTAs per location tile)
@@ -269,14 +303,16 @@ knn_tc(const float* __restrict__ Btiles, int64_t ntiles, int p, const double* __
   const uint32_t taddr = *tmem_base;
   volatile int* abort_v = abort_flag;
 
+  const int nti = (int)nt;
   if (warp == KT_EPI_WARPS) {
     // ---------------- producer ----------------
     if (lane == 0) {
-      int64_t issued = 0;
-      for (int64_t t = 0; t < nt; ++t) {
-        const int s = (int)(t % KT_STAGES);
+      int issued = 0;
+      int s = 0;
+      uint32_t ph = 1;          // phase of empty[s] to wait for, one ring behind
+      for (int t = 0; t < nti; ++t) {
         if (t >= KT_STAGES) {
-          if (*abort_v || !mbar_wait(&empty[s], (uint32_t)(((t / KT_STAGES) - 1) & 1))) {
+          if (*abort_v || !mbar_wait(&empty[s], ph)) {
             *abort_v = 1;
             break;
           }
@@ -285,45 +321,48 @@ knn_tc(const float* __restrict__ Btiles, int64_t ntiles, int p, const double* __
         bulk_g2s(smem + L::S_OFF + s * L::STAGE_BYTES,
                  Btiles + (t_lo + t) * (int64_t)(L::STAGE_BYTES / 4), L::STAGE_BYTES, &full[s]);
         issued = t + 1;
+        if (++s == KT_STAGES) { s = 0; ph ^= 1u; }
       }
       if (*abort_v) {   // copies in flight land before the CTA can exit
-        for (int64_t t = issued > KT_STAGES ? issued - KT_STAGES : 0; t < issued; ++t)
+        for (int t = issued > KT_STAGES ? issued - KT_STAGES : 0; t < issued; ++t)
           mbar_wait(&full[t % KT_STAGES], (uint32_t)((t / KT_STAGES) & 1));
       }
     }
   } else if (warp == KT_EPI_WARPS + 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(KT_N >> 3) << 17) |
-                             ((uint32_t)(KT_M >> 4) << 24);
-      const uint32_t sbo = (KA / 4) * 128;
-      const uint32_t a_hi = smem_u32(Ahi), a_lo = smem_u32(Alo);
-      int64_t committed = 0;
-      for (int64_t t = 0; t < nt; ++t) {
-        const int s = (int)(t % KT_STAGES), b = (int)(t % KT_GROUPS);
-        bool ok = !*abort_v && mbar_wait(&full[s], (uint32_t)((t / KT_STAGES) & 1));
-        if (ok && t >= KT_GROUPS)
-          ok = !*abort_v && mbar_wait(&tempty[b], (uint32_t)(((t / KT_GROUPS) - 1) & 1));
-        if (!ok) { *abort_v = 1; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t b_hi = smem_u32(smem + L::S_OFF + s * L::STAGE_BYTES);
-        const uint32_t b_lo = b_hi + L::TILE_BYTES;
-        const uint32_t d = taddr + (uint32_t)(b * KT_N);
+    // ---------------- MMA issuer (the whole warp; one lane issues) ----------------
+    const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(KT_N >> 3) << 17) |
+                           ((uint32_t)(KT_M >> 4) << 24);
+    const uint32_t sbo = (KA / 4) * 128;
+    const uint64_t a_hi = kt_desc(smem_u32(Ahi), sbo), a_lo = kt_desc(smem_u32(Alo), sbo);
+    const uint64_t b_hi0 = kt_desc(smem_u32(smem + L::S_OFF), sbo);
+    int committed = 0, s = 0;
+    uint32_t ph = 0;
+    for (int t = 0; t < nti; ++t) {
+      const int b = t % KT_GROUPS;
+      bool ok = !*abort_v && mbar_wait(&full[s], ph);
+      if (ok && t >= KT_GROUPS)
+        ok = !*abort_v && mbar_wait(&tempty[b], (uint32_t)(((t / KT_GROUPS) - 1) & 1));
+      if (!__all_sync(0xffffffffu, ok)) { *abort_v = 1; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      // (addresses below 256 KB: adding to the address field does not carry)
+      const uint64_t b_hi = b_hi0 + (uint64_t)(s * (L::STAGE_BYTES >> 4));
+      const uint64_t b_lo = b_hi + (L::TILE_BYTES >> 4);
+      const uint32_t d = taddr + (uint32_t)(b * KT_N);
 #pragma unroll
-        for (int ks = 0; ks < KA / 8; ++ks) {
-          const uint32_t ko = ks * 256;
-          kt_mma(d, kt_desc(a_hi + ko, sbo), kt_desc(b_hi + ko, sbo), idesc, ks > 0 ? 1u : 0u);
-          kt_mma(d, kt_desc(a_hi + ko, sbo), kt_desc(b_lo + ko, sbo), idesc, 1u);
-          kt_mma(d, kt_desc(a_lo + ko, sbo), kt_desc(b_hi + ko, sbo), idesc, 1u);
-        }
-        kt_commit(&empty[s]);
-        kt_commit(&tfull[b]);
-        committed = t + 1;
+      for (int ks = 0; ks < KA / 8; ++ks) {
+        const uint64_t ko = ks * (256 >> 4);
+        kt_mma(d, a_hi + ko, b_hi + ko, idesc, ks > 0 ? 1u : 0u);
+        kt_mma(d, a_hi + ko, b_lo + ko, idesc, 1u);
+        kt_mma(d, a_lo + ko, b_hi + ko, idesc, 1u);
       }
-      if (*abort_v && committed > 0) {   // the last MMAs finish before TMEM is freed
-        const int64_t t = committed - 1;
-        mbar_wait(&tfull[t % KT_GROUPS], (uint32_t)((t / KT_GROUPS) & 1));
-      }
+      kt_commit(&empty[s]);
+      kt_commit(&tfull[b]);
+      committed = t + 1;
+      if (++s == KT_STAGES) { s = 0; ph ^= 1u; }
+    }
+    if (*abort_v && committed > 0) {   // the last MMAs finish before TMEM is freed
+      const int t = committed - 1;
+      mbar_wait(&tfull[t % KT_GROUPS], (uint32_t)((t / KT_GROUPS) & 1));
     }
   } else {
     // ---------------- epilogue ----------------
@@ -333,9 +372,13 @@ knn_tc(const float* __restrict__ Btiles, int64_t ntiles, int p, const double* __
     const uint32_t lane_base = taddr + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(g * KT_N);
     const float keep = keep_sm[c], thr = thr_sm[c];
     const int seg = cap / KT_GROUPS;                       // this group's quarter of the buffer
-    KnnEntry* qb = buf + q * (int64_t)cap + g * seg;
+    // where this thread's passes go: its quarter of the buffer or, of a split
+    // launch, the whole buffer through the location's counter
+    KnnEntry* qb = buf + q * (int64_t)cap + (SPLIT ? 0 : g * seg);
+    int32_t* counter = seg_out + q * KT_GROUPS;
+    const int room = SPLIT ? cap : seg;
     int mycnt = 0, mybelow = 0;
-    for (int64_t t = g; t < nt; t += KT_GROUPS) {
+    for (int t = g; t < nti; t += KT_GROUPS) {
       const bool ok = !*abort_v && mbar_wait(&tfull[g], (uint32_t)((t / KT_GROUPS) & 1));
       if (!__all_sync(0xffffffffu, ok)) *abort_v = 1;
       if (*abort_v) {
@@ -347,42 +390,36 @@ knn_tc(const float* __restrict__ Btiles, int64_t ntiles, int p, const double* __
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int32_t pbase = (int32_t)((t_lo + t) * KT_N);
 #pragma unroll 1
-      for (int c0 = 0; c0 < KT_N; c0 += 64) {
-        // two 32-column loads, one wait
-        uint32_t v[64];
-        kt_ld32x2(lane_base + c0, v);
-        if (c0 == KT_N - 64) {
+      for (int c0 = 0; c0 < KT_N; c0 += 32) {
+        uint32_t v[32];
+        kt_ld32(lane_base + c0, v);
+        if (c0 == KT_N - 32) {
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
           kt_arrive(&tempty[g]);
         }
 #pragma unroll
-        for (int u4 = 0; u4 < 64; u4 += 4) {
+        for (int u4 = 0; u4 < 32; u4 += 4) {
           // at a pass rate of ~0.2%, most 4-value groups hold no pass in any
           // lane of the warp: the group's minimum, one vote, and the group is
-          // skipped without a compare and branch per value
-          const float m4 = fminf(fminf(__uint_as_float(v[u4]), __uint_as_float(v[u4 + 1])),
-                                 fminf(__uint_as_float(v[u4 + 2]), __uint_as_float(v[u4 + 3])));
+          // skipped without a compare and branch per value.  In most of the
+          // others no lane has more than one: it is the lane's minimum.
+          const float d0 = __uint_as_float(v[u4]), d1 = __uint_as_float(v[u4 + 1]);
+          const float d2 = __uint_as_float(v[u4 + 2]), d3 = __uint_as_float(v[u4 + 3]);
+          const float m4 = fminf(fminf(d0, d1), fminf(d2, d3));
           if (!__any_sync(0xffffffffu, m4 <= keep)) continue;
-#pragma unroll
-          for (int u = u4; u < u4 + 4; ++u) {
-            const float d = __uint_as_float(v[u]);
-            if (d <= keep) {
-              if (SPLIT) {
-                // segments of one location share its buffer through a counter
-                KnnEntry e;
-                e.d = fmaxf(d, 0.f);
-                e.idx = pbase + c0 + u;
-                const int slot = atomicAdd(&seg_out[q * KT_GROUPS], 1);
-                if (slot < cap) buf[q * (int64_t)cap + slot] = e;
-              } else if (mycnt < seg) {
-                KnnEntry e;
-                e.d = fmaxf(d, 0.f);
-                e.idx = pbase + c0 + u;
-                qb[mycnt] = e;
-              }
+          const int np = (d0 <= keep) + (d1 <= keep) + (d2 <= keep) + (d3 <= keep);
+          if (!__any_sync(0xffffffffu, np > 1)) {
+            if (np) {
+              const int u = m4 == d0 ? 0 : (m4 == d1 ? 1 : (m4 == d2 ? 2 : 3));
+              kt_put<SPLIT>(m4, pbase + c0 + u4 + u, qb, room, counter, mycnt);
               ++mycnt;
-              mybelow += (d <= thr) ? 1 : 0;
+              mybelow += (m4 <= thr) ? 1 : 0;
             }
+          } else {
+            const int2 add = kt_put4<SPLIT>(make_float4(d0, d1, d2, d3), keep, thr,
+                                            pbase + c0 + u4, qb, room, counter, mycnt);
+            mycnt += add.x;
+            mybelow += add.y;
           }
         }
       }
