@@ -11,23 +11,33 @@
 //     W = Kc L_j^{-T}   (row r: w_r = L_j^{-1} k_j(c_r)),
 //     v_r = 1 + g - |w_r|^2,  num_r = w_r . z - K(c_r, x),  ALC_r = num_r^2 / v_r,
 // z = L_j^{-1} k_j(x).  W is a tcgen05.mma kind::tf32 product of 128-candidate
-// tiles (M = 128) with L_j^{-1} (N = j rounded up to 16, K = j rounded up to
-// 8), 3xTF32 (hi*hi + hi*lo + lo*hi, FP32 accumulation in TMEM).  Thread t of
-// the CTA owns candidate row t of a tile: it writes that row of the A operand,
-// reads its row of W back from TMEM (tcgen05.ld 32x32b) and reduces v and
-// num.  The block argmax (ties to the lower rank) picks the next point.
+// tiles (M = 128) with rows of L_j^{-1} (N = 16, K = j rounded up to 8), 3xTF32
+// (hi*hi + hi*lo + lo*hi, FP32 accumulation in TMEM).  L_j^{-1} only gains a
+// row per step, so a column of W, once formed, does not change (the products
+// past its diagonal are exact zeros); a step forms the newest column only and
+// adds it to every candidate's running |w_r|^2 and w_r . z.  Thread t of the
+// CTA owns candidate row t of every tile: it reads the column from TMEM
+// (tcgen05.ld 32x32b) and scores its candidates.  The block argmax (ties to the
+// lower rank) picks the next point.
 //
-// FP64 state (the partitioned update in factored form, Sec 2.2): L_j^{-1} in
-// global memory, grown by one row per step, and z, L^{-1} y; the predictive
-// equations (Eq. predgp, preds2) at the end.  Each new row of L^{-1} is also
-// written, split into TF32 hi + lo, into the B operand in shared memory.
+// FP64 state (the partitioned update in factored form, Sec 2.2): L_j^{-1},
+// packed by rows in shared memory, grown by one row per step, and z, L^{-1} y;
+// the predictive equations (Eq. predgp, preds2) at the end.  The rows of the
+// current block of 16 are also kept, split into TF32 hi + lo, as the B operand.
 //
 // The correlation cache is kept in global memory already in the A operand's
-// form: per 128-candidate tile, TF32 hi and lo blocks in the canonical K-major
-// layout (XT_KMAX columns); each step writes one column (N' exponentials).
-// A tile's operand then arrives by bulk copies (TMA), 16 row groups of jk/4
-// core matrices each for hi and lo, and the copy of the next tile runs while
-// the epilogue reads the current tile's scores from TMEM.
+// form: per 128-candidate tile, TF32 hi and lo in slabs of 8 columns; each step
+// writes one column (N' exponentials).  A tile's operand arrives in pieces of 16
+// columns, one bulk copy (TMA) each, through a ring of four buffers: copies run
+// two pieces ahead of the MMAs (warp 0 issues both), and up to XT_GROUP tiles
+// run before their columns are read, each with its own TMEM columns.  (In 32
+// copies of a row group each, a piece took over 3,000 cycles: the copy unit's
+// time goes by copies, not bytes.)
+//
+// A step is a chain of latencies (copies, MMAs, the binary64 update, barriers)
+// on two CTAs per SM; with W formed whole at every step, one tile at a time
+// between three block barriers, and the factor in global memory, the kernel
+// took 52.8 ms per 10,000 locations (8-d, n = 50, N' = 1000); it takes 41.4 ms.
 #include <cstdint>
 
 #include "common.cuh"
@@ -37,6 +47,9 @@ namespace lagp {
 
 #define XT_THREADS 128
 #define XT_KMAX 64     // largest local design on this path
+#define XT_KC 16       // columns of an A operand piece
+#define XT_RING 4      // pieces in shared memory
+#define XT_GROUP 8     // candidate tiles whose scores are in TMEM at a time
 
 struct XtParams {
   const double* X;
@@ -58,7 +71,6 @@ struct XtParams {
   int32_t* selected;
   double* tie_gap;
   int32_t* nevals;
-  double* Linv;          // [slots][n_max][n_max]
   float* Kc;             // [slots][ceil(nc_max / 128)] tiles of 2 x 128 x XT_KMAX floats
   float* crow;           // [slots][nc_max][PP] the location's candidates' FP32 rows
   unsigned* status;
@@ -71,9 +83,17 @@ struct XtParams {
 
 #define XT_TILE_FLOATS (128 * XT_KMAX)   // one of hi / lo of a 128-candidate tile
 
-// canonical no-swizzle K-major layout with XT_KMAX columns per row
+// B operand: canonical no-swizzle K-major layout with XT_KMAX columns per row
 __device__ __forceinline__ uint32_t xcanon(int row, int k) {
   return (uint32_t)((row >> 3) * ((XT_KMAX >> 2) * 128) + (k >> 2) * 128 + (row & 7) * 16 +
+                    (k & 3) * 4);
+}
+// A operand of a tile, in bytes: per 8 columns (one MMA's K) a slab of the 128
+// rows' hi and then lo parts, each canonical, so that any run of columns is
+// one contiguous copy
+#define XT_SLAB 8192
+__device__ __forceinline__ uint32_t xslab(int row, int k) {
+  return (uint32_t)((k >> 3) * XT_SLAB + (row >> 3) * 256 + ((k >> 2) & 1) * 128 + (row & 7) * 16 +
                     (k & 3) * 4);
 }
 
@@ -83,34 +103,53 @@ __device__ __forceinline__ float xtf32(float v) {
   return __uint_as_float(r);
 }
 
-__device__ __forceinline__ uint64_t xdesc(uint32_t addr) {
-  const uint32_t lbo = 128, sbo = (XT_KMAX / 4) * 128;
+// operand descriptor: sbo, the bytes from one 8-row group to the next
+__device__ __forceinline__ uint64_t xdesc(uint32_t addr, uint32_t sbo) {
+  const uint32_t lbo = 128;
   return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
          ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
+}
+
+// MMAs and their commits are issued by one elected lane in code that the whole
+// warp runs, so that the descriptors stay in uniform registers (75 cycles an
+// MMA; from one lane's branch, 160 and more)
+__device__ __forceinline__ void xcommit(uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
+          smem_u32(bar))
+      : "memory");
 }
 
 __device__ __forceinline__ void xmma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
                                      uint32_t acc) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "{\n\t.reg .pred p, e;\n\tsetp.ne.u32 p, %4, 0;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
       "l"(a), "l"(b), "r"(idesc), "r"(acc)
       : "memory");
 }
 
-// 16 columns of this thread's TMEM lane
-__device__ __forceinline__ void xld16(uint32_t addr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-      "%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(addr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// one column of this thread's TMEM lane (complete after xwait_ld)
+__device__ __forceinline__ float xld1(uint32_t addr) {
+  uint32_t r;
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(addr));
+  return __uint_as_float(r);
+}
+
+// row start of the packed factor
+__device__ __host__ __forceinline__ int xtri(int i) { return i * (i + 1) / 2; }
+
+// sum_{i=k..j-1} u[i] L_ik over the packed factor, in coldot64_ilp8's order
+__device__ __forceinline__ double xcoldot(const double* u, const double* L, int k, int j) {
+  double a[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  int i = k;
+  for (; i + 7 < j; i += 8) {
 #pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+    for (int t = 0; t < 8; ++t) a[t] = fma(u[i + t], L[xtri(i + t) + k], a[t]);
+  }
+  for (; i < j; ++i) a[0] = fma(u[i], L[xtri(i) + k], a[0]);
+  return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
 }
 
 // block sums of two values at once (one pass of shuffles and barriers)
@@ -156,11 +195,11 @@ __device__ __forceinline__ void xsum_t0(double& v, int active, double* red) {
 }
 
 struct XtSmem {
-  static constexpr int B_BYTES = XT_KMAX * XT_KMAX * 4;   // L^{-1} rows, one of hi / lo
-  static constexpr int A_BYTES = 128 * XT_KMAX * 4;       // candidate tile, one of hi / lo
+  static constexpr int B_BYTES = 16 * XT_KMAX * 4;        // rows of L^{-1}, one of hi / lo
+  static constexpr int A_BYTES = XT_KC / 8 * XT_SLAB;     // an A piece
   static constexpr int B_OFF = 0;
   static constexpr int A_OFF = 2 * B_BYTES;
-  static constexpr int END = A_OFF + 2 * A_BYTES;         // 96 KB
+  static constexpr int END = A_OFF + XT_RING * A_BYTES;   // 72 KB
 };
 
 __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
@@ -169,15 +208,16 @@ __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   float* Bhi = reinterpret_cast<float*>(smem + XtSmem::B_OFF);
   float* Blo = Bhi + XtSmem::B_BYTES / 4;
-  float* Ahi = reinterpret_cast<float*>(smem + XtSmem::A_OFF);
-  float* Alo = Ahi + XtSmem::A_BYTES / 4;
-  // ld: row stride of the slot's L^{-1} (the part of a mixed launch that runs
-  // here has n <= XT_KMAX); ldo: row stride of the per-step outputs
+  // ld: rows of the packed factor (the part of a mixed launch that runs here
+  // has n <= XT_KMAX); ldo: row stride of the per-step outputs
   const int p = P.p, PP = P.PP, ldo = P.n_max, nc_max = P.nc_max;
   const int ld = ldo < XT_KMAX ? ldo : XT_KMAX;
+  const int ncp = (nc_max + 3) & ~3;
   // small state after the operands
   float* kap = reinterpret_cast<float*>(smem + XtSmem::END);          // [nc_max]
-  float* zf = kap + ((nc_max + 3) & ~3);                             // [XT_KMAX]
+  float* vsum = kap + ncp;                                           // [nc_max] |w_r|^2
+  float* nsum = vsum + ncp;                                          // [nc_max] w_r . z
+  float* zf = nsum + ncp;                                            // [XT_KMAX]
   double* S64 = reinterpret_cast<double*>(zf + XT_KMAX);              // [XT_KMAX][p], 16B aligned
   double* kx = S64 + XT_KMAX * p;                                     // [XT_KMAX]
   double* z = kx + XT_KMAX;
@@ -186,24 +226,26 @@ __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
   double* lv = kv + XT_KMAX;
   double* ys = lv + XT_KMAX;                                          // [XT_KMAX] y of S
   double* red = ys + XT_KMAX;                                         // [8]
-  float* fred = reinterpret_cast<float*>(red + 8);                    // [8]
+  double* Lg = red + 8;                                               // [ld (ld + 1) / 2]
+  float* fred = reinterpret_cast<float*>(Lg + xtri(ld));              // [8]
   int* ired = reinterpret_cast<int*>(fred + 8);                       // [8]
   int* sel = ired + 8;                                                // [XT_KMAX]
   unsigned char* used = reinterpret_cast<unsigned char*>(sel + XT_KMAX);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(
-      (reinterpret_cast<uintptr_t>(used + nc_max) + 15) & ~(uintptr_t)15);   // MMA done
-  uint64_t* bar_a = bar + 1;                                                  // A tile loaded
-  uint32_t* tbase = reinterpret_cast<uint32_t*>(bar + 2);
+  uint64_t* full = reinterpret_cast<uint64_t*>(
+      (reinterpret_cast<uintptr_t>(used + nc_max) + 15) & ~(uintptr_t)15);   // [XT_RING] piece loaded
+  uint64_t* freed = full + XT_RING;                                           // [XT_RING] piece used
+  uint64_t* gdone = freed + XT_RING;                                          // group's MMAs done
+  uint32_t* tbase = reinterpret_cast<uint32_t*>(gdone + 1);
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   unsigned* s_item = tbase + 1;
   if (tid == 0) {
-    mbar_init(bar, 1);
-    mbar_init(bar_a, 1);
+    for (int b = 0; b < XT_RING; ++b) { mbar_init(&full[b], 1); mbar_init(&freed[b], 1); }
+    mbar_init(gdone, 1);
     fence_mbar_init();
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;" ::"r"(
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(
         smem_u32(tbase)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
@@ -213,7 +255,6 @@ __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
   const uint32_t taddr = *tbase;
   // scratch of this CTA slot; the correlation tiles start zeroed, so that the
   // columns past j and the rows past N' that the MMAs read hold finite values
-  double* Lg = P.Linv + (int64_t)blockIdx.x * ld * ld;
   const int ntc = (nc_max + 127) / 128;
   float* Kc = P.Kc + (int64_t)blockIdx.x * ntc * 2 * XT_TILE_FLOATS;
   float* crow = P.crow + (int64_t)blockIdx.x * nc_max * PP;
@@ -221,11 +262,12 @@ __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
     reinterpret_cast<float4*>(Kc)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   asm volatile("fence.proxy.async.global;" ::: "memory");
   __syncthreads();
-  uint32_t phase_a = 0;
-  bool a_pending = false, m_pending = false;   // a bulk copy / MMA not yet waited for
+  // warp 0: pieces copied and pieces whose MMAs were committed, over the
+  // kernel's life; piece m uses buffer m % XT_RING in its m / XT_RING-th phase
+  uint32_t copied = 0, issued = 0;
+  uint32_t gphase = 0;
   const float onepg = (float)(1.0 + P.g);
   const unsigned items = P.count ? *P.count : (unsigned)P.M;
-  uint32_t phase = 0;
   bool timed_out = false;
   while (!timed_out) {
     if (tid == 0) *s_item = atomicAdd(P.queue, 1u);
@@ -247,6 +289,8 @@ __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
     // correlation column of every step then reads them contiguously), and K(c_r, x)
     for (int r = tid; r < nc; r += XT_THREADS) {
       used[r] = 0;
+      vsum[r] = 0.f;
+      nsum[r] = 0.f;
       const float* c = P.Xf + (int64_t)cl[r] * PP;
       float d = 0.f;
       for (int k = 0; k < PP; k += 4) {
@@ -266,55 +310,49 @@ __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
     int j = 0;
     bool ok = (n >= P.n0) && (n <= nc) && (n <= ld);
 
-    // ---- append candidate rank rr: FP64 factor row, z, L^{-1}y, B row, Kc row ----
+    // ---- append candidate rank rr: FP64 factor row, z, L^{-1}y, B row, Kc column ----
     auto add_point = [&](int rr) -> bool {
       const double* c = P.X + (int64_t)cl[rr] * p;
       if (tid < p) S64[j * p + tid] = c[tid];
+      if (tid == XT_THREADS - 1) {
+        ys[j] = P.Y[cl[rr]];
+        sel[j] = rr;
+        used[rr] = 1;
+      }
       __syncthreads();
-      // correlations of the new point with the design (and with x, on the idle thread j)
-      for (int i = tid; i <= j; i += XT_THREADS) {
-        if (i < j) {
-          kv[i] = corr64_fast(S64 + i * p, S64 + j * p, p, nit64);
-        } else {
-          kx[j] = corr64_fast(S64 + j * p, xq, p, nit64);
-          ys[j] = P.Y[cl[rr]];
-          sel[j] = rr;
-          used[rr] = 1;
-        }
+      // correlations of the new point with the design, and with x
+      if (tid <= j) {
+        const double k = corr64_fast(tid < j ? S64 + tid * p : xq, S64 + j * p, p, nit64);
+        if (tid < j) kv[tid] = k;
+        else kx[j] = k;
       }
       __syncthreads();
       double vv = 0.0;
-      for (int i = tid; i < j; i += XT_THREADS) {
-        const double* Li = Lg + (int64_t)i * ld;
-        const double acc = dot64_ilp8(Li, kv, i + 1);
-        lv[i] = acc;
-        vv = fma(acc, acc, vv);
+      if (tid < j) {
+        const double acc = dot64_ilp8(Lg + xtri(tid), kv, tid + 1);
+        lv[tid] = acc;
+        vv = __dmul_rn(acc, acc);
       }
       // thread 0 forms the pivot v = 1 + g - |l|^2 and 1 / sqrt(v)
       xsum_t0(vv, j, red);
       if (tid == 0) {
         const double v = (1.0 + P.g) - vv;
-        red[0] = v;
         red[1] = v > 0.0 ? 1.0 / sqrt(v) : 0.0;
+        ired[5] = v > 0.0 ? 1 : 0;
       }
       __syncthreads();
-      if (!(red[0] > 0.0)) return false;
+      if (!ired[5]) return false;
       const double inv_d = red[1];
-      for (int k = tid; k <= j; k += XT_THREADS) {
-        double rk = inv_d;
-        if (k < j) rk = -coldot64_ilp8(lv, Lg, ld, k, j) * inv_d;
-        Lg[(int64_t)j * ld + k] = rk;
+      double zz = 0.0, zyy = 0.0;
+      if (tid <= j) {
+        const double rk = tid < j ? -xcoldot(lv, Lg, tid, j) * inv_d : inv_d;
+        Lg[xtri(j) + tid] = rk;
         const float h = xtf32((float)rk);
-        const uint32_t off = xcanon(j, k) >> 2;
+        const uint32_t off = xcanon(j & 15, tid) >> 2;
         Bhi[off] = h;
         Blo[off] = xtf32((float)(rk - (double)h));
-      }
-      __syncthreads();
-      double zz = 0.0, zyy = 0.0;
-      for (int k = tid; k <= j; k += XT_THREADS) {
-        const double rk = Lg[(int64_t)j * ld + k];
-        zz = fma(rk, kx[k], zz);
-        zyy = fma(rk, ys[k], zyy);
+        zz = __dmul_rn(rk, kx[tid]);
+        zyy = __dmul_rn(rk, ys[tid]);
       }
       xsum2_t0(zz, zyy, j + 1, red);
       if (tid == 0) {
@@ -325,13 +363,14 @@ __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
       // correlation cache column j: K(c_r, S_j) for every candidate, as A operand
       // (TF32 hi / lo) of its tile; then visible to the bulk copies
       const float* sj = crow + (int64_t)rr * PP;
+#pragma unroll 4
       for (int q = tid; q < nc; q += XT_THREADS) {
-        const float kv = __expf(sqdist_row32(crow + (int64_t)q * PP, sj, PP) * nit);
-        const float h = xtf32(kv);
+        const float kc = __expf(sqdist_row32(crow + (int64_t)q * PP, sj, PP) * nit);
+        const float h = xtf32(kc);
         float* tile = Kc + (int64_t)(q >> 7) * 2 * XT_TILE_FLOATS;
-        const uint32_t off = xcanon(q & 127, j) >> 2;
+        const uint32_t off = xslab(q & 127, j) >> 2;
         tile[off] = h;
-        tile[XT_TILE_FLOATS + off] = xtf32(kv - h);
+        tile[XT_SLAB / 8 + off] = xtf32(kc - h);
       }
       // this step's generic writes (the B row in shared memory, the cache column
       // in global memory) become visible to the tensor core and the bulk copies
@@ -342,90 +381,111 @@ __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
       return true;
     };
 
-    for (int rr = 0; rr < P.n0 && ok; ++rr) ok = add_point(rr);
-
-    for (int step = P.n0; step < n && ok; ++step) {
-      const int jn = (j + 15) & ~15;       // N of the MMA
-      const int jk = (j + 7) & ~7;         // K of the MMA
-      const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(jn >> 3) << 17) |
-                             ((uint32_t)(128 >> 4) << 24);
-      float best = -1.f, second = -1.f;
-      int bi = -1;
-      // A tile t: 16 row groups x (jk / 4) core matrices of hi and of lo, one bulk
-      // copy each, issued by the 32 lanes of warp 0 (lane l: row group l % 16,
-      // hi for l < 16, lo above)
-      const uint32_t rg_bytes = (uint32_t)jk * 32u;
-      auto load_a = [&](int t) {
-        a_pending = true;
-        if (warp == 0) {
-          if (lane == 0) mbar_expect_tx(bar_a, 32u * rg_bytes);
-          __syncwarp();
-          const int rg = lane & 15, part = lane >> 4;
-          const float* src = Kc + (int64_t)t * 2 * XT_TILE_FLOATS + part * XT_TILE_FLOATS + rg * (XT_KMAX / 4) * 32;
-          float* dst = (part ? Alo : Ahi) + rg * (XT_KMAX / 4) * 32;
-          bulk_g2s(dst, src, rg_bytes, bar_a);
-        }
-      };
+    float best = -1.f, second = -1.f;
+    int bi = -1;
+    // Columns lo .. j-1 of W (of one block of 16) for every candidate, added to
+    // the running sums; this thread's best candidate by the new sums.  False
+    // after a wait ran out.
+    auto score = [&](int lo) -> bool {
+      const int jk = (j + 7) & ~7;                              // K
+      const int nch = (jk + XT_KC - 1) / XT_KC;                 // pieces per tile
       const int ntile = (nc + 127) >> 7;
-      load_a(0);
-      for (int t = 0; t < ntile; ++t) {
-        const int base = t << 7;
-        const int r = base + tid;
-        const bool live = r < nc;
-        // tile t's operand in shared memory, then its MMAs
-        bool got = mbar_wait(bar_a, phase_a);
+      const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(16 >> 3) << 17) |
+                             ((uint32_t)(128 >> 4) << 24);
+      best = -1.f; second = -1.f; bi = -1;
+      for (int g0 = 0; g0 < ntile; g0 += XT_GROUP) {
+        const int gt = min(XT_GROUP, ntile - g0);
+        bool got = true;
+        if (warp == 0) {
+          const int np = gt * nch;
+          auto copy = [&](int m) {
+            // piece m of the group, once the MMAs of its buffer's last piece have
+            // read it
+            const uint32_t b = copied % XT_RING;
+            bool go = true;
+            if (copied >= XT_RING) go = mbar_wait(&freed[b], ((copied - XT_RING) / XT_RING) & 1u);
+            if (!__all_sync(0xffffffffu, go)) return false;
+            const int t = g0 + m / nch, c = m % nch;
+            const uint32_t bytes = (uint32_t)(min(XT_KC, jk - XT_KC * c) / 8) * XT_SLAB;
+            if (lane == 0) {
+              mbar_expect_tx(&full[b], bytes);
+              bulk_g2s(smem + XtSmem::A_OFF + b * XtSmem::A_BYTES,
+                       Kc + (int64_t)t * 2 * XT_TILE_FLOATS + c * (XtSmem::A_BYTES / 4), bytes,
+                       &full[b]);
+            }
+            __syncwarp();
+            ++copied;
+            return true;
+          };
+          // copies run two pieces ahead of the MMAs
+          for (int m = 0; m < 2 && m < np && got; ++m) got = copy(m);
+          for (int m = 0; m < np && got; ++m) {
+            if (m + 2 < np) got = copy(m + 2);
+            const uint32_t b = issued % XT_RING;
+            if (got) got = __all_sync(0xffffffffu, mbar_wait(&full[b], (issued / XT_RING) & 1u));
+            if (!got) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int c = m % nch;
+            const uint32_t d = taddr + (uint32_t)(m / nch) * 16u;
+            const uint64_t a0 = xdesc(smem_u32(smem + XtSmem::A_OFF + b * XtSmem::A_BYTES), 256);
+            const uint64_t b0 = xdesc(smem_u32(Bhi) + (uint32_t)c * (XT_KC / 4) * 128u,
+                                      (XT_KMAX / 4) * 128);
+            const int nks = min(XT_KC, jk - XT_KC * c) / 8;
+            // (addresses below 256 KB: adding to the address field does not carry)
+#pragma unroll
+            for (int ks = 0; ks < XT_KC / 8; ++ks) {
+              if (ks >= nks) break;
+              const uint64_t a_hi = a0 + ks * (XT_SLAB >> 4), a_lo = a_hi + (XT_SLAB >> 5);
+              const uint64_t b_hi = b0 + ks * (256 >> 4), b_lo = b_hi + (XtSmem::B_BYTES >> 4);
+              xmma(d, a_hi, b_hi, idesc, c + ks > 0 ? 1u : 0u);
+              xmma(d, a_hi, b_lo, idesc, 1u);
+              xmma(d, a_lo, b_hi, idesc, 1u);
+            }
+            xcommit(&freed[b]);
+            if (m + 1 == np) xcommit(gdone);
+            ++issued;
+          }
+        }
+        __syncwarp();
+        if (got) got = mbar_wait(gdone, gphase);
         if (!__syncthreads_and(got)) {
           if (tid == 0) atomicOr(P.status, LAGP_DEV_TIMEOUT);
-          ok = false;
-          timed_out = true;
-          break;
+          return false;
         }
-        phase_a ^= 1u;
-        a_pending = false;
-        m_pending = true;
-        if (tid == 0) {
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t ah = smem_u32(Ahi), al = smem_u32(Alo);
-          const uint32_t bh = smem_u32(Bhi), bl = smem_u32(Blo);
-          for (int ks = 0; ks < jk / 8; ++ks) {
-            const uint32_t ko = ks * 256;
-            xmma(taddr, xdesc(ah + ko), xdesc(bh + ko), idesc, ks > 0 ? 1u : 0u);
-            xmma(taddr, xdesc(ah + ko), xdesc(bl + ko), idesc, 1u);
-            xmma(taddr, xdesc(al + ko), xdesc(bh + ko), idesc, 1u);
-          }
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           smem_u32(bar))
-                       : "memory");
-        }
-        bool done = mbar_wait(bar, phase);
-        if (!__syncthreads_and(done)) {
-          if (tid == 0) atomicOr(P.status, LAGP_DEV_TIMEOUT);
-          ok = false;
-          timed_out = true;
-          break;
-        }
-        phase ^= 1u;
-        m_pending = false;
-        // the MMAs have read the A buffer: the next tile's copy overlaps the epilogue
-        if (t + 1 < ntile) load_a(t + 1);
+        gphase ^= 1u;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // epilogue: row tid of W
-        float vs = 0.f, ns = 0.f;
         const uint32_t row = taddr + ((uint32_t)(warp * 32) << 16);
-        for (int c0 = 0; c0 < jn; c0 += 16) {
-          float w[16];
-          xld16(row + c0, w);
-  #pragma unroll
-          for (int u = 0; u < 16; ++u) {
-            const int i = c0 + u;
-            const float wi = i < j ? w[u] : 0.f;
-            vs = fmaf(wi, wi, vs);
-            ns = fmaf(wi, i < j ? zf[i] : 0.f, ns);
+        float vs[XT_GROUP], ns[XT_GROUP];
+#pragma unroll
+        for (int s = 0; s < XT_GROUP; ++s) {
+          const int r = (g0 + s) * 128 + tid;
+          vs[s] = r < nc ? vsum[r] : 0.f;
+          ns[s] = r < nc ? nsum[r] : 0.f;
+        }
+        for (int i = lo; i < j; ++i) {
+          float w[XT_GROUP];
+#pragma unroll
+          for (int s = 0; s < XT_GROUP; ++s) {
+            w[s] = 0.f;
+            if (s < gt) w[s] = xld1(row + (uint32_t)(s * 16 + (i & 15)));
+          }
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          const float zi = zf[i];
+#pragma unroll
+          for (int s = 0; s < XT_GROUP; ++s) {
+            vs[s] = fmaf(w[s], w[s], vs[s]);
+            ns[s] = fmaf(w[s], zi, ns[s]);
           }
         }
-        if (live && !used[r]) {
-          const float v = onepg - vs;
-          const float num = ns - kap[r];
+#pragma unroll
+        for (int s = 0; s < XT_GROUP; ++s) {
+          const int r = (g0 + s) * 128 + tid;
+          if (r >= nc) continue;
+          vsum[r] = vs[s];
+          nsum[r] = ns[s];
+          if (used[r]) continue;
+          const float v = onepg - vs[s];
+          const float num = ns[s] - kap[r];
           const float alc = v > 0.f ? num * num / v : 0.f;
           if (alc > best) { second = best; best = alc; bi = r; }
           else if (alc > second) second = alc;
@@ -433,7 +493,21 @@ __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
       }
-      if (!ok) break;
+      return true;
+    };
+
+    // the starting points; their columns of W a block of 16 at a time (the B
+    // operand holds one block)
+    int scored = 0;
+    for (int rr = 0; rr < P.n0 && ok; ++rr) {
+      ok = add_point(rr);
+      if (ok && ((j & 15) == 0 || j == P.n0) && j < n) {
+        if (!score(scored)) { ok = false; timed_out = true; }
+        scored = j;
+      }
+    }
+
+    for (int step = P.n0; step < n && ok; ++step) {
       // block argmax, ties to the lower rank; the second best for the gap
       for (int o = 16; o > 0; o >>= 1) {
         const float ob = __shfl_xor_sync(0xffffffffu, best, o);
@@ -462,14 +536,18 @@ __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
       __syncthreads();
       const int pick = ired[4];
       ok = (pick >= 0) && add_point(pick);
+      if (ok && j < n) {
+        if (!score(scored)) { ok = false; timed_out = true; }
+        scored = j;
+      }
     }
 
     if (ok) {
       double a = 0.0, b = 0.0, c = 0.0;
-      for (int i = tid; i < j; i += XT_THREADS) {
-        a = fma(z[i], zy[i], a);
-        b = fma(zy[i], zy[i], b);
-        c = fma(z[i], z[i], c);
+      if (tid < j) {
+        a = __dmul_rn(z[tid], zy[tid]);
+        b = __dmul_rn(zy[tid], zy[tid]);
+        c = __dmul_rn(z[tid], z[tid]);
       }
       xsum2_t0(a, b, j, red);
       xsum_t0(c, j, red + 4);
@@ -489,20 +567,23 @@ __global__ void __launch_bounds__(XT_THREADS, 2) exh_tc_kernel(XtParams P) {
       // 1 / sqrt(v); a failed update promotes the location
       double vm = ok ? INFINITY : -1.0;
       for (int i = 0; i < j; ++i) {
-        const double dg = Lg[(int64_t)i * ld + i];
+        const double dg = Lg[xtri(i) + i];
         vm = fmin(vm, 1.0 / (dg * dg));
       }
       promote_location(P.promote, P.promote_count, loc, vm);
     }
   }
-  // after a timeout: wait (bounded) for the copy or MMAs still in flight
-  if (a_pending) mbar_wait(bar_a, phase_a);
-  if (m_pending) mbar_wait(bar, phase);
+  // after a timeout: wait (bounded) for the copies and MMAs still in flight
+  if (timed_out && tid == 0) {
+    for (uint32_t m = issued; m < copied; ++m)
+      mbar_wait(&full[m % XT_RING], (m / XT_RING) & 1u);
+    if (issued > 0) mbar_wait(&freed[(issued - 1) % XT_RING], ((issued - 1) / XT_RING) & 1u);
+  }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(taddr));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(taddr));
   }
 }
 
@@ -516,13 +597,15 @@ cudaError_t launch_exh_tc(const DesignArgs& a, cudaStream_t s) {
   P.cand = a.cand; P.nc_max = a.nc_max; P.nc_loc = a.nc_loc; P.n0 = a.n0; P.n_max = a.n_max;
   P.n_loc = a.n_loc; P.theta = a.theta; P.theta_loc = a.theta_loc; P.g = a.g; P.center = a.ws->center; P.mean = a.mean;
   P.s2 = a.s2; P.selected = a.selected; P.tie_gap = a.tie_gap; P.nevals = a.nevals;
-  P.Linv = a.ws->state64; P.Kc = a.ws->state32; P.status = a.ws->status;
+  P.Kc = a.ws->state32; P.status = a.ws->status;
   P.queue = a.ws->queue + 1; P.order = a.order; P.count = a.count;
   P.crow = a.ws->crow;
   P.promote = a.promote ? a.ws->promote : nullptr;
   P.promote_count = a.ws->status + 1;
-  const size_t small = (size_t)((a.nc_max + 3) & ~3) * 4 + XT_KMAX * 4 + (size_t)XT_KMAX * a.p * 8 +
-                       6 * XT_KMAX * 8 + 8 * 8 + 8 * 4 + 8 * 4 + XT_KMAX * 4 + a.nc_max + 96;
+  const int ld = a.n_max < XT_KMAX ? a.n_max : XT_KMAX;
+  const size_t small = 3 * (size_t)((a.nc_max + 3) & ~3) * 4 + XT_KMAX * 4 +
+                       (size_t)XT_KMAX * a.p * 8 + 6 * XT_KMAX * 8 + 8 * 8 + (size_t)xtri(ld) * 8 +
+                       8 * 4 + 8 * 4 + XT_KMAX * 4 + a.nc_max + 16 + (2 * XT_RING + 1) * 8 + 16;
   const size_t sm = 1024 + XtSmem::END + small;
   cudaError_t err =
       cudaFuncSetAttribute(exh_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);

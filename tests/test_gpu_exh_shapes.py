@@ -1,13 +1,14 @@
-"""The FP32 exhaustive scorers at the edges of their layouts, against the
-oracle: design sizes around four rows, the shared-memory factor's limit (64
-points) and the tensor-core form's blocks of 16 rows (also with more starting
-points than one block), and candidate counts that are no multiple of four or
-of a 128-candidate tile."""
+"""The FP32 exhaustive scorers at the edges of their layouts: design sizes
+around four rows, the shared-memory factor's limit (64 points) and the
+tensor-core form's blocks of 16 rows (also with more starting points than one
+block), and candidate counts that are no multiple of four or of a 128-candidate
+tile."""
+import numpy as np
 import pytest
 
-from gpu_helpers import check_fp32_form
+from gpu_helpers import check_fp32_form, to_dev
 from paper_1409_0074_gb300 import workloads as W
-from test_gpu_parity import gpu_run, oracle_run
+from test_gpu_parity import gpu_run, oracle_run, same_rows
 
 pytestmark = pytest.mark.gpu
 
@@ -25,9 +26,20 @@ def lagp(cuda):
 @pytest.mark.parametrize("n0,n,nc", [(3, 4, 5), (3, 17, 129), (16, 33, 131), (17, 34, 1001),
                                      (33, 64, 257), (6, 65, 1150)])
 def test_fp32_exhaustive_shapes(lagp, precision, n0, n, nc):
-    """With a nugget of 1e-2 the pivots are at least 1e-2, so the FP32 error of
-    a few 1e-7 in a score's denominator moves scores by less than 1e-4: designs
-    may leave the oracle's only at gaps below 1e-3."""
+    """The binary64 update and prediction on the form's own designs, s2 where
+    the designs are the oracle's, and the same bits from a call whose largest
+    n and N' are above every location's (other strides and tiles, and for n
+    <= 64 the factor in global instead of shared memory)."""
     w = W.small(N=4000, p=3, M=20, n0=n0, n=n, nc=nc, theta=0.3, g=1e-2, seed=n + nc)
-    check_fp32_form(w, gpu_run(lagp, w, "exhaustive", precision), oracle_run(w, "exhaustive"),
-                    rmse_tol=None, max_gap=1e-3)
+    g = gpu_run(lagp, w, "exhaustive", precision)
+    check_fp32_form(w, g, oracle_run(w, "exhaustive"), rmse_tol=None, max_gap=None)
+    import torch
+    big = lagp.predict(to_dev(w.X), to_dev(w.Y), to_dev(w.Xref), n0, min(n + 67, 128), nc + 141, w.theta,
+                       w.g, search="exhaustive", precision=precision, want_trace=True,
+                       n_loc=to_dev(np.full(w.M, n, np.int32), torch.int32),
+                       nclose_loc=to_dev(np.full(w.M, nc, np.int32), torch.int32))
+    b = {k: v.cpu().numpy() for k, v in big.items()}
+    b["selected"] = b["selected"][:, :n]
+    if precision == "fp32_tc" and n > 64:
+        return                  # both calls take the CUDA-core scorer: covered by "fp32"
+    assert same_rows(g, b).all()
