@@ -2,12 +2,20 @@
 //
 // Level L (0 .. D-1) orders the positions of every level-L node by the
 // node's split coordinate L mod p: one stable least-significant-digit radix
-// sort of the keys (node << 32 | coordinate bits), 8 bits a pass, over all
-// positions.  Sorting by node as the high digits keeps every node's points in
-// its own range, so after the last level each node's children are the lower
-// and upper halves of its range.  Ties in a coordinate keep the previous
-// order, so the tree is deterministic.  Then the tree-ordered FP32 rows are
-// gathered and the node boxes are formed from the leaves upwards.
+// sort of the keys (node << 24 | coordinate in units of 2^-24 of the design's
+// box), 8 bits a pass, over all positions.  Sorting by node as the high digits
+// keeps every node's points in its own range, so after the last level each
+// node's children are the lower and upper halves of its range.  Ties in a key
+// keep the previous order, so the tree is deterministic; a query is exact for
+// any order, since every node keeps the exact box of its points (and 2^-24 of the
+// box is what the FP32 rows resolve away from its centre).  Then the tree-ordered
+// FP32 rows are gathered and the node boxes are formed from the leaves upwards.
+//
+// A pass (tile histograms, their scan, a stable scatter by one warp per tile) is
+// bound by the scatter's chain of dependent steps, so tiles are small (1,024
+// keys: about six warps per SM at N = 1e6), the next keys are loaded ahead, and
+// the scan takes a block per digit.  N = 1e6, p = 8: 2.75 ms; with tiles of 4,096,
+// 32-bit coordinates (a pass more per level) and one block for the scan, 10.6 ms.
 #include <cstdint>
 
 #include "kdtree.cuh"
@@ -15,7 +23,7 @@
 
 namespace lagp {
 
-#define RS_TILE 4096
+#define RS_TILE 1024
 
 static int rs_blocks(int64_t N) { return (int)((N + RS_TILE - 1) / RS_TILE); }
 
@@ -26,7 +34,7 @@ size_t kd_bytes(int64_t N, int p, int PP) {
   return al256(sizeof(int32_t) * N) + al256(sizeof(float) * N * PP) +
          al256(sizeof(float) * nodes * 2 * PP) + al256(sizeof(double) * nodes * 2 * p) +
          al256(sizeof(uint64_t) * 2 * N) + al256(sizeof(int32_t) * N) +
-         al256(sizeof(uint32_t) * 256 * (size_t)rs_blocks(N));
+         al256(sizeof(uint32_t) * 256 * ((size_t)rs_blocks(N) + 1));
 }
 
 void kd_carve(int64_t N, int p, int PP, char* base, KdTree* t) {
@@ -41,14 +49,18 @@ void kd_carve(int64_t N, int p, int PP, char* base, KdTree* t) {
   t->box64 = reinterpret_cast<double*>(take(sizeof(double) * nodes * 2 * p));
   t->keys = reinterpret_cast<uint64_t*>(take(sizeof(uint64_t) * 2 * N));
   t->vals = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * N));
-  t->hist = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * (size_t)rs_blocks(N)));
+  t->hist = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * ((size_t)rs_blocks(N) + 1)));
 }
 
 // keys of level `level`: the position's node (relative index within the level)
-// in the high word, the order-preserving bits of coordinate `dim` below
+// above 24 bits of coordinate `dim` (centred on the design's box, so within
+// half its extent of zero)
 __global__ void kd_keys(const int32_t* __restrict__ perm, const float* __restrict__ Xf, int64_t N,
-                        int PP, int level, int dim, int first, uint64_t* __restrict__ keys,
+                        int PP, int level, int dim, int first, const double* __restrict__ lo_box,
+                        const double* __restrict__ hi_box, uint64_t* __restrict__ keys,
                         int32_t* __restrict__ vals) {
+  const float ext = (float)(hi_box[dim] - lo_box[dim]);
+  const float unit = ext > 0.f ? 16777215.f / ext : 0.f, mid = 0.5f * ext;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t gi = first ? (int32_t)i : perm[i];
@@ -59,9 +71,8 @@ __global__ void kd_keys(const int32_t* __restrict__ perm, const float* __restric
       if (i < m) { hi = m; node = node << 1; }
       else { lo = m; node = (node << 1) | 1u; }
     }
-    uint32_t u = __float_as_uint(Xf[(int64_t)gi * PP + dim]);
-    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-    keys[i] = ((uint64_t)node << 32) | u;
+    const float u = (Xf[(int64_t)gi * PP + dim] + mid) * unit;
+    keys[i] = ((uint64_t)node << 24) | (uint32_t)fminf(fmaxf(u, 0.f), 16777215.f);
     vals[i] = gi;
   }
 }
@@ -80,52 +91,74 @@ __global__ void rs_hist(const uint64_t* __restrict__ keys, int64_t N, int shift,
   hist[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = cnt[threadIdx.x];
 }
 
-// exclusive prefix sum of hist[0 .. total) in place (one block of 1024 threads)
-__global__ void rs_scan(uint32_t* __restrict__ hist, int64_t total) {
-  __shared__ uint32_t part[1024];
-  const int t = threadIdx.x;
-  const int64_t per = (total + 1023) / 1024;
-  const int64_t a = t * per, b = a + per < total ? a + per : total;
-  uint32_t s = 0;
-  for (int64_t i = a; i < b; ++i) s += hist[i];
-  part[t] = s;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {     // inclusive scan of the partial sums
-    const uint32_t v = t >= o ? part[t - o] : 0u;
+// exclusive prefix sums of each digit's row of tile counts, in place, and the
+// row's total into total[digit] (one block of 256 threads per digit)
+__global__ void rs_scan(uint32_t* __restrict__ hist, int nblk, uint32_t* __restrict__ total) {
+  __shared__ uint32_t wsum[8];
+  uint32_t* row = hist + (int64_t)blockIdx.x * nblk;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  uint32_t run = 0;
+  for (int c0 = 0; c0 < nblk; c0 += 256) {
+    const uint32_t v = c0 + t < nblk ? row[c0 + t] : 0u;
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) wsum[warp] = incl;
     __syncthreads();
-    part[t] += v;
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+      before += w < warp ? wsum[w] : 0u;
+      all += wsum[w];
+    }
+    if (c0 + t < nblk) row[c0 + t] = run + before + incl - v;
+    run += all;
     __syncthreads();
   }
-  uint32_t run = t > 0 ? part[t - 1] : 0u;
-  for (int64_t i = a; i < b; ++i) {
-    const uint32_t c = hist[i];
-    hist[i] = run;
-    run += c;
-  }
+  if (t == 0) total[blockIdx.x] = run;
 }
 
 // stable scatter of one tile by one warp, 32 keys at a time in order
 __global__ void rs_scatter(const uint64_t* __restrict__ kin, const int32_t* __restrict__ vin,
                            uint64_t* __restrict__ kout, int32_t* __restrict__ vout, int64_t N,
-                           int shift, const uint32_t* __restrict__ hist) {
+                           int shift, const uint32_t* __restrict__ hist,
+                           const uint32_t* __restrict__ total) {
   __shared__ uint32_t base[256];
   const int lane = threadIdx.x;
-  for (int d = lane; d < 256; d += 32) base[d] = hist[(int64_t)d * gridDim.x + blockIdx.x];
+  // where each digit starts: the digits' totals before it, then the tiles before
+  uint32_t start = 0;
+  for (int d0 = 0; d0 < 256; d0 += 32) {
+    const uint32_t v = total[d0 + lane];
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    base[d0 + lane] = start + incl - v + hist[(int64_t)(d0 + lane) * gridDim.x + blockIdx.x];
+    start += __shfl_sync(0xffffffffu, incl, 31);
+  }
   __syncwarp();
   const int64_t t0 = (int64_t)blockIdx.x * RS_TILE;
   const int64_t t1 = t0 + RS_TILE < N ? t0 + RS_TILE : N;
+  uint64_t kn = t0 + lane < t1 ? kin[t0 + lane] : 0;
+  int32_t vn = t0 + lane < t1 ? vin[t0 + lane] : 0;
   for (int64_t c0 = t0; c0 < t1; c0 += 32) {
-    const int64_t i = c0 + lane;
-    const bool valid = i < t1;
+    const uint64_t k = kn;
+    const int32_t v = vn;
+    const bool valid = c0 + lane < t1;
+    if (c0 + 32 + lane < t1) { kn = kin[c0 + 32 + lane]; vn = vin[c0 + 32 + lane]; }
     const unsigned act = __ballot_sync(0xffffffffu, valid);
     if (valid) {
-      const uint64_t k = kin[i];
       const uint32_t dig = (uint32_t)(k >> shift) & 255u;
       const unsigned peers = __match_any_sync(act, dig);
       const unsigned below = peers & ((1u << lane) - 1u);
       const uint32_t pos = base[dig] + (uint32_t)__popc(below);
       kout[pos] = k;
-      vout[pos] = vin[i];
+      vout[pos] = v;
       __syncwarp(act);
       if (below == 0u) base[dig] += (uint32_t)__popc(peers);   // the group's first lane
     }
@@ -203,26 +236,28 @@ __global__ void kd_up(int level, int p, int PP, float* __restrict__ box32,
   }
 }
 
-cudaError_t launch_kd_build(const double* X, const float* Xf, int64_t N, int p, int PP,
-                            const KdTree& t, cudaStream_t s) {
+cudaError_t launch_kd_build(const double* X, const float* Xf, const double* lo, const double* hi,
+                            int64_t N, int p, int PP, const KdTree& t, cudaStream_t s) {
   const int D = t.D;
   if ((D + KD_FAN - 1) / KD_FAN * 32 > KD_STACK) return cudaErrorInvalidValue;
   const int nblk = rs_blocks(N);
   const unsigned g = (unsigned)((N + 255) / 256 < 4096 ? (N + 255) / 256 : 4096);
   prof_begin("kd_build", s);
   uint64_t* kb[2] = {t.keys, t.keys + N};
+  uint32_t* total = t.hist + 256 * (size_t)nblk;     // [256] digit totals of a pass
   for (int level = 0; level < D; ++level) {
     // keys into buffer 0 (values: the current order, identity at level 0)
-    kd_keys<<<g, 256, 0, s>>>(t.perm, Xf, N, PP, level, level % p, level == 0, kb[0], t.vals);
+    kd_keys<<<g, 256, 0, s>>>(t.perm, Xf, N, PP, level, level % p, level == 0, lo, hi, kb[0],
+                              t.vals);
     int cur = 0;                 // keys in kb[cur]; values in t.vals for cur = 0 at start
     int32_t* vcur = t.vals;
     int32_t* valt = t.perm;
-    const int passes = 4 + (level + 7) / 8;
+    const int passes = 3 + (level + 7) / 8;
     for (int ps = 0; ps < passes; ++ps) {
       const int shift = 8 * ps;
       rs_hist<<<nblk, 256, 0, s>>>(kb[cur], N, shift, t.hist);
-      rs_scan<<<1, 1024, 0, s>>>(t.hist, (int64_t)256 * nblk);
-      rs_scatter<<<nblk, 32, 0, s>>>(kb[cur], vcur, kb[cur ^ 1], valt, N, shift, t.hist);
+      rs_scan<<<256, 256, 0, s>>>(t.hist, nblk, total);
+      rs_scatter<<<nblk, 32, 0, s>>>(kb[cur], vcur, kb[cur ^ 1], valt, N, shift, t.hist, total);
       cur ^= 1;
       int32_t* tmp = vcur;
       vcur = valt;
@@ -230,7 +265,7 @@ cudaError_t launch_kd_build(const double* X, const float* Xf, int64_t N, int p, 
     }
     if (vcur != t.perm) kd_copy<<<g, 256, 0, s>>>(vcur, t.perm, N);
   }
-  if (D == 0) kd_keys<<<g, 256, 0, s>>>(t.perm, Xf, N, PP, 0, 0, 1, kb[0], t.perm);
+  if (D == 0) kd_keys<<<g, 256, 0, s>>>(t.perm, Xf, N, PP, 0, 0, 1, lo, hi, kb[0], t.perm);
   kd_gather<<<g, 256, 0, s>>>(t.perm, Xf, N, PP, t.pts32);
   const int64_t nleaf = (int64_t)1 << D;
   kd_leaf_box<<<(unsigned)((nleaf * 32 + 255) / 256), 256, 0, s>>>(t.perm, t.pts32, X, N, p, PP,

@@ -237,12 +237,13 @@ struct KdTree {
   double* box64;     // [nodes][2][p]
   uint64_t* keys;    // [2][N] sort scratch
   int32_t* vals;     // [N] sort scratch
-  uint32_t* hist;    // [256][blocks] sort scratch
+  uint32_t* hist;    // [256][blocks] sort scratch, then [256] totals
 };
 
 size_t kd_bytes(int64_t N, int p, int PP);
 void kd_carve(int64_t N, int p, int PP, char* base, KdTree* t);
-cudaError_t launch_kd_build(const double* X, const float* Xf, int64_t N, int p, int PP,
-                            const KdTree& t, cudaStream_t s);
+// (lo, hi: the design's bounding box, the origin of Xf its centre)
+cudaError_t launch_kd_build(const double* X, const float* Xf, const double* lo, const double* hi,
+                            int64_t N, int p, int PP, const KdTree& t, cudaStream_t s);
 
 }  // namespace lagp
