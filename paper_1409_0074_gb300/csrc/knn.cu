@@ -16,7 +16,7 @@
 // least N' points have d32 <= tau, so the N'-th smallest d64 is at most
 // tau + err, and any member has d32 <= d64 + err <= tau + 2 err.
 //
-// Pilot threshold (N >= 32 N').  Before the stream, knn_pilot estimates each
+// Pilot threshold (knn_has_pilot).  Before the stream, knn_pilot estimates each
 // location's N'-th distance from a stride sample of S = min(32768, N / 16)
 // design points: with
 // lambda = S N'/N sample points expected inside it, the m-th smallest sample
@@ -28,6 +28,7 @@
 // too, and every point that could belong was admitted); a location that fails
 // the check is streamed again with tau = infinity.
 #include <cfloat>
+#include <cmath>
 #include <cstdint>
 
 #include "common.cuh"
@@ -630,15 +631,40 @@ size_t knn_smem_stream(int PP) {
   return (size_t)2 * LAGP_KNN_TILE * PP * 4 + 2 * LAGP_KNN_TILE * 4 + KNN_WARPS * 256 * 4 + 16;
 }
 
+// Pilot thresholds pay where the design is large against N' and there is work
+// enough for the pilot's own 30 us.  Streams without and with them (pilot and
+// redo included): 5,000 locations at p = 8, N = 2 N' (4000) 321 us against 313,
+// N = 4 N' (4000) 567 against 240, N = 8 N' (1024) 128 against 104; at p = 4, 8
+// locations, N = 8 N': 60 against 69 us at 1024, 80 against 83 at 2000, 142
+// against 107 at 4000; one location, N = 16 N': 92 against 97 us at 8000, 169
+// against 150 at 16000.
+static int64_t knn_sample(int64_t N) { return N / 16 < 32768 ? N / 16 : 32768; }
+static bool knn_uses_tc(int64_t N, int nc_max) { return N >= (int64_t)32 * nc_max; }
+static bool knn_mid(int64_t N, int nc_max) { return N >= (int64_t)4 * nc_max && N >= 1024; }
+static bool knn_has_pilot(int64_t N, int64_t M, int nc_max) {
+  return knn_uses_tc(N, nc_max) || (knn_mid(N, nc_max) && M * N >= 16384);
+}
+
 // Buffer entries per location: room for N' survivors, a whole tile of new
 // inserts before the next compaction, and N'/2 (at least 64) entries of slack
-// for distances within the error margin of the N'-th.  A power of two, as the
+// for distances within the error margin of the N'-th; with a pilot threshold
+// also for the points that it is expected to admit and the two tiles that the
+// pilot asks for beside them.  Without that room, as for N' <= 307 at N = 1e6, the
+// pilot gives no threshold and every location streams the whole design from
+// infinity: 5.2 ms for one location and 9.5 ms for 10,000 at N' = 250, p = 4,
+// where the tensor-core filter takes 0.035 and 4.0 ms.  A power of two, as the
 // bitonic sort of knn_rank wants.
-int knn_cap(int nc_max) {
-  // with the pilot threshold about 2.2 N' points are admitted
+int knn_cap(int nc_max, int64_t N) {
   const int need = (5 * nc_max) / 2 + LAGP_KNN_TILE;
   int cap = 512;
   while (cap < need) cap <<= 1;
+  if (knn_uses_tc(N, nc_max) || knn_mid(N, nc_max)) {
+    const double ratio = (double)N / (double)knn_sample(N), lam = nc_max / ratio;
+    const double admits = (lam + 4.5 * sqrt(lam) + 6.0) * ratio;
+    int more = cap;
+    while (more < 16384 && admits > more - 2 * LAGP_KNN_TILE) more <<= 1;
+    if (admits <= more - 2 * LAGP_KNN_TILE) cap = more;
+  }
   return cap;
 }
 
@@ -665,14 +691,13 @@ cudaError_t launch_prepare(const double* X, int64_t N, int p, int PP, int64_t Np
 cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
                        const double* xref, int64_t M, int nc_max, const int32_t* nc_loc,
                        int32_t* cand, const Workspace& ws, cudaStream_t s) {
-  const int cap = knn_cap(nc_max);
+  const int cap = knn_cap(nc_max, N);
   const int64_t ntiles = Npad / LAGP_KNN_TILE;
   const int qpb = KNN_WARPS * KNN_QW;
   dim3 grid((unsigned)((M + qpb - 1) / qpb));
   size_t sm = knn_smem_stream(PP);
-  // pilot thresholds where the design is large against N'
-  const bool pilot = N >= (int64_t)32 * nc_max;
-  const int64_t S = N / 16 < 32768 ? N / 16 : 32768;
+  const bool tc = knn_uses_tc(N, nc_max), pilot = knn_has_pilot(N, M, nc_max);
+  const int64_t S = knn_sample(N);
   KnnEntry* kbuf = reinterpret_cast<KnnEntry*>(ws.knn_buf);
   // a batch of a few locations per SM: one pilot block each (per wave of two
   // blocks per SM about 0.025 ms, 0.05 at S = 32768; the shared form takes its
@@ -697,7 +722,7 @@ cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
                                                      ws.knn_thr);                            \
       prof_end(s);                                                                           \
     }                                                                                        \
-    if (pilot) {                                                                             \
+    if (tc) {                                                                                \
       err = launch_knn_tc(Npad, p, xref, M, nc_max, nc_loc, cap, ws, s);                     \
       if (err != cudaSuccess) return err;                                                    \
     } else {                                                                                 \
@@ -705,7 +730,7 @@ cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
       knn_stream<V><<<grid, KNN_WARPS * 32, sm, s>>>(ws.Xf, ws.nx, N, ntiles, p, xref, M,    \
                                                      ws.center, ws.maxn2, nc_max, nc_loc,    \
                                                      cap, kbuf, ws.knn_cnt, ws.status,       \
-                                                     nullptr, 0);                            \
+                                                     pilot ? ws.knn_thr : nullptr, 0);       \
       prof_end(s);                                                                           \
     }                                                                                        \
     if (pilot) {                                                                             \

@@ -15,7 +15,7 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 static int64_t chunk_for(int64_t M, int search, int precision, int nc_max, int64_t N) {
   int64_t cap = 131072;
   if (search == LAGP_EXHAUSTIVE && precision == LAGP_FP64) cap = 16384;
-  const int64_t per_loc = (int64_t)8 * knn_cap(nc_max);
+  const int64_t per_loc = (int64_t)8 * knn_cap(nc_max, N);
   const int64_t by_mem = ((int64_t)16 << 30) / per_loc;
   if (by_mem < cap) cap = by_mem > 128 ? by_mem : 128;
   return M < cap ? (M > 0 ? M : 1) : cap;
@@ -41,7 +41,7 @@ size_t layout_request(const Shape& sh, void* base, Workspace* ws) {
   Carver c{static_cast<char*>(base), 0};
   w->status = static_cast<unsigned*>(c.take(4 * sizeof(unsigned)));
   const int64_t ch = sh.chunk;
-  w->knn_buf = c.take((size_t)8 * ch * knn_cap(sh.nc_max));
+  w->knn_buf = c.take((size_t)8 * ch * knn_cap(sh.nc_max, sh.N));
   w->knn_cnt = static_cast<int32_t*>(c.take(sizeof(int32_t) * ch));
   w->knn_thr = static_cast<float*>(c.take(sizeof(float) * ch));
   w->knn_seg = static_cast<int32_t*>(c.take(sizeof(int32_t) * 4 * ch));

@@ -120,7 +120,7 @@ size_t layout_workspace(const Shape& sh, void* base, Workspace* ws);
 size_t layout_request(const Shape& sh, void* base, Workspace* ws);
 size_t layout_design(const Shape& sh, void* base, Workspace* ws);
 
-int knn_cap(int nc_max);
+int knn_cap(int nc_max, int64_t N);
 size_t knn_smem_stream(int PP);
 
 cudaError_t launch_prepare(const double* X, int64_t N, int p, int PP, int64_t Npad,
