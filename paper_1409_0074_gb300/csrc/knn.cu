@@ -9,9 +9,9 @@
 //     buffer when d32 <= tau + 2 err, where tau is the N'-th smallest buffered
 //     d32 and err a proven bound on |d32 - d64|.  A warp radix-selects tau and
 //     compacts the buffer whenever the next tile might overflow it.
-//  2. knn_rank: one CTA per location computes the exact binary64 distances of
-//     the surviving points in the oracle's operation order and bitonic-sorts
-//     (d64, index) pairs; the first N' indices are the candidate list.
+//  2. knn_rank: one CTA per location puts the surviving points in the order of
+//     (d64, index), d64 the binary64 distance in the oracle's operation order;
+//     the first N' indices are the candidate list.
 // Every true member of the N'-nearest set survives stage 1: at the end at
 // least N' points have d32 <= tau, so the N'-th smallest d64 is at most
 // tau + err, and any member has d32 <= d64 + err <= tau + 2 err.
@@ -476,82 +476,212 @@ knn_stream(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N
 }
 
 // ---------------------------------------------------------------------------
-// Exact ranking: binary64 distances in the oracle's order, bitonic sort of
-// (d64, index), first N' indices out.  Distances are non-negative, so their
-// IEEE bit patterns order like the values: the sort compares 64-bit integers
-// (FP64 compares would run on GB300's narrow FP64 pipe).  Up to 1024 pairs
-// are sorted in registers, four per thread (element 4 t + u on thread t):
-// strides 1 and 2 inside a thread, 4 to 64 between the lanes of a warp by
-// shuffles, 128 to 512 through shared memory.  Larger sets take the same
-// network entirely in shared memory.  The real pairs are distinct (distinct
-// indices), so either way the order is the unique sorted one.
+// Exact ranking: the candidates in the order of (binary64 distance in the
+// oracle's order of operations, index), the first N' of them out.
+//
+// The binary64 distances of every survivor were most of this kernel (24 FP64
+// instructions a pair at p = 8, on GB300's narrow FP64 pipe), and few of them
+// decide anything: the order of two points is known from binary32 distances
+// unless these lie within their error bounds.  So the pairs (binary32 distance,
+// index) are sorted as one 64-bit word each, neighbours closer than their bounds
+// are joined into runs, and only the members of runs (a few per cent) get
+// their binary64 distance and are ranked within their run by counting.  The
+// bound grows with the distance, so the cut between two runs separates
+// everything below from everything above.  Runs longer than RANK_RUN (designs
+// with many equal distances) and values that leave binary32's range sort all the
+// (binary64 distance, index) pairs instead; both give the one order.  100,000
+// locations, p = 8, N' = 1000: 3.33 ms, 6.12 with all distances in binary64;
+// 10,000 locations, p = 4, N' = 200: 0.06 against 0.42 ms (a network of 1024
+// whatever the list's length).
+//
+// Sorts are bitonic.  Up to 2048 pairs are held in registers, E per thread
+// (element E t + u on thread t): strides below E inside a thread, then between
+// the lanes of a warp by shuffles, the largest through shared memory.  Distances
+// are non-negative, so their IEEE bit patterns order like the values.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool kv_less(unsigned long long ka, int32_t ia, unsigned long long kb,
-                                        int32_t ib) {
-  return ka < kb || (ka == kb && ia < ib);
-}
+#define RANK_THREADS 256
+#define RANK_RUN 64
+#define RANK_MAX (8 * RANK_THREADS)
 
-// Sorts the 1024 pairs in kr/ir (four per thread) and leaves them in order in
-// key/idx[0..1024), which must hold 1024 entries; blockDim.x == 256.
-__device__ __forceinline__ void rank_sort1024(unsigned long long* kr, int32_t* ir,
-                                              unsigned long long* key, int32_t* idx) {
+// Sorts the RANK_THREADS * E words (WIDE: pairs of a word and an index) in kr
+// (and ir); key and idx: shared memory for as many entries.
+template <int E, bool WIDE>
+__device__ __forceinline__ void rank_sort(unsigned long long (&kr)[E], int32_t (&ir)[E],
+                                          unsigned long long* key, int32_t* idx) {
   const int t = threadIdx.x;
-  for (int k = 2; k <= 1024; k <<= 1) {
-    for (int jj = k >> 1; jj > 0; jj >>= 1) {
-      if (jj >= 4) {
-        const int pt = t ^ (jj >> 2);   // the partner thread, same u
-        unsigned long long pk[4];
-        int32_t pi[4];
-        if (jj >= 128) {                 // another warp: through shared memory
-          __syncthreads();
+  auto less = [](unsigned long long ka, int32_t ia, unsigned long long kb, int32_t ib) {
+    return WIDE ? (ka < kb || (ka == kb && ia < ib)) : ka < kb;
+  };
+#pragma unroll 1
+  for (int k = 2; k <= RANK_THREADS * E; k <<= 1) {
+#pragma unroll 1
+    for (int jj = k >> 1; jj >= E; jj >>= 1) {
+      const int x = jj / E, pt = t ^ x;    // the partner thread, same u
+      if (x >= 32) {                       // another warp: through shared memory
+        __syncthreads();
 #pragma unroll
-          for (int u = 0; u < 4; ++u) { key[4 * t + u] = kr[u]; idx[4 * t + u] = ir[u]; }
-          __syncthreads();
-#pragma unroll
-          for (int u = 0; u < 4; ++u) { pk[u] = key[4 * pt + u]; pi[u] = idx[4 * pt + u]; }
-        } else {
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            pk[u] = __shfl_xor_sync(0xffffffffu, kr[u], jj >> 2);
-            pi[u] = __shfl_xor_sync(0xffffffffu, ir[u], jj >> 2);
-          }
+        for (int u = 0; u < E; ++u) {
+          key[u * RANK_THREADS + t] = kr[u];
+          if (WIDE) idx[u * RANK_THREADS + t] = ir[u];
         }
+        __syncthreads();
+      }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = 4 * t + u;
-          // the lower element of an ascending pair (or the upper of a
-          // descending one) keeps the smaller
-          const bool keep_min = ((i & jj) == 0) == ((i & k) == 0);
-          const bool p_less = kv_less(pk[u], pi[u], kr[u], ir[u]);
-          if (keep_min ? p_less : !p_less) { kr[u] = pk[u]; ir[u] = pi[u]; }
-        }
-      } else {
-        // pairs (u, u + jj) inside the thread, with constant register indices
-        auto ce = [&](unsigned long long& ka, int32_t& ia, unsigned long long& kb, int32_t& ib,
-                      int u) {
-          const bool up = ((4 * t + u) & k) == 0;
-          if (kv_less(kb, ib, ka, ia) == up) {
-            const unsigned long long tk = ka; ka = kb; kb = tk;
-            const int32_t ti = ia; ia = ib; ib = ti;
-          }
-        };
-        if (jj == 2) {
-          ce(kr[0], ir[0], kr[2], ir[2], 0);
-          ce(kr[1], ir[1], kr[3], ir[3], 1);
+      for (int u = 0; u < E; ++u) {
+        const int i = E * t + u;
+        // the lower element of an ascending pair (or the upper of a descending
+        // one) keeps the smaller
+        const bool keep_min = ((i & jj) == 0) == ((i & k) == 0);
+        unsigned long long pk;
+        int32_t pi = 0;
+        if (x >= 32) {
+          pk = key[u * RANK_THREADS + pt];
+          if (WIDE) pi = idx[u * RANK_THREADS + pt];
         } else {
-          ce(kr[0], ir[0], kr[1], ir[1], 0);
-          ce(kr[2], ir[2], kr[3], ir[3], 2);
+          pk = __shfl_xor_sync(0xffffffffu, kr[u], x);
+          if (WIDE) pi = __shfl_xor_sync(0xffffffffu, ir[u], x);
+        }
+        if (less(pk, pi, kr[u], ir[u]) == keep_min) { kr[u] = pk; ir[u] = pi; }
+      }
+    }
+#pragma unroll
+    for (int J = E / 2; J > 0; J >>= 1) {  // inside the thread, constant registers
+      if (J < k) {
+#pragma unroll
+        for (int u = 0; u < E; ++u) {
+          if (u & J) continue;
+          const bool up = ((E * t + u) & k) == 0;
+          if (less(kr[u | J], ir[u | J], kr[u], ir[u]) == up) {
+            const unsigned long long tk = kr[u]; kr[u] = kr[u | J]; kr[u | J] = tk;
+            const int32_t ti = ir[u]; ir[u] = ir[u | J]; ir[u | J] = ti;
+          }
         }
       }
     }
   }
   __syncthreads();
-#pragma unroll
-  for (int u = 0; u < 4; ++u) { key[4 * t + u] = kr[u]; idx[4 * t + u] = ir[u]; }
-  __syncthreads();
 }
-__global__ void __launch_bounds__(256)
-knn_rank(const double* __restrict__ X, int p, const double* __restrict__ xref, int64_t M,
+
+// Bound on |d - D| for D the exact squared distance and d the binary32 one from
+// coordinates rounded to binary32 about the centre (relative error u = 2^-24
+// each, so at most u (|a| + |q|) on the difference, with |a| <= |q| + sqrt(d)):
+// 2 u sqrt(d) (2|q| + sqrt(d)) from the rounded inputs, (p + 4) u d from the
+// arithmetic, both with 25%, the square of the input error, and what
+// underflow can lose.  The binary64 distance's own error is far below the 25%.
+__device__ __forceinline__ float rank_err(float d, float qn, int p) {
+  const float u = 0x1p-24f, r = sqrtf(d), s = 2.f * qn + r;
+  return 1.25f * u * (2.f * r * s + (float)(p + 4) * d) + 4.f * (u * s) * (u * s) + 1e-36f;
+}
+
+struct RankRuns {
+  uint32_t joined[RANK_MAX / 32];   // bit i: element i joins i - 1
+  uint16_t list[RANK_MAX];          // the members of runs
+  int nlist;
+};
+
+// c <= RANK_THREADS * E survivors, at least nc of them
+template <int E>
+__device__ void rank_location(const double* __restrict__ X, const float* __restrict__ Xf, int p,
+                              int PP, const double* xq, const float* qf, float qn,
+                              const KnnEntry* __restrict__ e, int c, int nc,
+                              unsigned long long* key, int32_t* idx, RankRuns& runs,
+                              int32_t* __restrict__ out) {
+  uint32_t* joined = runs.joined;
+  uint16_t* list = runs.list;
+  const int t = threadIdx.x;
+  unsigned long long kr[E];
+  int32_t ir[E];
+  bool wide = false;
+#pragma unroll
+  for (int u = 0; u < E; ++u) {
+    const int i = E * t + u;
+    kr[u] = ~0ull;
+    ir[u] = 0;
+    if (i < c) {
+      const int32_t gi = e[i].idx;
+      const float4* x = reinterpret_cast<const float4*>(Xf + (int64_t)gi * PP);
+      float d = 0.f;
+      for (int k = 0; k < PP / 4; ++k) {
+        const float4 v = __ldg(x + k);
+        const float a = v.x - qf[4 * k], b = v.y - qf[4 * k + 1];
+        const float g = v.z - qf[4 * k + 2], h = v.w - qf[4 * k + 3];
+        d = fmaf(a, a, d);
+        d = fmaf(b, b, d);
+        d = fmaf(g, g, d);
+        d = fmaf(h, h, d);
+      }
+      wide |= !(d < 1e36f);
+      kr[u] = ((unsigned long long)__float_as_uint(d) << 32) | (uint32_t)gi;
+    }
+  }
+  if (t < RANK_THREADS * E / 32) joined[t] = 0u;
+  if (t == 0) runs.nlist = 0;
+  if (!__syncthreads_or(wide || !(qn < 1e18f))) {
+    rank_sort<E, false>(kr, ir, key, idx);
+#pragma unroll
+    for (int u = 0; u < E; ++u) {
+      key[E * t + u] = kr[u];
+      idx[E * t + u] = (int32_t)(uint32_t)kr[u];
+    }
+    __syncthreads();
+    uint32_t bits = 0u;
+    float before = t > 0 ? __uint_as_float((uint32_t)(key[E * t - 1] >> 32)) : 0.f;
+#pragma unroll
+    for (int u = 0; u < E; ++u) {
+      const int i = E * t + u;
+      const float d = __uint_as_float((uint32_t)(kr[u] >> 32));
+      if (i > 0 && i < c && d - before <= 2.002f * rank_err(d, qn, p)) bits |= 1u << u;
+      before = d;
+    }
+    if (bits) atomicOr(&joined[E * t >> 5], bits << (E * t & 31));
+    __syncthreads();
+    auto joins = [&](int i) { return i < c && (joined[i >> 5] >> (i & 31) & 1u) != 0u; };
+#pragma unroll
+    for (int u = 0; u < E; ++u) {
+      const int i = E * t + u;
+      if (i >= c) continue;
+      if (joins(i) || joins(i + 1)) list[atomicAdd(&runs.nlist, 1)] = (uint16_t)i;
+      else if (i < nc) out[i] = (int32_t)(uint32_t)kr[u];
+    }
+    __syncthreads();
+    const int nl = runs.nlist;
+    for (int l = t; l < nl; l += RANK_THREADS) {
+      const int i = list[l];
+      key[i] = (unsigned long long)__double_as_longlong(sqdist64(X + (int64_t)idx[i] * p, xq, p));
+    }
+    __syncthreads();
+    for (int l = t; l < nl; l += RANK_THREADS) {
+      const int i = list[l];
+      int a = i, b = i + 1;
+      while (b - a <= RANK_RUN && joins(a)) --a;
+      while (b - a <= RANK_RUN && joins(b)) ++b;
+      if (b - a > RANK_RUN) { wide = true; continue; }
+      int at = a;
+      for (int m = a; m < b; ++m)
+        at += (key[m] < key[i] || (key[m] == key[i] && idx[m] < idx[i])) ? 1 : 0;
+      if (at < nc) out[at] = idx[i];
+    }
+    if (!__syncthreads_or(wide)) return;
+  }
+#pragma unroll
+  for (int u = 0; u < E; ++u) {
+    const int i = E * t + u;
+    kr[u] = ~0ull;
+    ir[u] = 0x7fffffff;
+    if (i < c) {
+      ir[u] = e[i].idx;
+      kr[u] = (unsigned long long)__double_as_longlong(sqdist64(X + (int64_t)ir[u] * p, xq, p));
+    }
+  }
+  rank_sort<E, true>(kr, ir, key, idx);
+#pragma unroll
+  for (int u = 0; u < E; ++u)
+    if (E * t + u < nc) out[E * t + u] = ir[u];
+}
+
+__global__ void __launch_bounds__(RANK_THREADS, 4)
+knn_rank(const double* __restrict__ X, const float* __restrict__ Xf, int p, int PP,
+         const double* __restrict__ xref, const double* __restrict__ center, int64_t M,
          int nc_max, const int32_t* __restrict__ nc_loc, int cap,
          const KnnEntry* __restrict__ buf, const int32_t* __restrict__ cnt,
          int32_t* __restrict__ cand /*[M][nc_max]*/, unsigned* __restrict__ status) {
@@ -562,30 +692,29 @@ knn_rank(const double* __restrict__ X, int p, const double* __restrict__ xref, i
   const int nc = nc_loc ? nc_loc[q] : nc_max;
   unsigned long long* key = reinterpret_cast<unsigned long long*>(smem_rank);
   int32_t* idx = reinterpret_cast<int32_t*>(key + cap);
+  int32_t* out = cand + q * nc_max;
   __shared__ double xq[LAGP_MAX_P];
+  __shared__ float qf[LAGP_MAX_P];
+  __shared__ RankRuns runs;
   if (threadIdx.x < p) xq[threadIdx.x] = xref[q * p + threadIdx.x];
-  int sz = 1;
-  while (sz < c) sz <<= 1;
+  if (threadIdx.x < PP)
+    qf[threadIdx.x] =
+        threadIdx.x < p ? (float)(xref[q * p + threadIdx.x] - center[threadIdx.x]) : 0.f;
   __syncthreads();
   const KnnEntry* e = buf + q * (int64_t)cap;
-  // the register form needs 1024 slots of shared memory for its exchanges
-  if (sz <= 1024 && cap >= 1024 && blockDim.x == 256) {
-    unsigned long long kr[4];
-    int32_t ir[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = 4 * threadIdx.x + u;
-      if (i < c) {
-        const int32_t gi = e[i].idx;
-        kr[u] = (unsigned long long)__double_as_longlong(sqdist64(X + (int64_t)gi * p, xq, p));
-        ir[u] = gi;
-      } else {
-        kr[u] = ~0ull;
-        ir[u] = 0x7fffffff;
-      }
-    }
-    rank_sort1024(kr, ir, key, idx);
-  } else {
+  if (c >= nc && c <= RANK_MAX) {
+    float qn = 0.f;
+    for (int k = 0; k < p; ++k) qn = fmaf(qf[k], qf[k], qn);
+    qn = sqrtf(qn) * 1.0001f;
+    if (c <= 256) rank_location<1>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
+    else if (c <= 512) rank_location<2>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
+    else if (c <= 1024) rank_location<4>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
+    else rank_location<8>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
+    for (int r = nc + threadIdx.x; r < nc_max; r += blockDim.x) out[r] = -1;
+    return;
+  }
+  int sz = 1;
+  while (sz < c) sz <<= 1;
   for (int i = threadIdx.x; i < sz; i += blockDim.x) {
     if (i < c) {
       int32_t gi = e[i].idx;
@@ -615,13 +744,12 @@ knn_rank(const double* __restrict__ X, int p, const double* __restrict__ xref, i
       __syncthreads();
     }
   }
-  }
   if (c < nc && threadIdx.x == 0) atomicOr(status, LAGP_DEV_KNN_OVERFLOW);
   // ranks this location lacks (a flagged overflow or timeout) repeat a valid
   // index, so that the design kernels never read outside the design
   const int32_t fill = c > 0 ? idx[0] : 0;
   for (int r = threadIdx.x; r < nc_max; r += blockDim.x)
-    cand[q * nc_max + r] = (r < nc) ? (r < c ? idx[r] : fill) : -1;
+    out[r] = (r < nc) ? (r < c ? idx[r] : fill) : -1;
 }
 
 // ---------------------------------------------------------------------------
@@ -754,9 +882,9 @@ cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
   err = cudaFuncSetAttribute(knn_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
   if (err != cudaSuccess) return err;
   prof_begin("knn_rank", s);
-  knn_rank<<<(unsigned)M, 256, smr, s>>>(X, p, xref, M, nc_max, nc_loc, cap,
-                                         reinterpret_cast<const KnnEntry*>(ws.knn_buf),
-                                         ws.knn_cnt, cand, ws.status);
+  knn_rank<<<(unsigned)M, RANK_THREADS, smr, s>>>(
+      X, ws.Xf, p, PP, xref, ws.center, M, nc_max, nc_loc, cap,
+      reinterpret_cast<const KnnEntry*>(ws.knn_buf), ws.knn_cnt, cand, ws.status);
   prof_end(s);
   return cudaGetLastError();
 }
