@@ -90,7 +90,7 @@ __global__ void bbox_final(const double* __restrict__ part, int nparts, int p,
 }
 
 // Xf[i][0..PP) = fl32(X[i] - center) (zero padded), nx[i] = |Xf[i]|^2 in FP32;
-// rows N..Npad-1 are zero with nx = 1e30.  maxn2 receives max_{i<N} nx[i]
+// rows N..Npad-1 are zero with nx = NaN.  maxn2 receives max_{i<N} nx[i]
 // (as ordered bits).
 __global__ void design_to_f32(const double* __restrict__ X, int64_t N, int64_t Npad, int p, int PP,
                               const double* __restrict__ center, float* __restrict__ Xf,
@@ -105,8 +105,9 @@ __global__ void design_to_f32(const double* __restrict__ X, int64_t N, int64_t N
       Xf[i * PP + k] = v;
       acc = fmaf(v, v, acc);
     }
-    // padding rows get |x|^2 = 1e30, so that no distance to them passes
-    nx[i] = i < N ? acc : 1e30f;
+    // padding rows get |x|^2 = NaN, so that no distance to them passes whatever
+    // the design's scale and the threshold (1e30 passed from coordinates of 1e15 on)
+    nx[i] = i < N ? acc : __int_as_float(0x7fc00000);
     if (i < N) local_max = fmaxf(local_max, acc);
   }
   for (int o = 16; o > 0; o >>= 1) local_max = fmaxf(local_max, __shfl_xor_sync(0xffffffffu, local_max, o));

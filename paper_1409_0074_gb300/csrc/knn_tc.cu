@@ -87,7 +87,7 @@ __device__ __forceinline__ float kt_err(int KA, float r) {
 
 // Design tiles [tile][hi | lo][KT_N rows x KA] in canonical order from the
 // centred FP32 copy: row i = [Xf_i, 1, |Xf_i|^2, 0..]; rows past N are
-// [0.., 0, 1e30, 0..] (distance 1e30: they never pass).
+// [0.., 0, NaN, 0..] (distance NaN: they never pass).
 __global__ void design_to_tc(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N,
                              int64_t Npad, int p, int PP, int KA, float* __restrict__ out) {
   const int64_t total = Npad * KA;
@@ -102,7 +102,7 @@ __global__ void design_to_tc(const float* __restrict__ Xf, const float* __restri
       else if (k == p) v = 1.f;
       else if (k == p + 1) v = nx[i];
     } else if (k == p + 1) {
-      v = 1e30f;
+      v = __int_as_float(0x7fc00000);
     }
     const float hi = kt_tf32(v);
     const float lo = kt_tf32(v - hi);
