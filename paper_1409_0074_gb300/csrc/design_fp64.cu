@@ -36,7 +36,8 @@
 
 namespace lagp {
 
-#define D64_THREADS 256
+#define D64_THREADS 256        // of a block; D64_SMALL of the blocks of a small batch
+#define D64_SMALL 512
 #define D64_WARPS (D64_THREADS / 32)
 
 enum { SEARCH_EXHAUSTIVE = 0, SEARCH_RAY = 1 };
@@ -631,9 +632,10 @@ __device__ void design64_location(const D64Params& P, const int64_t loc, double*
   L.xq = dp; dp += p;
   L.lo = dp; dp += p;
   L.hi = dp; dp += p;
-  L.rkz = dp; dp += D64_WARPS * ld;
-  L.ru = dp; dp += D64_WARPS * ld;
-  L.rz = dp; dp += D64_WARPS * p;
+  const int nw = blockDim.x >> 5;
+  L.rkz = dp; dp += nw * ld;
+  L.ru = dp; dp += nw * ld;
+  L.rz = dp; dp += nw * p;
   L.rA = dp; dp += R * p;
   L.rE = dp; dp += R * p;
   L.ralc = dp; dp += R;
@@ -642,7 +644,7 @@ __device__ void design64_location(const D64Params& P, const int64_t loc, double*
   L.xs = dp; dp += p;
   L.scal = dp; dp += 4;
   L.bnd = dp; dp += KD_STACK;
-  L.red = reinterpret_cast<Top2*>(dp); dp += 3 * D64_WARPS;
+  L.red = reinterpret_cast<Top2*>(dp); dp += 3 * nw;
   int* ip = reinterpret_cast<int*>(dp);
   L.sel = ip; ip += ld;
   L.gsel = ip; ip += ld;
@@ -702,8 +704,8 @@ __device__ void design64_location(const D64Params& P, const int64_t loc, double*
 // Without a list, CTA b solves location b.  With a list (the locations an
 // FP32 form hands over for a binary64 re-solve), the CTAs stride over its
 // *count entries, each with its own slot of the exhaustive cache.
-template <int SEARCH>
-__global__ void __launch_bounds__(D64_THREADS) design64(D64Params P) {
+template <int SEARCH, int THREADS>
+__global__ void __launch_bounds__(THREADS) design64(D64Params P) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int64_t ldc = (int64_t)P.n_max * P.nc_max;
   if (!P.list) {
@@ -719,12 +721,25 @@ __global__ void __launch_bounds__(D64_THREADS) design64(D64Params P) {
     design64_location<SEARCH>(P, (int64_t)P.list[it], Kc_slot, smem);
 }
 
-static size_t smem_design64(int n_max, int p, int nc_max, int R) {
+static size_t smem_design64(int n_max, int p, int nc_max, int R, int warps) {
   size_t d = (size_t)n_max * n_max + (size_t)n_max * p + 3 * n_max + 3 * p +
-             2 * D64_WARPS * n_max + D64_WARPS * p + 2 * R * p + 3 * R + p + 4 +
-             3 * D64_WARPS * ((sizeof(Top2) + 7) / 8) + KD_STACK;
+             2 * (size_t)warps * n_max + warps * p + 2 * R * p + 3 * R + p + 4 +
+             3 * warps * ((sizeof(Top2) + 7) / 8) + KD_STACK;
   size_t i = 2 * (size_t)n_max + KD_STACK + 2 * R + 4;
   return d * 8 + i * 4 + nc_max + 16;
+}
+
+// Whether exhaustive blocks have twice the threads: where the batch leaves at most
+// one block per SM, a block has the SM's binary64 pipes to itself, and its step is
+// bound by the latency of each thread's candidates, which there must be enough of
+// (100 locations, n = 30, N' = 500, p = 2: 2.63 ms, with 256 threads 3.02).
+static bool d64_small_batch(const DesignArgs& a, bool list) {
+  int dev = 0, sms = 0;
+  if (list || a.nc_max <= D64_THREADS || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return false;
+  return a.M <= sms &&
+         smem_design64(a.n_max, a.p, a.nc_max, a.nrays, D64_SMALL / 32) <= 227 * 1024;
 }
 
 cudaError_t launch_design_fp64(const DesignArgs& a, int search, cudaStream_t s,
@@ -747,27 +762,23 @@ cudaError_t launch_design_fp64(const DesignArgs& a, int search, cudaStream_t s,
   } else {
     std::memset(&P.kd, 0, sizeof(P.kd));
   }
-  size_t sm = smem_design64(a.n_max, a.p, a.nc_max, a.nrays);
+  // rays: a warp per ray, at least four for the steps the block shares
+  int warps = a.nrays < 4 ? 4 : (a.nrays < D64_WARPS ? a.nrays : D64_WARPS);
+  if (search == SEARCH_EXHAUSTIVE)
+    warps = d64_small_batch(a, list != nullptr) ? D64_SMALL / 32 : D64_WARPS;
+  size_t sm = smem_design64(a.n_max, a.p, a.nc_max, a.nrays, warps);
   const int64_t grid = list ? (a.M < grid_cap ? a.M : grid_cap) : a.M;
   if (grid <= 0) return cudaSuccess;
   cudaError_t err;
-  if (search == SEARCH_EXHAUSTIVE) {
-    err = cudaFuncSetAttribute(design64<SEARCH_EXHAUSTIVE>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (err != cudaSuccess) return err;
-    prof_begin("design64_exhaustive", s);
-    design64<SEARCH_EXHAUSTIVE><<<(unsigned)grid, D64_THREADS, sm, s>>>(P);
-    prof_end(s);
-  } else {
-    err = cudaFuncSetAttribute(design64<SEARCH_RAY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)sm);
-    if (err != cudaSuccess) return err;
-    // one warp per ray, at least four for the steps the block shares
-    const int warps = a.nrays < 4 ? 4 : (a.nrays < D64_WARPS ? a.nrays : D64_WARPS);
-    prof_begin("design64_ray", s);
-    design64<SEARCH_RAY><<<(unsigned)grid, warps * 32, sm, s>>>(P);
-    prof_end(s);
-  }
+  void (*kern)(D64Params) = design64<SEARCH_RAY, D64_THREADS>;
+  if (search == SEARCH_EXHAUSTIVE)
+    kern = warps > D64_WARPS ? design64<SEARCH_EXHAUSTIVE, D64_SMALL>
+                             : design64<SEARCH_EXHAUSTIVE, D64_THREADS>;
+  err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (err != cudaSuccess) return err;
+  prof_begin(search == SEARCH_EXHAUSTIVE ? "design64_exhaustive" : "design64_ray", s);
+  kern<<<(unsigned)grid, warps * 32, sm, s>>>(P);
+  prof_end(s);
   return cudaGetLastError();
 }
 
