@@ -63,8 +63,8 @@ extern "C" {
  *   Exhaustive search keeps every candidate's running |L^{-1} k|^2 and
  *   (L^{-1} k) . (L^{-1} k(x)), extended by one term per step (the factor
  *   only gains a row), on the FP32 CUDA cores.
- * LAGP_FP32_SCORE_TC: as LAGP_FP32_SCORE, but exhaustive search forms all of
- *   W = Kc L_j^{-T} at every step as a dense contraction on the tensor cores
+ * LAGP_FP32_SCORE_TC: as LAGP_FP32_SCORE, but exhaustive search forms each
+ *   step's new column of W = Kc L_j^{-T} as a contraction on the tensor cores
  *   (3xTF32 split products, FP32 accumulation) for local designs up to 64
  *   points (larger ones as LAGP_FP32_SCORE).  Same method and tolerances,
  *   other rounding; ray search is the same as LAGP_FP32_SCORE.

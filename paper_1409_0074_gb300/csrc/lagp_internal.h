@@ -29,7 +29,7 @@ struct Workspace {
   int32_t* cand;        // [chunk][nc_max] candidate design indices, nearest first
   double* state64;      // FP64 state: FP64 form, exhaustive: [chunk][nc_max][n_max]
                         // correlation cache; FP32 form: per slot, L^{-1} and its vectors
-  float* state32;       // FP32 form, exhaustive: [slots][n_max][nc_max] correlation cache
+  float* state32;       // FP32 form, exhaustive: [slots][n_max][nc_max, rounded up to 4] correlation cache
   float* crow;          // FP32 form, exhaustive: [CTA slots][nc_max][PP] candidate rows
   unsigned* queue;      // [4] work counters of the persistent kernels
   int32_t* order;       // [2][chunk] work order (largest local designs first), two parts
