@@ -95,7 +95,7 @@ extern "C" {
 /* Return codes. */
 #define LAGP_OK 0
 #define LAGP_ERR_INVALID (-1)   /* an argument is out of range or a pointer is NULL */
-#define LAGP_ERR_WORKSPACE (-2) /* workspace_bytes is below laGP_workspace_bytes */
+#define LAGP_ERR_WORKSPACE (-2) /* workspace_bytes is too small (laGP_workspace_bytes) */
 #define LAGP_ERR_CUDA (-3)      /* a CUDA call or kernel launch failed */
 #define LAGP_ERR_DEVICE (-4)    /* laGP_status: the device reported a failure */
 #define LAGP_BUSY 1             /* laGP_ctx_submit: no free slot or arena region now */
@@ -107,9 +107,18 @@ extern "C" {
                                        mean and s2 are NaN */
 
 /*
- * Bytes of device workspace laGP_build_and_predict needs for these sizes.
+ * Bytes of device workspace for laGP_build_and_predict at these sizes.
  * Arguments as in laGP_build_and_predict (n and N_close are the maxima when
  * per-location arrays are used).  Returns 0 when the sizes are invalid.
+ *
+ * Of these, 8 bytes per location of a chunk (at most 131072) and entry are the
+ * kNN candidate buffers.  They have the power of two at or above 5 N_close / 2
+ * + 256 entries (at least 512), or up to 16384 where the fast filter's threshold
+ * admits more (N_close <= 102 and 177 to 307 up to N = 5e5; <= 307 at N = 1e6;
+ * <= 1536 at N = 1e7).  An entry point that takes a workspace also runs in what remains
+ * with the smaller buffers, in the time that its search without that threshold
+ * takes, and with fewer equal distances before LAGP_STATUS_CAPACITY; below that
+ * it returns LAGP_ERR_WORKSPACE.
  */
 size_t laGP_workspace_bytes(int64_t N, int p, int64_t M, int n, int N_close, int nrays,
                             int search, int precision);
@@ -150,7 +159,7 @@ size_t laGP_workspace_bytes(int64_t N, int p, int64_t M, int n, int N_close, int
  *             the snap); 0 elsewhere
  *   nevals    device [M][n] int32 out or NULL: ALC evaluations of ray step j
  *             at entry j - n0 (0 for the exhaustive search)
- *   workspace device scratch of workspace_bytes >= laGP_workspace_bytes(...)
+ *   workspace device scratch, workspace_bytes as laGP_workspace_bytes(...) says
  *   stream    cudaStream_t
  *
  * A location whose update meets v <= 0 gets NaN in mean and s2 and sets
@@ -189,9 +198,10 @@ int laGP_knn(const double* design, int64_t N, int p, const double* xref, int64_t
  *   status    device unsigned* or NULL: receives the LAGP_STATUS_* bits of
  *             this call once the stream reaches the end of it (0 when M = 0)
  *   stream    cudaStream_t
- * Limits: the scratch needed, laGP_knn_workspace_bytes(N, p, M, N_close),
- * must not exceed LAGP_KNN_NOALLOC_SCRATCH_BYTES (64 MiB); larger requests
- * return LAGP_ERR_WORKSPACE before any device work.  Every GPU that loads the
+ * Limits: the scratch needed, laGP_knn_workspace_bytes(N, p, M, N_close) with
+ * the smaller candidate buffers (laGP_workspace_bytes), must not exceed
+ * LAGP_KNN_NOALLOC_SCRATCH_BYTES (64 MiB); larger requests return
+ * LAGP_ERR_WORKSPACE before any device work.  Every GPU that loads the
  * library holds that array until the process exits.
  * The first call on a device looks up the array's device address (with that
  * device current); make that first call before any stream capture.  A call
@@ -420,8 +430,9 @@ int laGP_plan_destroy(laGP_plan* plan);
  * laGP_ctx_request_bytes(N, p, M, n, N_close, nrays, search, precision,
  * selected != NULL) bytes; it copies the inputs, enqueues the path on the
  * slot's stream, queues the copies of the outputs and returns LAGP_OK with a
- * ticket.  Without a free slot or region it returns LAGP_BUSY and does
- * nothing.  Host buffers should be page-locked: a pageable output makes the
+ * ticket.  A request whose region would not fit into the arena even alone gets
+ * the smaller candidate buffers (laGP_workspace_bytes) and a smaller region.
+ * Without a free slot or region it returns LAGP_BUSY and does nothing.  Host buffers should be page-locked: a pageable output makes the
  * call wait for the request to finish.  Results of a location do not depend
  * on the other locations of its request nor on concurrent requests.
  *

@@ -34,6 +34,7 @@
 #include "common.cuh"
 #include "knn_common.cuh"
 #include "lagp_internal.h"
+#include "launch_plan.h"
 
 namespace lagp {
 
@@ -792,34 +793,8 @@ size_t knn_smem_stream(int PP) {
 // locations, N = 8 N': 60 against 69 us at 1024, 80 against 83 at 2000, 142
 // against 107 at 4000; one location, N = 16 N': 92 against 97 us at 8000, 169
 // against 150 at 16000.
-static int64_t knn_sample(int64_t N) { return N / 16 < 32768 ? N / 16 : 32768; }
-static bool knn_uses_tc(int64_t N, int nc_max) { return N >= (int64_t)32 * nc_max; }
-static bool knn_mid(int64_t N, int nc_max) { return N >= (int64_t)4 * nc_max && N >= 1024; }
 static bool knn_has_pilot(int64_t N, int64_t M, int nc_max) {
   return knn_uses_tc(N, nc_max) || (knn_mid(N, nc_max) && M * N >= 16384);
-}
-
-// Buffer entries per location: room for N' survivors, a whole tile of new
-// inserts before the next compaction, and N'/2 (at least 64) entries of slack
-// for distances within the error margin of the N'-th; with a pilot threshold
-// also for the points that it is expected to admit and the two tiles that the
-// pilot asks for beside them.  Without that room, as for N' <= 307 at N = 1e6, the
-// pilot gives no threshold and every location streams the whole design from
-// infinity: 5.2 ms for one location and 9.5 ms for 10,000 at N' = 250, p = 4,
-// where the tensor-core filter takes 0.035 and 4.0 ms.  A power of two, as the
-// bitonic sort of knn_rank wants.
-int knn_cap(int nc_max, int64_t N) {
-  const int need = (5 * nc_max) / 2 + LAGP_KNN_TILE;
-  int cap = 512;
-  while (cap < need) cap <<= 1;
-  if (knn_uses_tc(N, nc_max) || knn_mid(N, nc_max)) {
-    const double ratio = (double)N / (double)knn_sample(N), lam = nc_max / ratio;
-    const double admits = (lam + 4.5 * sqrt(lam) + 6.0) * ratio;
-    int more = cap;
-    while (more < 16384 && admits > more - 2 * LAGP_KNN_TILE) more <<= 1;
-    if (admits <= more - 2 * LAGP_KNN_TILE) cap = more;
-  }
-  return cap;
 }
 
 cudaError_t launch_prepare(const double* X, int64_t N, int p, int PP, int64_t Npad,
@@ -844,8 +819,7 @@ cudaError_t launch_prepare(const double* X, int64_t N, int p, int PP, int64_t Np
 
 cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
                        const double* xref, int64_t M, int nc_max, const int32_t* nc_loc,
-                       int32_t* cand, const Workspace& ws, cudaStream_t s) {
-  const int cap = knn_cap(nc_max, N);
+                       int cap, int32_t* cand, const Workspace& ws, cudaStream_t s) {
   const int64_t ntiles = Npad / LAGP_KNN_TILE;
   const int qpb = KNN_WARPS * KNN_QW;
   dim3 grid((unsigned)((M + qpb - 1) / qpb));

@@ -13,6 +13,7 @@
 #include <mutex>
 
 #include "../../include/lagp.h"
+#include "lagp_internal.h"
 
 // The scratch array.  Every GPU that loads the library reserves this much
 // device memory until the process exits.
@@ -85,7 +86,7 @@ int scratch_for_current_device(void** out) {
 extern "C" int laGP_knn_noalloc(const double* design, int64_t N, int p, const double* xref,
                                 int64_t M, int N_close, int32_t* cand, unsigned* status,
                                 void* stream) {
-  const size_t need = laGP_knn_workspace_bytes(N, p, M, N_close);
+  const size_t need = lagp::knn_least_bytes(N, p, M, N_close);
   if (need == 0) return LAGP_ERR_INVALID;
   if (need > (size_t)LAGP_KNN_NOALLOC_SCRATCH_BYTES) return LAGP_ERR_WORKSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -100,7 +101,7 @@ extern "C" int laGP_knn_noalloc(const double* design, int64_t N, int p, const do
   int rc = scratch_for_current_device(&ws);
   if (rc != LAGP_OK) return rc;
   // laGP_knn clears the status word and rewrites every scratch region it reads.
-  rc = laGP_knn(design, N, p, xref, M, N_close, cand, ws, need, stream);
+  rc = laGP_knn(design, N, p, xref, M, N_close, cand, ws, LAGP_KNN_NOALLOC_SCRATCH_BYTES, stream);
   if (rc != LAGP_OK) return rc;
   if (status) {
     // the status word leads the scratch layout

@@ -10,15 +10,19 @@ namespace lagp {
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Locations per chunk: bounded by a per-search cap and by keeping the kNN
+// Locations per chunk: bounded by a per-search limit and by keeping the kNN
 // candidate buffers within 16 GiB.
-static int64_t chunk_for(int64_t M, int search, int precision, int nc_max, int64_t N) {
-  int64_t cap = 131072;
-  if (search == LAGP_EXHAUSTIVE && precision == LAGP_FP64) cap = 16384;
-  const int64_t per_loc = (int64_t)8 * knn_cap(nc_max, N);
-  const int64_t by_mem = ((int64_t)16 << 30) / per_loc;
-  if (by_mem < cap) cap = by_mem > 128 ? by_mem : 128;
-  return M < cap ? (M > 0 ? M : 1) : cap;
+static int64_t chunk_for(const Shape& sh) {
+  int64_t lim = 131072;
+  if (sh.search == LAGP_EXHAUSTIVE && sh.precision == LAGP_FP64) lim = 16384;
+  const int64_t by_mem = ((int64_t)16 << 30) / ((int64_t)8 * sh.cap);
+  if (by_mem < lim) lim = by_mem > 128 ? by_mem : 128;
+  return sh.M < lim ? (sh.M > 0 ? sh.M : 1) : lim;
+}
+
+void set_cap(Shape* sh, int cap) {
+  sh->cap = cap;
+  sh->chunk = chunk_for(*sh);
 }
 
 namespace {
@@ -41,7 +45,7 @@ size_t layout_request(const Shape& sh, void* base, Workspace* ws) {
   Carver c{static_cast<char*>(base), 0};
   w->status = static_cast<unsigned*>(c.take(4 * sizeof(unsigned)));
   const int64_t ch = sh.chunk;
-  w->knn_buf = c.take((size_t)8 * ch * knn_cap(sh.nc_max, sh.N));
+  w->knn_buf = c.take((size_t)8 * ch * sh.cap);
   w->knn_cnt = static_cast<int32_t*>(c.take(sizeof(int32_t) * ch));
   w->knn_thr = static_cast<float*>(c.take(sizeof(float) * ch));
   w->knn_seg = static_cast<int32_t*>(c.take(sizeof(int32_t) * 4 * ch));
@@ -111,6 +115,8 @@ size_t layout_workspace(const Shape& sh, void* base, Workspace* ws) {
   return r + d;
 }
 
+size_t workspace_need(const Shape& sh) { return layout_workspace(sh, nullptr, nullptr); }
+
 bool make_shape(int64_t N, int p, int64_t M, int n0, int n, int N_close, int nrays, int search,
                 int precision, Shape* sh, bool knn_only) {
   if (p < 1 || p > LAGP_MAX_P || N < 1 || M < 0) return false;
@@ -137,13 +143,20 @@ bool make_shape(int64_t N, int p, int64_t M, int n0, int n, int N_close, int nra
   sh->search = search;
   sh->precision = form;
   sh->promote = (precision & LAGP_PROMOTE) != 0;
-  sh->chunk = chunk_for(M, search, form, N_close, N);
+  set_cap(sh, knn_cap(N_close, N));
   return true;
 }
 
 }  // namespace lagp
 
 using namespace lagp;
+
+size_t lagp::knn_least_bytes(int64_t N, int p, int64_t M, int N_close) {
+  Shape sh;
+  if (!make_shape(N, p, M, 1, 1, N_close, 1, LAGP_RAY, LAGP_FP64, &sh, true)) return 0;
+  set_cap(&sh, knn_cap_least(N_close));
+  return workspace_need(sh);
+}
 
 extern "C" size_t laGP_workspace_bytes(int64_t N, int p, int64_t M, int n, int N_close,
                                        int nrays, int search, int precision) {
@@ -243,7 +256,7 @@ int enqueue(const Shape& sh, const Call& c, const Workspace& ws, const Tune& t, 
     const int64_t Mc = (sh.M - c0 < sh.chunk) ? sh.M - c0 : sh.chunk;
     const int32_t* ncl = c.nclose_loc ? c.nclose_loc + c0 : nullptr;
     if (launch_knn(c.design, sh.N, sh.p, sh.PP, sh.Npad, c.xref + c0 * sh.p, Mc, sh.nc_max, ncl,
-                   ws.cand, ws, s) != cudaSuccess)
+                   sh.cap, ws.cand, ws, s) != cudaSuccess)
       return LAGP_ERR_CUDA;
     const DesignArgs a = chunk_args(sh, c, ws, c0, Mc, t);
     if (run_design(a, sh.search, sh.precision, uneven, s) != cudaSuccess) return LAGP_ERR_CUDA;
@@ -259,8 +272,8 @@ static int check_call(int64_t N, int p, const double* xref, int64_t M, int n0, i
   if (!(theta > 0.0) || !(g >= 0.0) || theta != theta) return LAGP_ERR_INVALID;
   if (M == 0) return 1;
   if (!design || !y || !xref || !mean || !s2 || !workspace) return LAGP_ERR_INVALID;
-  const size_t need = layout_workspace(*sh, workspace, ws);
-  if (workspace_bytes < need) return LAGP_ERR_WORKSPACE;
+  if (!fit_cap(sh, workspace_bytes, workspace_need)) return LAGP_ERR_WORKSPACE;
+  layout_workspace(*sh, workspace, ws);
   return LAGP_OK;
 }
 
@@ -321,8 +334,8 @@ extern "C" int laGP_autotune(const double* design, const double* y, int64_t N, i
   const int64_t Mc = sh.M < sh.chunk ? sh.M : sh.chunk;
   if (cudaMemsetAsync(ws.status, 0, 3 * sizeof(unsigned), s) != cudaSuccess) return LAGP_ERR_CUDA;
   if (launch_prepare(design, sh.N, sh.p, sh.PP, sh.Npad, ws, s) != cudaSuccess) return LAGP_ERR_CUDA;
-  if (launch_knn(design, sh.N, sh.p, sh.PP, sh.Npad, xref, Mc, sh.nc_max, nclose_loc, ws.cand, ws,
-                 s) != cudaSuccess)
+  if (launch_knn(design, sh.N, sh.p, sh.PP, sh.Npad, xref, Mc, sh.nc_max, nclose_loc, sh.cap,
+                 ws.cand, ws, s) != cudaSuccess)
     return LAGP_ERR_CUDA;
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess) return LAGP_ERR_CUDA;
@@ -388,16 +401,16 @@ extern "C" int laGP_knn(const double* design, int64_t N, int p, const double* xr
     return LAGP_ERR_INVALID;
   if (M == 0) return LAGP_OK;
   if (!design || !xref || !cand || !workspace) return LAGP_ERR_INVALID;
+  if (!fit_cap(&sh, workspace_bytes, workspace_need)) return LAGP_ERR_WORKSPACE;
   Workspace ws;
-  const size_t need = layout_workspace(sh, workspace, &ws);
-  if (workspace_bytes < need) return LAGP_ERR_WORKSPACE;
+  layout_workspace(sh, workspace, &ws);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(ws.status, 0, 3 * sizeof(unsigned), s) != cudaSuccess) return LAGP_ERR_CUDA;
   if (launch_prepare(design, N, p, sh.PP, sh.Npad, ws, s) != cudaSuccess) return LAGP_ERR_CUDA;
   for (int64_t c0 = 0; c0 < M; c0 += sh.chunk) {
     const int64_t Mc = (M - c0 < sh.chunk) ? M - c0 : sh.chunk;
     if (launch_knn(design, N, p, sh.PP, sh.Npad, xref + c0 * p, Mc, N_close, nullptr,
-                   cand + c0 * N_close, ws, s) != cudaSuccess)
+                   sh.cap, cand + c0 * N_close, ws, s) != cudaSuccess)
       return LAGP_ERR_CUDA;
   }
   return LAGP_OK;
@@ -470,12 +483,16 @@ extern "C" int laGP_build_and_predict_host(const double* design, const double* y
                                            int32_t* selected, double* tie_gap, int32_t* nevals,
                                            void* workspace, size_t workspace_bytes,
                                            void* stream) {
-  const size_t wsb = laGP_workspace_bytes(N, p, M, n, N_close, nrays, search, precision);
-  if (wsb == 0) return LAGP_ERR_INVALID;
+  Shape sh;
+  if (!make_shape(N, p, M, 1, n, N_close, nrays, search, precision, &sh)) return LAGP_ERR_INVALID;
   if (M == 0) return LAGP_OK;
   if (!design || !y || !xref || !mean || !s2 || !workspace) return LAGP_ERR_INVALID;
-  HostLayout h = host_layout(N, p, M, n, wsb);
-  if (workspace_bytes < h.total) return LAGP_ERR_WORKSPACE;
+  if (!fit_cap(&sh, workspace_bytes, [&](const Shape& t) {
+        return host_layout(N, p, M, n, workspace_need(t)).total;
+      }))
+    return LAGP_ERR_WORKSPACE;
+  const size_t wsb = workspace_need(sh);
+  const HostLayout h = host_layout(N, p, M, n, wsb);
   char* b = static_cast<char*>(workspace);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   auto h2d = [&](size_t off, const void* src, size_t bytes) {
@@ -533,8 +550,11 @@ extern "C" int laGP_build_and_predict_mle(const double* design, const double* y,
                             design, y, mean, s2, workspace, workspace_bytes, &sh, &ws);
   if (rc != LAGP_OK) return rc > 0 ? LAGP_OK : rc;
   if (!theta_out) return LAGP_ERR_INVALID;
-  const size_t base = layout_workspace(sh, nullptr, nullptr);
-  if (workspace_bytes < base + align256(sizeof(int32_t) * sh.chunk * n)) return LAGP_ERR_WORKSPACE;
+  if (!fit_cap(&sh, workspace_bytes, [&](const Shape& t) {
+        return workspace_need(t) + align256(sizeof(int32_t) * t.chunk * n);
+      }))
+    return LAGP_ERR_WORKSPACE;
+  const size_t base = layout_workspace(sh, workspace, &ws);
   int32_t* selbuf = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + base);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(ws.status, 0, 3 * sizeof(unsigned), s) != cudaSuccess) return LAGP_ERR_CUDA;
@@ -544,7 +564,7 @@ extern "C" int laGP_build_and_predict_mle(const double* design, const double* y,
   for (int64_t c0 = 0; c0 < sh.M; c0 += sh.chunk) {
     const int64_t Mc = (sh.M - c0 < sh.chunk) ? sh.M - c0 : sh.chunk;
     if (launch_knn(design, sh.N, sh.p, sh.PP, sh.Npad, xref + c0 * sh.p, Mc, sh.nc_max, nullptr,
-                   ws.cand, ws, s) != cudaSuccess)
+                   sh.cap, ws.cand, ws, s) != cudaSuccess)
       return LAGP_ERR_CUDA;
     // stage 1: the design at theta0, then theta-hat on it (and the prediction there)
     const Call c{design, y, xref, theta0, g, nullptr, nullptr, mean, s2, nullptr, nullptr,

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "kdtree.cuh"
+#include "launch_plan.h"
 
 namespace lagp {
 
@@ -109,8 +110,20 @@ struct Shape {
   int n0, n_max, nc_max, nrays;
   int search, precision;      // precision: the form, LAGP_PROMOTE stripped
   bool promote;               // FP32 forms with LAGP_PROMOTE
+  int cap;                    // entries of a location's kNN candidate buffer
   int64_t chunk;
 };
+
+// Sets the kNN buffers' size and with it the chunk (make_shape: knn_cap).
+void set_cap(Shape* sh, int cap);
+// Keeps the buffers of make_shape where need(shape) bytes are there, else takes
+// the smallest that a search can run with; false when those do not fit either.
+template <typename Need>
+bool fit_cap(Shape* sh, size_t bytes, Need need) {
+  if (need(*sh) <= bytes) return true;
+  set_cap(sh, knn_cap_least(sh->nc_max));
+  return need(*sh) <= bytes;
+}
 
 // Layout of the workspace for a shape; returns total bytes.  With base != null
 // fills ws with pointers into [base, base + bytes).  The workspace is the
@@ -119,8 +132,8 @@ struct Shape {
 size_t layout_workspace(const Shape& sh, void* base, Workspace* ws);
 size_t layout_request(const Shape& sh, void* base, Workspace* ws);
 size_t layout_design(const Shape& sh, void* base, Workspace* ws);
+size_t workspace_need(const Shape& sh);   // bytes of layout_workspace
 
-int knn_cap(int nc_max, int64_t N);
 size_t knn_smem_stream(int PP);
 
 cudaError_t launch_prepare(const double* X, int64_t N, int p, int PP, int64_t Npad,
@@ -132,7 +145,7 @@ cudaError_t launch_knn_tc(int64_t Npad, int p, const double* xref, int64_t M, in
                           const int32_t* nc_loc, int cap, const Workspace& ws, cudaStream_t s);
 cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
                        const double* xref, int64_t M, int nc_max, const int32_t* nc_loc,
-                       int32_t* cand, const Workspace& ws, cudaStream_t s);
+                       int cap, int32_t* cand, const Workspace& ws, cudaStream_t s);
 
 // Greedy local design and prediction for one chunk of locations.
 struct DesignArgs {
@@ -171,6 +184,8 @@ cudaError_t launch_order(const DesignArgs& a, int search, int split_n, int lpt, 
 // Validated shape of a call (false if an argument is out of range).
 bool make_shape(int64_t N, int p, int64_t M, int n0, int n, int N_close, int nrays, int search,
                 int precision, Shape* sh, bool knn_only = false);
+// Bytes below which a candidate search of this shape is refused (0: invalid).
+size_t knn_least_bytes(int64_t N, int p, int64_t M, int N_close);
 
 // Arguments of one predictive call (device pointers).
 struct Call {

@@ -1,6 +1,7 @@
 // launch_plan.h -- host-side launch arithmetic of the persistent and tiled
 // kernels, kept free of CUDA so that it compiles and is tested on any host.
 #pragma once
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 
@@ -48,6 +49,42 @@ inline int warps_per_cta_for_residency(size_t warp_bytes, size_t smem_sm, size_t
     }
   }
   return best;
+}
+
+// Sample rows of the kNN pilot.
+inline int64_t knn_sample(int64_t N) { return N / 16 < 32768 ? N / 16 : 32768; }
+// The tensor-core filter, and the sizes below it whose stream may take a pilot
+// threshold too.
+inline bool knn_uses_tc(int64_t N, int nc_max) { return N >= (int64_t)32 * nc_max; }
+inline bool knn_mid(int64_t N, int nc_max) { return N >= (int64_t)4 * nc_max && N >= 1024; }
+
+// Entries of a location's kNN candidate buffer.  It needs room for N'
+// survivors, a whole tile of 256 new inserts before the next compaction, and
+// N'/2 (at least 64) entries of slack for distances within the error margin of
+// the N'-th; a power of two, as the bitonic sort of knn_rank wants.
+inline int knn_cap_least(int nc_max) {
+  const int need = (5 * nc_max) / 2 + 256;
+  int cap = 512;
+  while (cap < need) cap <<= 1;
+  return cap;
+}
+// With a pilot threshold it is also to hold the points that the threshold is
+// expected to admit and the two tiles that the pilot asks for beside them.
+// Without that room, as for N' <= 307 at N = 1e6, the pilot gives no threshold
+// and every location streams the whole design from infinity: 5.2 ms for one
+// location and 9.5 ms for 10,000 at N' = 250, p = 4, where the tensor-core filter
+// takes 0.035 and 4.0 ms.  The lists are the same either way, so a call whose
+// workspace has no room for these buffers runs with the smallest ones.
+inline int knn_cap(int nc_max, int64_t N) {
+  int cap = knn_cap_least(nc_max);
+  if (knn_uses_tc(N, nc_max) || knn_mid(N, nc_max)) {
+    const double ratio = (double)N / (double)knn_sample(N), lam = nc_max / ratio;
+    const double admits = (lam + 4.5 * std::sqrt(lam) + 6.0) * ratio;
+    int more = cap;
+    while (more < 16384 && admits > more - 512) more <<= 1;
+    if (admits <= more - 512) cap = more;
+  }
+  return cap;
 }
 
 }  // namespace lagp

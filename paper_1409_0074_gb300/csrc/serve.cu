@@ -43,8 +43,9 @@ extern "C" int laGP_plan_create(const double* design, const double* y, int64_t N
     return LAGP_ERR_INVALID;
   if (!(theta > 0.0) || !(g >= 0.0) || theta != theta) return LAGP_ERR_INVALID;
   if (!design || !y || !xref || !mean || !s2 || !workspace) return LAGP_ERR_INVALID;
+  if (!fit_cap(&sh, workspace_bytes, workspace_need)) return LAGP_ERR_WORKSPACE;
   Workspace ws;
-  if (workspace_bytes < layout_workspace(sh, workspace, &ws)) return LAGP_ERR_WORKSPACE;
+  layout_workspace(sh, workspace, &ws);
   const Call c{design, y, xref, theta, g, n_loc, nclose_loc, mean, s2, selected, tie_gap, nevals};
   cudaStream_t cs;
   if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return LAGP_ERR_CUDA;
@@ -252,8 +253,13 @@ extern "C" int laGP_ctx_submit(laGP_ctx* c, const double* xref, int64_t M, int n
   if (!c || !xref || !mean || !s2 || !ticket || M < 1) return LAGP_ERR_INVALID;
   std::lock_guard<std::mutex> lk(c->mu);
   bool ok = false;
-  const Shape sh = ctx_shape(c, M, n, &ok);
+  Shape sh = ctx_shape(c, M, n, &ok);
   if (!ok) return LAGP_ERR_INVALID;
+  // an arena too small for the request's larger kNN buffers gives it the
+  // smallest: by the arena's size, not by what is free in it, so that the same
+  // request runs the same way whatever else is in flight
+  const size_t room = c->arena_bytes - up256(c->design_bytes);
+  fit_cap(&sh, room, [&](const Shape& t) { return req_layout(t, selected != nullptr).total; });
   int si = -1;
   for (size_t i = 0; i < c->slots.size(); ++i)
     if (!c->slots[i].busy) { si = (int)i; break; }
