@@ -34,7 +34,7 @@ size_t kd_bytes(int64_t N, int p, int PP) {
   return al256(sizeof(int32_t) * N) + al256(sizeof(float) * N * PP) +
          al256(sizeof(float) * nodes * 2 * PP) + al256(sizeof(double) * nodes * 2 * p) +
          al256(sizeof(uint64_t) * 2 * N) + al256(sizeof(int32_t) * N) +
-         al256(sizeof(uint32_t) * 256 * ((size_t)rs_blocks(N) + 1));
+         al256(sizeof(uint32_t) * 256);
 }
 
 void kd_carve(int64_t N, int p, int PP, char* base, KdTree* t) {
@@ -49,7 +49,11 @@ void kd_carve(int64_t N, int p, int PP, char* base, KdTree* t) {
   t->box64 = reinterpret_cast<double*>(take(sizeof(double) * nodes * 2 * p));
   t->keys = reinterpret_cast<uint64_t*>(take(sizeof(uint64_t) * 2 * N));
   t->vals = reinterpret_cast<int32_t*>(take(sizeof(int32_t) * N));
-  t->hist = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * ((size_t)rs_blocks(N) + 1)));
+  t->total = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * 256));
+  // the tile counts are needed until the rows and boxes are written, and take
+  // less (N + 1,024 bytes at most, against 16 N of the rows and, where N < 64, 256
+  // of the boxes after them)
+  t->hist = reinterpret_cast<uint32_t*>(t->pts32);
 }
 
 // keys of level `level`: the position's node (relative index within the level)
@@ -244,7 +248,6 @@ cudaError_t launch_kd_build(const double* X, const float* Xf, const double* lo, 
   const unsigned g = (unsigned)((N + 255) / 256 < 4096 ? (N + 255) / 256 : 4096);
   prof_begin("kd_build", s);
   uint64_t* kb[2] = {t.keys, t.keys + N};
-  uint32_t* total = t.hist + 256 * (size_t)nblk;     // [256] digit totals of a pass
   for (int level = 0; level < D; ++level) {
     // keys into buffer 0 (values: the current order, identity at level 0)
     kd_keys<<<g, 256, 0, s>>>(t.perm, Xf, N, PP, level, level % p, level == 0, lo, hi, kb[0],
@@ -256,8 +259,9 @@ cudaError_t launch_kd_build(const double* X, const float* Xf, const double* lo, 
     for (int ps = 0; ps < passes; ++ps) {
       const int shift = 8 * ps;
       rs_hist<<<nblk, 256, 0, s>>>(kb[cur], N, shift, t.hist);
-      rs_scan<<<256, 256, 0, s>>>(t.hist, nblk, total);
-      rs_scatter<<<nblk, 32, 0, s>>>(kb[cur], vcur, kb[cur ^ 1], valt, N, shift, t.hist, total);
+      rs_scan<<<256, 256, 0, s>>>(t.hist, nblk, t.total);
+      rs_scatter<<<nblk, 32, 0, s>>>(kb[cur], vcur, kb[cur ^ 1], valt, N, shift, t.hist,
+                                      t.total);
       cur ^= 1;
       int32_t* tmp = vcur;
       vcur = valt;

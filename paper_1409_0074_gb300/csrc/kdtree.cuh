@@ -237,7 +237,8 @@ struct KdTree {
   double* box64;     // [nodes][2][p]
   uint64_t* keys;    // [2][N] sort scratch
   int32_t* vals;     // [N] sort scratch
-  uint32_t* hist;    // [256][blocks] sort scratch, then [256] totals
+  uint32_t* total;   // [256] digit totals of a sort pass
+  uint32_t* hist;    // [256][blocks] tile counts, in the place of pts32 and box32
 };
 
 size_t kd_bytes(int64_t N, int p, int PP);

@@ -29,3 +29,23 @@ def test_noalloc_takes_what_its_scratch_holds_with_the_smallest_buffers(lib):
     assert lib.laGP_knn_noalloc(None, N, P, None, M, NC, None, None, None) == -1
     more = M + (scratch - least) // 4096
     assert lib.laGP_knn_noalloc(None, N, P, None, more, NC, None, None, None) == -2
+
+
+@pytest.mark.parametrize("n,p", [(40, 1), (64, 2), (5000, 3), (100_000, 8), (1_000_000, 16)])
+def test_unlimited_scope_adds_the_tree_and_its_keys(lib, n, p):
+    """The tree (order, FP32 rows, both boxes of every node) and what its sort
+    takes beside it: two key buffers, one of positions, and no more than a
+    kilobyte per 4,096 points."""
+    from paper_1409_0074_gb300 import lagp
+
+    def up(x):
+        return (x + 255) & ~255
+
+    size = [lib.laGP_workspace_bytes(n, p, 10, 8, 20, 2, s, lagp.LAGP_FP32_SCORE)
+            for s in (lagp.LAGP_RAY, lagp.LAGP_RAY_FULL)]
+    depth = 0
+    while -(-n // (1 << depth)) > 32:
+        depth += 1
+    nodes, pp = 2 << depth, -(-p // 4) * 4
+    tree = up(4 * n) + up(4 * n * pp) + up(4 * nodes * 2 * pp) + up(8 * nodes * 2 * p)
+    assert size[1] - size[0] <= tree + up(16 * n) + up(4 * n) + 1024 * -(-n // 4096)
