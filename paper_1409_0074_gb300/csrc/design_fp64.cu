@@ -141,8 +141,8 @@ struct Loc {
   Top2* red;         // [WARPS]
   int* sel;          // [n_max] selected ranks (-1: not a candidate)
   int* gsel;         // [n_max] selected design indices
-  int* stk;          // [KD_STACK] k-d tree walk (full scope): nodes
-  double* bnd;       // [KD_STACK] and their box distances
+  int* stk;          // [KD_STACK] k-d tree walk (full scope only): nodes
+  double* bnd;       // [KD_BOUNDS] and their descendants' box distances
   int* rnev;         // [R]
   int* starts;       // [R]
   int* iscal;        // [4]
@@ -643,12 +643,12 @@ __device__ void design64_location(const D64Params& P, const int64_t loc, double*
   L.rgap = dp; dp += R;
   L.xs = dp; dp += p;
   L.scal = dp; dp += 4;
-  L.bnd = dp; dp += KD_STACK;
+  L.bnd = dp; dp += P.full ? KD_BOUNDS : 0;
   L.red = reinterpret_cast<Top2*>(dp); dp += 3 * nw;
   int* ip = reinterpret_cast<int*>(dp);
   L.sel = ip; ip += ld;
   L.gsel = ip; ip += ld;
-  L.stk = ip; ip += KD_STACK;
+  L.stk = ip; ip += P.full ? KD_STACK : 0;
   L.rnev = ip; ip += R;
   L.starts = ip; ip += R;
   L.iscal = ip; ip += 4;
@@ -721,11 +721,11 @@ __global__ void __launch_bounds__(THREADS) design64(D64Params P) {
     design64_location<SEARCH>(P, (int64_t)P.list[it], Kc_slot, smem);
 }
 
-static size_t smem_design64(int n_max, int p, int nc_max, int R, int warps) {
+static size_t smem_design64(int n_max, int p, int nc_max, int R, int warps, bool full) {
   size_t d = (size_t)n_max * n_max + (size_t)n_max * p + 3 * n_max + 3 * p +
              2 * (size_t)warps * n_max + warps * p + 2 * R * p + 3 * R + p + 4 +
-             3 * warps * ((sizeof(Top2) + 7) / 8) + KD_STACK;
-  size_t i = 2 * (size_t)n_max + KD_STACK + 2 * R + 4;
+             3 * warps * ((sizeof(Top2) + 7) / 8) + (full ? KD_BOUNDS : 0);
+  size_t i = 2 * (size_t)n_max + (full ? KD_STACK : 0) + 2 * R + 4;
   return d * 8 + i * 4 + nc_max + 16;
 }
 
@@ -739,7 +739,7 @@ static bool d64_small_batch(const DesignArgs& a, bool list) {
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return false;
   return a.M <= sms &&
-         smem_design64(a.n_max, a.p, a.nc_max, a.nrays, D64_SMALL / 32) <= 227 * 1024;
+         smem_design64(a.n_max, a.p, a.nc_max, a.nrays, D64_SMALL / 32, false) <= 227 * 1024;
 }
 
 cudaError_t launch_design_fp64(const DesignArgs& a, int search, cudaStream_t s,
@@ -766,7 +766,7 @@ cudaError_t launch_design_fp64(const DesignArgs& a, int search, cudaStream_t s,
   int warps = a.nrays < 4 ? 4 : (a.nrays < D64_WARPS ? a.nrays : D64_WARPS);
   if (search == SEARCH_EXHAUSTIVE)
     warps = d64_small_batch(a, list != nullptr) ? D64_SMALL / 32 : D64_WARPS;
-  size_t sm = smem_design64(a.n_max, a.p, a.nc_max, a.nrays, warps);
+  size_t sm = smem_design64(a.n_max, a.p, a.nc_max, a.nrays, warps, a.full_scope != 0);
   const int64_t grid = list ? (a.M < grid_cap ? a.M : grid_cap) : a.M;
   if (grid <= 0) return cudaSuccess;
   cudaError_t err;

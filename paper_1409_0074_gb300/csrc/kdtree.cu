@@ -243,7 +243,7 @@ __global__ void kd_up(int level, int p, int PP, float* __restrict__ box32,
 cudaError_t launch_kd_build(const double* X, const float* Xf, const double* lo, const double* hi,
                             int64_t N, int p, int PP, const KdTree& t, cudaStream_t s) {
   const int D = t.D;
-  if ((D + KD_FAN - 1) / KD_FAN * 32 > KD_STACK) return cudaErrorInvalidValue;
+  if ((D + KD_FAN - 1) / KD_FAN > KD_STACK) return cudaErrorInvalidValue;
   const int nblk = rs_blocks(N);
   const unsigned g = (unsigned)((N + 255) / 256 < 4096 ? (N + 255) / 256 : 4096);
   prof_begin("kd_build", s);

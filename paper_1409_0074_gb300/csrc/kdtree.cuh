@@ -33,9 +33,13 @@ namespace lagp {
 
 #define KD_LEAF 32
 #define KD_FAN 5
-// one row of 32 box distances per visit in progress: ceil(D / KD_FAN) of them,
-// D <= 26 (int32 design indices)
-#define KD_STACK 192
+// visits in progress, each with its first descendant and a row of 32 box
+// distances: ceil(D / KD_FAN) of them, D <= 26 (int32 design indices).  (A word
+// per box distance for the descendants too was 384 words of every warp of the ray
+// kernel, also where no walk runs: with one ray, n = 64 and N' = 1000 that left 18
+// instead of 20 warps per SM, 28.4 against 26.8 ms per 20,000 locations.)
+#define KD_STACK 6
+#define KD_BOUNDS (32 * KD_STACK)
 
 __host__ __device__ inline int kd_depth(int64_t N) {
   int D = 0;
@@ -153,9 +157,9 @@ __device__ __forceinline__ double kd_warp_min(double v) {
 // allow_starts) says whether design point gi (at tree position pos) may not be
 // picked; with no allowed point at all the search repeats with the ray starts
 // allowed.  dist(pos, gi) and distx(pos, gi) give a point's squared distances
-// to x* and to x in the form's own arithmetic.  stk / bnd: KD_STACK entries
-// per warp (the first descendant of each visit in progress, and the
-// descendants' box distances).
+// to x* and to x in the form's own arithmetic.  stk / bnd: KD_STACK and
+// KD_BOUNDS entries per warp (the first descendant of each visit in progress, and
+// the descendants' box distances).
 template <bool TOP2, typename T, typename Excl, typename Dist, typename DistX>
 __device__ KdTop<T> kd_nearest(const KdView<T>& V, const T* xs, T margin, int* stk, T* bnd,
                                Excl excluded, Dist dist, DistX distx) {

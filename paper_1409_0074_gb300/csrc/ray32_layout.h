@@ -1,7 +1,8 @@
 // ray32_layout.h -- shared-memory layout of one warp (one location) of the
 // FP32-scoring ray kernel, and the index arithmetic of its row storage.  Free
 // of CUDA so that the host tests compile it; KD_STACK (the k-d tree walk's
-// stack depth) comes from kdtree.cuh, or from the compiler's command line.
+// visits in progress, 32 box distances each) comes from kdtree.cuh, or from the
+// compiler's command line.
 #pragma once
 
 #ifndef KD_STACK
@@ -64,7 +65,7 @@ LAGP_HDI WarpLayout warp_layout(int n, int PP, int RP, int nc) {
   // the factor update's two binary64 work vectors (n each) run after the
   // step's evaluations and reuse this space
   const int cbw = 2 * RP * kz_ld(n);
-  w.cb = take(cbw > 2 * KD_STACK ? cbw : 2 * KD_STACK);
+  w.cb = take(cbw > 33 * KD_STACK ? cbw : 33 * KD_STACK);
   w.stk = w.cb;
   w.bnd = w.cb + KD_STACK;
   w.zf = take((n + 3) & ~3);
