@@ -51,6 +51,13 @@ inline int warps_per_cta_for_residency(size_t warp_bytes, size_t smem_sm, size_t
   return best;
 }
 
+// Threads of a block of the local inference for the lengthscale (the results are
+// the same).  10,000 locations with 128 against 256: 13.6 and 25.2 ms at n = 2,
+// 10.3 and 18.4 at n = 10, 17.6 and 27.2 at n = 24; one location 0.56 and 0.70, 1.03
+// and 1.17, 0.79 and 0.82 ms.  From n = 28 on a single wave is faster with 256 (150
+// locations 2.63 against 2.65 ms, at n = 33 3.19 against 3.37).
+inline int mle_threads(int n) { return n <= 24 ? 128 : 256; }
+
 // Sample rows of the kNN pilot.
 inline int64_t knn_sample(int64_t N) { return N / 16 < 32768 ? N / 16 : 32768; }
 // The tensor-core filter, and the sizes below it whose stream may take a pilot

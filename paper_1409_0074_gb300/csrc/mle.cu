@@ -2,7 +2,7 @@
 // (Gramacy & Haaland, Sec 5: local designs are coupled with Newton-like
 // maximisation of the local posterior of theta; Sec 2.1, Eq. gpk), then the
 // predictive equations (Eq. predgp, preds2) at the estimate.  Binary64, one CTA
-// of 256 threads per predictive location, the local matrices in shared memory
+// of 256 threads (128 up to n = 24) per predictive location, the local matrices in shared memory
 // (n <= 64).
 //
 // Objective (readings M1, M2): the log marginal likelihood of Eq. gpk with the
@@ -32,6 +32,8 @@
 // On the gridded 2-d experiment (n = 50, two stages of 9,801 locations) the
 // kernel takes 103.3 ms against 201.2 ms with 128 threads, the factor by
 // left-looking columns and both triangles; the pipe is 83% busy (66% before).
+// Small designs leave most of 256 threads idle at the barriers and halve the
+// blocks on an SM: up to n = 24 a block has 128 threads (mle_threads).
 //
 // Maximiser (reading M3): Newton's method from theta0, safeguarded by a bracket
 // [a, b] kept from the sign of l'; a step outside the bracket, or taken where
@@ -47,8 +49,6 @@
 
 namespace lagp {
 
-#define MLE_THREADS 256
-#define MLE_WARPS (MLE_THREADS / 32)
 #define MLE_SUM 128        // threads whose partial sums make up a block sum
 #define MLE_SUM_WARPS (MLE_SUM / 32)
 #define MLE_NMAX 64
@@ -117,7 +117,7 @@ __device__ __forceinline__ void mle_pivot(int n, int k, double* Cm, int* flag) {
 // Log-likelihood (without its theta-free constant) and derivatives at theta
 // (FULL; else K^{-1}, alpha and psi only).  Leaves C (Cholesky factor, lower
 // triangle; K'' above it), Ki = K^{-1} and al = K^{-1} y.
-template <bool FULL>
+template <int THREADS, bool FULL>
 __device__ MleEval mle_eval(int n, double theta, double g, const double* D, const double* y,
                             double* Cm, double* Ki, double* K1, double* A, double* al,
                             double* u, double* red, int* flag) {
@@ -128,7 +128,7 @@ __device__ MleEval mle_eval(int n, double theta, double g, const double* D, cons
   r.ok = false;
   r.ll = r.d1 = r.d2 = r.psi = 0.0;
   const double c2 = 2.0 / theta;
-  for (int e = tid; e < np; e += MLE_THREADS) {
+  for (int e = tid; e < np; e += THREADS) {
     int a, b;
     mle_pair(e, &a, &b);
     const int lo = a * n + b, up = b * n + a;
@@ -163,7 +163,7 @@ __device__ MleEval mle_eval(int n, double theta, double g, const double* D, cons
       if (k + 1 < n) mle_pivot(n, k + 1, Cm, flag);
     } else {
       // row i > k: C^{-1} up to column k, C right of it
-      for (int i = k + warp; i < n; i += MLE_WARPS - 1) {
+      for (int i = k + warp; i < n; i += THREADS / 32 - 1) {
         const double m = -Cm[i * n + k];
         for (int x = lane; x < i; x += 32) {
           double* t = (x <= k ? A : Cm) + i * n + x;
@@ -175,7 +175,7 @@ __device__ MleEval mle_eval(int n, double theta, double g, const double* D, cons
   }
   if (*flag) return r;
   // K^{-1} = C^{-T} C^{-1}
-  for (int e = tid; e < np; e += MLE_THREADS) {
+  for (int e = tid; e < np; e += THREADS) {
     int i, j;
     mle_pair(e, &i, &j);
     double t = 0.0;
@@ -188,7 +188,7 @@ __device__ MleEval mle_eval(int n, double theta, double g, const double* D, cons
   double ld = 0.0;
   if (FULL && tid < MLE_SUM)
     for (int j = tid; j < n; j += MLE_SUM) ld += log(Cm[j * n + j]);
-  for (int i = tid; i < n; i += MLE_THREADS) {
+  for (int i = tid; i < n; i += THREADS) {
     double t = 0.0;
     for (int k = 0; k < n; ++k) t = fma(Ki[i * n + k], y[k], t);
     al[i] = t;
@@ -203,13 +203,13 @@ __device__ MleEval mle_eval(int n, double theta, double g, const double* D, cons
   r.ok = psi > 0.0;
   if (!FULL) return r;
   // A = K^{-1} K' (overwrites C^{-1}); u = K' alpha
-  for (int e = tid; e < nn; e += MLE_THREADS) {
+  for (int e = tid; e < nn; e += THREADS) {
     const int i = e / n, j = e - i * n;
     double t = 0.0;
     for (int k = 0; k < n; ++k) t = fma(Ki[i * n + k], K1[k * n + j], t);
     A[e] = t;
   }
-  for (int i = MLE_THREADS - 1 - tid; i < n; i += MLE_THREADS) {
+  for (int i = THREADS - 1 - tid; i < n; i += THREADS) {
     double t = 0.0;
     for (int k = 0; k < n; ++k) t = fma(K1[i * n + k], al[k], t);
     u[i] = t;
@@ -243,7 +243,9 @@ __device__ MleEval mle_eval(int n, double theta, double g, const double* D, cons
   return r;
 }
 
-__global__ void __launch_bounds__(MLE_THREADS, 2) mle_kernel(MleParams P) {
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 128 ? 6 : 2)
+mle_kernel(MleParams P) {
   extern __shared__ __align__(16) double sm[];
   __shared__ double red[MLE_SUM_WARPS];
   __shared__ int flag;
@@ -261,20 +263,20 @@ __global__ void __launch_bounds__(MLE_THREADS, 2) mle_kernel(MleParams P) {
   const int32_t* sl = P.sel + loc * n;
   if (tid == 0) flag = 0;
   __syncthreads();
-  for (int e = tid; e < n * p; e += MLE_THREADS) {
+  for (int e = tid; e < n * p; e += THREADS) {
     const int i = e / p, k = e - i * p;
     const int32_t gi = sl[i];
     if (gi < 0 || gi >= P.N) { flag = 1; S[e] = 0.0; continue; }
     S[e] = P.X[(int64_t)gi * p + k];
   }
-  for (int i = tid; i < n; i += MLE_THREADS) {
+  for (int i = tid; i < n; i += THREADS) {
     const int32_t gi = sl[i];
     y[i] = (gi >= 0 && gi < P.N) ? P.Y[gi] : 0.0;
   }
   __syncthreads();
   const bool bad_index = flag != 0;
   __syncthreads();
-  for (int e = tid; e < n * n; e += MLE_THREADS) {
+  for (int e = tid; e < n * n; e += THREADS) {
     const int a = e / n, b = e - a * n;
     D[e] = sqdist64(S + a * p, S + b * p, p);
   }
@@ -287,7 +289,7 @@ __global__ void __launch_bounds__(MLE_THREADS, 2) mle_kernel(MleParams P) {
   bool ok = !bad_index;
   while (ok && it < P.maxit) {
     ++it;
-    const MleEval e = mle_eval<true>(n, t, P.g, D, y, Cm, Ki, K1, A, al, u, red, &flag);
+    const MleEval e = mle_eval<THREADS, true>(n, t, P.g, D, y, Cm, Ki, K1, A, al, u, red, &flag);
     __syncthreads();
     if (!e.ok || !(e.ll == e.ll) || !(e.d1 == e.d1)) break;
     if (e.d1 > 0.0) lo = t; else hi = t;
@@ -301,12 +303,12 @@ __global__ void __launch_bounds__(MLE_THREADS, 2) mle_kernel(MleParams P) {
   // predictive equations at the estimate
   double mu = 0.0, s2 = 0.0;
   if (ok) {
-    const MleEval e = mle_eval<false>(n, t, P.g, D, y, Cm, Ki, K1, A, al, u, red, &flag);
+    const MleEval e = mle_eval<THREADS, false>(n, t, P.g, D, y, Cm, Ki, K1, A, al, u, red, &flag);
     __syncthreads();
     ok = e.ok;
     if (ok) {
       const double* x = P.xref + loc * p;
-      for (int i = tid; i < n; i += MLE_THREADS) {
+      for (int i = tid; i < n; i += THREADS) {
         const double d = sqdist64(S + i * p, x, p);
         u[i] = exp_neg_fma(-(d / t));
       }
@@ -354,11 +356,12 @@ cudaError_t launch_mle(const double* X, const double* Y, int64_t N, int p, const
   P.tol = 1e-10; P.maxit = 200;
   P.theta_out = theta_out; P.mean = mean; P.s2 = s2; P.iters = iters; P.status = status;
   const size_t sm = mle_smem(n, p);
-  cudaError_t e = cudaFuncSetAttribute(mle_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sm);
+  const int threads = mle_threads(n);
+  auto k = threads == 128 ? mle_kernel<128> : mle_kernel<256>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   prof_begin("mle_theta", s);
-  mle_kernel<<<(unsigned)M, MLE_THREADS, sm, s>>>(P);
+  k<<<(unsigned)M, threads, sm, s>>>(P);
   prof_end(s);
   return cudaGetLastError();
 }

@@ -1,0 +1,30 @@
+"""Which form of a kernel a call takes (csrc/launch_plan.h), compiled with the host
+C++ compiler and checked on the CPU against the sides that were measured."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(HERE, "..", "paper_1409_0074_gb300", "csrc")
+
+
+def values(tmp_path, expressions):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        pytest.skip("no host C++ compiler")
+    src, exe = tmp_path / "rule.cpp", tmp_path / "rule"
+    body = "".join('  std::printf("%%lld\\n", (long long)(%s));\n' % e for e in expressions)
+    src.write_text('#include <cstdio>\n#include "launch_plan.h"\nusing namespace lagp;\n'
+                   "int main() {\n%s}\n" % body)
+    subprocess.run([cxx, "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout
+    return [int(v) for v in out.split()]
+
+
+def test_local_inference_of_small_designs_takes_small_blocks(tmp_path):
+    """With 256 threads, 10,000 designs of 2 to 10 points took 1.4 to 1.75 times
+    as long as with 128."""
+    got = values(tmp_path, ["mle_threads(%d)" % n for n in (1, 2, 10, 24, 28, 50, 64)])
+    assert got == [128, 128, 128, 128, 256, 256, 256]
