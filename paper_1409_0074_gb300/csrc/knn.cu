@@ -515,8 +515,9 @@ knn_stream(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N
 // their binary64 distance and are ranked within their run by counting.  The
 // bound grows with the distance, so the cut between two runs separates
 // everything below from everything above.  Runs longer than RANK_RUN (designs
-// with many equal distances) and values that leave binary32's range sort all the
-// (binary64 distance, index) pairs instead; both give the one order.  100,000
+// with many equal distances) then sort all the (distance, index) pairs, the members
+// of runs by their binary64 distances; values that leave binary32's range sort the
+// (binary64 distance, index) pairs at once; all give the one order.  100,000
 // locations, p = 8, N' = 1000: 3.33 ms, 6.12 with all distances in binary64;
 // 10,000 locations, p = 4, N' = 200: 0.06 against 0.42 ms (a network of 1024
 // whatever the list's length).
@@ -526,21 +527,22 @@ knn_stream(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N
 // the lanes of a warp by shuffles, the largest through shared memory.  Distances
 // are non-negative, so their IEEE bit patterns order like the values.
 // ---------------------------------------------------------------------------
-#define RANK_THREADS 256
 #define RANK_RUN 64
-#define RANK_MAX (8 * RANK_THREADS)
 
-// Sorts the RANK_THREADS * E words (WIDE: pairs of a word and an index) in kr
-// (and ir); key and idx: shared memory for as many entries.
-template <int E, bool WIDE>
+// Sorts the T * E words (WIDE: pairs of a word and an index) in kr (and ir); key
+// and idx: shared memory for as many entries.  With one element per thread only
+// the first `size` of them (a power of two) go through the network; the others
+// are the largest word.
+template <int T, int E, bool WIDE>
 __device__ __forceinline__ void rank_sort(unsigned long long (&kr)[E], int32_t (&ir)[E],
-                                          unsigned long long* key, int32_t* idx) {
+                                          unsigned long long* key, int32_t* idx, int size) {
   const int t = threadIdx.x;
+  const int last = E == 1 ? size : T * E;
   auto less = [](unsigned long long ka, int32_t ia, unsigned long long kb, int32_t ib) {
     return WIDE ? (ka < kb || (ka == kb && ia < ib)) : ka < kb;
   };
 #pragma unroll 1
-  for (int k = 2; k <= RANK_THREADS * E; k <<= 1) {
+  for (int k = 2; k <= last; k <<= 1) {
 #pragma unroll 1
     for (int jj = k >> 1; jj >= E; jj >>= 1) {
       const int x = jj / E, pt = t ^ x;    // the partner thread, same u
@@ -548,8 +550,8 @@ __device__ __forceinline__ void rank_sort(unsigned long long (&kr)[E], int32_t (
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < E; ++u) {
-          key[u * RANK_THREADS + t] = kr[u];
-          if (WIDE) idx[u * RANK_THREADS + t] = ir[u];
+          key[u * T + t] = kr[u];
+          if (WIDE) idx[u * T + t] = ir[u];
         }
         __syncthreads();
       }
@@ -562,8 +564,8 @@ __device__ __forceinline__ void rank_sort(unsigned long long (&kr)[E], int32_t (
         unsigned long long pk;
         int32_t pi = 0;
         if (x >= 32) {
-          pk = key[u * RANK_THREADS + pt];
-          if (WIDE) pi = idx[u * RANK_THREADS + pt];
+          pk = key[u * T + pt];
+          if (WIDE) pi = idx[u * T + pt];
         } else {
           pk = __shfl_xor_sync(0xffffffffu, kr[u], x);
           if (WIDE) pi = __shfl_xor_sync(0xffffffffu, ir[u], x);
@@ -600,18 +602,19 @@ __device__ __forceinline__ float rank_err(float d, float qn, int p) {
   return 1.25f * u * (2.f * r * s + (float)(p + 4) * d) + 4.f * (u * s) * (u * s) + 1e-36f;
 }
 
+template <int MAX>
 struct RankRuns {
-  uint32_t joined[RANK_MAX / 32];   // bit i: element i joins i - 1
-  uint16_t list[RANK_MAX];          // the members of runs
+  uint32_t joined[MAX / 32];   // bit i: element i joins i - 1
+  uint16_t list[MAX];          // the members of runs
   int nlist;
 };
 
-// c <= RANK_THREADS * E survivors, at least nc of them
-template <int E>
+// c <= T * E survivors, at least nc of them
+template <int T, int E, typename Runs>
 __device__ void rank_location(const double* __restrict__ X, const float* __restrict__ Xf, int p,
                               int PP, const double* xq, const float* qf, float qn,
                               const KnnEntry* __restrict__ e, int c, int nc,
-                              unsigned long long* key, int32_t* idx, RankRuns& runs,
+                              unsigned long long* key, int32_t* idx, Runs& runs,
                               int32_t* __restrict__ out) {
   uint32_t* joined = runs.joined;
   uint16_t* list = runs.list;
@@ -641,10 +644,13 @@ __device__ void rank_location(const double* __restrict__ X, const float* __restr
       kr[u] = ((unsigned long long)__float_as_uint(d) << 32) | (uint32_t)gi;
     }
   }
-  if (t < RANK_THREADS * E / 32) joined[t] = 0u;
+  int size = T;                        // (E > 1: the whole network)
+  if (E == 1)
+    while (size > 2 && size / 2 >= c) size >>= 1;
+  if (t < T * E / 32) joined[t] = 0u;
   if (t == 0) runs.nlist = 0;
   if (!__syncthreads_or(wide || !(qn < 1e18f))) {
-    rank_sort<E, false>(kr, ir, key, idx);
+    rank_sort<T, E, false>(kr, ir, key, idx, size);
 #pragma unroll
     for (int u = 0; u < E; ++u) {
       key[E * t + u] = kr[u];
@@ -672,12 +678,12 @@ __device__ void rank_location(const double* __restrict__ X, const float* __restr
     }
     __syncthreads();
     const int nl = runs.nlist;
-    for (int l = t; l < nl; l += RANK_THREADS) {
+    for (int l = t; l < nl; l += T) {
       const int i = list[l];
       key[i] = (unsigned long long)__double_as_longlong(sqdist64(X + (int64_t)idx[i] * p, xq, p));
     }
     __syncthreads();
-    for (int l = t; l < nl; l += RANK_THREADS) {
+    for (int l = t; l < nl; l += T) {
       const int i = list[l];
       int a = i, b = i + 1;
       while (b - a <= RANK_RUN && joins(a)) --a;
@@ -689,24 +695,38 @@ __device__ void rank_location(const double* __restrict__ X, const float* __restr
       if (at < nc) out[at] = idx[i];
     }
     if (!__syncthreads_or(wide)) return;
-  }
+    // a run too long: all pairs, the members of runs with the distances they have
+    // and the others with the binary32 one, which is on the right side of every cut
 #pragma unroll
-  for (int u = 0; u < E; ++u) {
-    const int i = E * t + u;
-    kr[u] = ~0ull;
-    ir[u] = 0x7fffffff;
-    if (i < c) {
-      ir[u] = e[i].idx;
-      kr[u] = (unsigned long long)__double_as_longlong(sqdist64(X + (int64_t)ir[u] * p, xq, p));
+    for (int u = 0; u < E; ++u) {
+      const int i = E * t + u;
+      ir[u] = i < c ? (int32_t)(uint32_t)kr[u] : 0x7fffffff;
+      if (joins(i) || joins(i + 1)) kr[u] = key[i];
+      else if (i < c)
+        kr[u] = (unsigned long long)__double_as_longlong((double)__uint_as_float((uint32_t)(kr[u] >> 32)));
+    }
+    __syncthreads();
+  } else {
+#pragma unroll
+    for (int u = 0; u < E; ++u) {
+      const int i = E * t + u;
+      kr[u] = ~0ull;
+      ir[u] = 0x7fffffff;
+      if (i < c) {
+        ir[u] = e[i].idx;
+        kr[u] = (unsigned long long)__double_as_longlong(sqdist64(X + (int64_t)ir[u] * p, xq, p));
+      }
     }
   }
-  rank_sort<E, true>(kr, ir, key, idx);
+  rank_sort<T, E, true>(kr, ir, key, idx, size);
 #pragma unroll
   for (int u = 0; u < E; ++u)
     if (E * t + u < nc) out[E * t + u] = ir[u];
 }
 
-__global__ void __launch_bounds__(RANK_THREADS, 4)
+// T = 256 threads for lists of any length; T = 128 for short ones (rank_threads)
+template <int T>
+__global__ void __launch_bounds__(T, T == 128 ? 12 : 4)
 knn_rank(const double* __restrict__ X, const float* __restrict__ Xf, int p, int PP,
          const double* __restrict__ xref, const double* __restrict__ center, int64_t M,
          int nc_max, const int32_t* __restrict__ nc_loc, int cap,
@@ -722,21 +742,24 @@ knn_rank(const double* __restrict__ X, const float* __restrict__ Xf, int p, int 
   int32_t* out = cand + q * nc_max;
   __shared__ double xq[LAGP_MAX_P];
   __shared__ float qf[LAGP_MAX_P];
-  __shared__ RankRuns runs;
+  constexpr int MAX = T == 128 ? 512 : 2048;
+  __shared__ RankRuns<MAX> runs;
   if (threadIdx.x < p) xq[threadIdx.x] = xref[q * p + threadIdx.x];
   if (threadIdx.x < PP)
     qf[threadIdx.x] =
         threadIdx.x < p ? (float)(xref[q * p + threadIdx.x] - center[threadIdx.x]) : 0.f;
   __syncthreads();
   const KnnEntry* e = buf + q * (int64_t)cap;
-  if (c >= nc && c <= RANK_MAX) {
+  if (c >= nc && c <= MAX) {
     float qn = 0.f;
     for (int k = 0; k < p; ++k) qn = fmaf(qf[k], qf[k], qn);
     qn = sqrtf(qn) * 1.0001f;
-    if (c <= 256) rank_location<1>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
-    else if (c <= 512) rank_location<2>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
-    else if (c <= 1024) rank_location<4>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
-    else rank_location<8>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
+    if (c <= T) rank_location<T, 1>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
+    else if (c <= 2 * T) rank_location<T, 2>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
+    else if (T == 128 || c <= 4 * T)
+      rank_location<T, 4>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
+    else
+      rank_location<T, MAX / T>(X, Xf, p, PP, xq, qf, qn, e, c, nc, key, idx, runs, out);
     for (int r = nc + threadIdx.x; r < nc_max; r += blockDim.x) out[r] = -1;
     return;
   }
@@ -879,10 +902,12 @@ cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
       return cudaErrorInvalidValue;
   }
   size_t smr = (size_t)cap * (8 + 4);
-  err = cudaFuncSetAttribute(knn_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
+  const int threads = rank_threads(nc_max);
+  auto rank = threads == 128 ? knn_rank<128> : knn_rank<256>;
+  err = cudaFuncSetAttribute(rank, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smr);
   if (err != cudaSuccess) return err;
   prof_begin("knn_rank", s);
-  knn_rank<<<(unsigned)M, RANK_THREADS, smr, s>>>(
+  rank<<<(unsigned)M, threads, smr, s>>>(
       X, ws.Xf, p, PP, xref, ws.center, M, nc_max, nc_loc, cap,
       reinterpret_cast<const KnnEntry*>(ws.knn_buf), ws.knn_cnt, cand, ws.status);
   prof_end(s);

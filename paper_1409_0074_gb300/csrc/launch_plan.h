@@ -58,6 +58,13 @@ inline int warps_per_cta_for_residency(size_t warp_bytes, size_t smem_sm, size_t
 // locations 2.63 against 2.65 ms, at n = 33 3.19 against 3.37).
 inline int mle_threads(int n) { return n <= 24 ? 128 : 256; }
 
+// Threads of a block of the exact ranking.  A short list is a chain of latencies
+// that more blocks per SM hide, and its network is short: 20,000 locations at p = 4
+// take 0.049 ms with 128 threads and 0.178 with 256 and a network of 256 at N' = 30,
+// 0.070 and 0.186 at N' = 100; at N' = 200 0.147 and 0.184, but one location there
+// 10.1 us and 8.2.
+inline int rank_threads(int nc_max) { return nc_max <= 128 ? 128 : 256; }
+
 // Sample rows of the kNN pilot.
 inline int64_t knn_sample(int64_t N) { return N / 16 < 32768 ? N / 16 : 32768; }
 // The tensor-core filter, and the sizes below it whose stream may take a pilot

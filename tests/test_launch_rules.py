@@ -28,3 +28,9 @@ def test_local_inference_of_small_designs_takes_small_blocks(tmp_path):
     as long as with 128."""
     got = values(tmp_path, ["mle_threads(%d)" % n for n in (1, 2, 10, 24, 28, 50, 64)])
     assert got == [128, 128, 128, 128, 256, 256, 256]
+
+
+def test_short_lists_are_ranked_by_small_blocks(tmp_path):
+    """With 256 threads and a network of 256, lists of 30 took twice as long."""
+    got = values(tmp_path, ["rank_threads(%d)" % n for n in (1, 30, 100, 128, 200, 1000, 4096)])
+    assert got == [128, 128, 128, 128, 256, 256, 256]
