@@ -272,9 +272,9 @@ knn_pilot(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N,
   }
 }
 
-// The same thresholds for a small batch: one block per location instead of one
-// per 32 locations, whose two passes over the sample a lone location waits for
-// (0.65 ms at S = 32768).  Every thread keeps its at most 32 distances in
+// The same thresholds for a small batch (knn_pilot_alone): one block per location
+// instead of one per 32 locations, whose two passes over the sample a lone location
+// waits for (0.65 ms at S = 32768).  Every thread keeps its at most 32 distances in
 // registers; the bin of the m-th smallest comes from 16 halvings of the 16-bit
 // bin number by counting: 0.058 ms for one location, 0.36 ms for 1,024.
 #define KNN_PILOT1_THREADS 1024
@@ -850,12 +850,12 @@ cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
   const bool tc = knn_uses_tc(N, nc_max), pilot = knn_has_pilot(N, M, nc_max);
   const int64_t S = knn_sample(N);
   KnnEntry* kbuf = reinterpret_cast<KnnEntry*>(ws.knn_buf);
-  // a batch of a few locations per SM: one pilot block each (per wave of two
-  // blocks per SM about 0.025 ms, 0.05 at S = 32768; the shared form takes its
-  // two passes over the sample whatever the batch: 0.06 ms at S = 2500, 0.61
-  // at S = 32768, p = 8)
-  const bool small = M <= 304 || (M <= 1024 && S >= 16384);
   cudaError_t err;
+  int dev = 0, sms = 0;
+  if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
+  if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+    return err;
+  const bool alone = knn_pilot_alone(M, S, PP, sms);
   switch (PP) {
 #define KNN_CASE(V)                                                                          \
   case V:                                                                                    \
@@ -864,7 +864,7 @@ cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
     if (err != cudaSuccess) return err;                                                      \
     if (pilot) {                                                                             \
       prof_begin("knn_pilot", s);                                                            \
-      if (small)                                                                             \
+      if (alone)                                                                             \
         knn_pilot1<V><<<(unsigned)M, KNN_PILOT1_THREADS, 0, s>>>(                            \
             ws.Xf, ws.nx, N, S, p, xref, M, ws.center, nc_max, nc_loc, cap, ws.knn_thr);     \
       else                                                                                   \

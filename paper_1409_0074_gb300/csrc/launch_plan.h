@@ -72,6 +72,17 @@ inline int64_t knn_sample(int64_t N) { return N / 16 < 32768 ? N / 16 : 32768; }
 inline bool knn_uses_tc(int64_t N, int nc_max) { return N >= (int64_t)32 * nc_max; }
 inline bool knn_mid(int64_t N, int nc_max) { return N >= (int64_t)4 * nc_max && N >= 1024; }
 
+// Whether the pilot takes a block per location (knn_pilot1) instead of one per 32
+// (knn_pilot), of S sample rows padded to PP coordinates: by the lines through what
+// both took, in microseconds.  A block per location: 23 for up to one location per
+// SM at S = 68 (p = 4), 31 at 6,250 (p = 8), 57 at 32,768, and for two per SM 41, 57
+// and 109.  A block per 32: 12 at S = 68, 26 at 1,250 and 65 at 6,250 (p = 4), 35, 94
+// and (at 18,750) 287 at p = 8, for any batch of up to 32 locations per SM.
+inline bool knn_pilot_alone(int64_t M, int64_t S, int PP, int64_t sms) {
+  const double per_sm = (double)((M + sms - 1) / sms);
+  return 2.0 + per_sm * (21.0 + S / 960.0) < 9.0 + 0.75 * PP + S * (3.2 + 1.35 * PP) * 1e-3;
+}
+
 // Entries of a location's kNN candidate buffer.  It needs room for N'
 // survivors, a whole tile of 256 new inserts before the next compaction, and
 // N'/2 (at least 64) entries of slack for distances within the error margin of

@@ -34,3 +34,13 @@ def test_short_lists_are_ranked_by_small_blocks(tmp_path):
     """With 256 threads and a network of 256, lists of 30 took twice as long."""
     got = values(tmp_path, ["rank_threads(%d)" % n for n in (1, 30, 100, 128, 200, 1000, 4096)])
     assert got == [128, 128, 128, 128, 256, 256, 256]
+
+
+def test_pilot_takes_a_block_per_location_where_that_was_faster(tmp_path):
+    """(M, S, PP): a block per location lost at small samples (one location at
+    S = 68 23 against 12 us) and at many locations, and won at large samples."""
+    sides = {(1, 68, 4): 0, (32, 312, 4): 0, (300, 1875, 4): 0, (1000, 6250, 4): 0, (304, 1250, 8): 0,
+             (608, 6250, 8): 0, (10_000, 32768, 8): 0, (1, 1875, 4): 1, (300, 6250, 4): 1,
+             (152, 1250, 8): 1, (456, 6250, 8): 1, (1, 32768, 8): 1, (1024, 32768, 8): 1}
+    got = values(tmp_path, ["knn_pilot_alone(%d, %d, %d, 152)" % k for k in sides])
+    assert got == list(sides.values())
