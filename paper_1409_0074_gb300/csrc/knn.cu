@@ -165,15 +165,44 @@ __device__ __forceinline__ int64_t pilot_row(int64_t i, int64_t step) {
   return i * step + __umulhi((uint32_t)i * 2654435769u, (uint32_t)step);
 }
 
+__device__ __forceinline__ float pilot_err2(float errc, float nq, unsigned maxn2) {
+  const float r = (sqrtf(__uint_as_float(maxn2)) + sqrtf(nq)) * 1.0001f;
+  return 2.f * errc * r * r;
+}
+// Rows up to the threshold + err2 are counted by bins (2^-8 of an octave) where that
+// stays in the threshold's octave b1, and else by whole octaves: those up to the one
+// reached where err2 alone leads past b1 (pilot_past, 0 where it does not), else those
+// up to b1.
+__device__ __forceinline__ uint32_t pilot_past(uint32_t b1, float err2) {
+  const uint32_t e = __float_as_uint(__uint_as_float(b1 << 23) + err2) >> 23;
+  return e > b1 ? e + 1u : 0u;
+}
+// the first n of 256 counts, over the warp (lane l owning counts 8l..8l+7)
+__device__ __forceinline__ int pilot_count(const uint32_t* h, uint32_t n) {
+  const int lane = threadIdx.x & 31;
+  int c = 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) c += lane * 8 + u < (int)n ? (int)h[lane * 8 + u] : 0;
+  return __reduce_add_sync(0xffffffffu, c);
+}
+
 // Pilot thresholds: per location the upper edge of the 2^-8-wide bin (by the
 // float bit pattern: exponent, then the top 8 mantissa bits) that holds the
 // m-th smallest d32 of the S sample rows; +inf where the pilot
-// does not apply (m > S, or more than cap - 2 tiles expected below it).
-template <int PP>
+// does not apply (m > S, or more than cap - 2 tiles expected below it).  CHECK: nor
+// where the tensor-core filter, which admits up to the threshold + 2 err, err = errc
+// (|a| + |b|)^2, would admit too many, more than `fit` sample rows lying below that.
+// That is for strongly clustered designs, with buffers that are larger for the
+// threshold's sake: 20,000 points in 20 clusters that err spans, 5,000 locations,
+// N' = 30 took 1.11 ms with thresholds that admitted whole clusters, 0.51 streamed
+// from infinity with the smallest buffers, and take 0.58.  The check costs the
+// pilot 2 to 10% (1.50 to 1.62 ms for 40,000 locations, p = 4).
+template <int PP, bool CHECK>
 __global__ void __launch_bounds__(KNN_WARPS * 32)
 knn_pilot(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N, int64_t S, int p,
           const double* __restrict__ xref, int64_t M, const double* __restrict__ center,
-          int nc_max, const int32_t* __restrict__ nc_loc, int cap, float* __restrict__ thr_out) {
+          int nc_max, const int32_t* __restrict__ nc_loc, int cap, float errc, int fit,
+          const unsigned* __restrict__ maxn2_bits, float* __restrict__ thr_out) {
   // the sample rows pass through shared memory a tile at a time, shared by
   // the CTA's warps (each sample row is read from L2 once per CTA and pass);
   // a tile holds the rows' first four coordinates, then their next four, ...,
@@ -268,10 +297,22 @@ knn_pilot(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N,
       if (pass == 0) {
         const int b = warp_bin_of_kth(hist[warp][a], m[a] > 0 ? m[a] : 1, &below[a]);
         b1[a] = b < 0 ? 0u : (uint32_t)b;
+        if (CHECK) {
+          const uint32_t past = pilot_past(b1[a], pilot_err2(errc, nq[a], *maxn2_bits));
+          if (past && pilot_count(hist[warp][a], past) > fit) m[a] = 0;
+        }
       } else {
         int dummy = 0;
         const int b = warp_bin_of_kth(hist[warp][a], m[a] > 0 ? m[a] - below[a] : 1, &dummy);
         float thr = __uint_as_float((b1[a] << 23) | ((uint32_t)(b < 0 ? 255 : b) << 15) | 0x7fffu);
+        if (CHECK) {
+          const float err2 = pilot_err2(errc, nq[a], *maxn2_bits);
+          if (!pilot_past(b1[a], err2)) {
+            const uint32_t k = __float_as_uint(thr + err2) >> 15;
+            const uint32_t n = k >> 8 == b1[a] ? (k & 255u) + 1u : 256u;
+            if (below[a] + pilot_count(hist[warp][a], n) > fit) m[a] = 0;
+          }
+        }
         if (m[a] == 0 || b < 0 || !(thr < __int_as_float(0x7f800000))) thr = __int_as_float(0x7f800000);
         if (lane == 0 && q0 + a < M) thr_out[q0 + a] = thr;
       }
@@ -286,11 +327,12 @@ knn_pilot(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N,
 // registers; the bin of the m-th smallest comes from 16 halvings of the 16-bit
 // bin number by counting: 0.058 ms for one location, 0.36 ms for 1,024.
 #define KNN_PILOT1_THREADS 1024
-template <int PP>
+template <int PP, bool CHECK>
 __global__ void __launch_bounds__(KNN_PILOT1_THREADS)
 knn_pilot1(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N, int64_t S, int p,
            const double* __restrict__ xref, int64_t M, const double* __restrict__ center,
-           int nc_max, const int32_t* __restrict__ nc_loc, int cap, float* __restrict__ thr_out) {
+           int nc_max, const int32_t* __restrict__ nc_loc, int cap, float errc, int fit,
+           const unsigned* __restrict__ maxn2_bits, float* __restrict__ thr_out) {
   constexpr int T = 32768 / KNN_PILOT1_THREADS;    // S <= 32768
   __shared__ int cnt[2][KNN_PILOT1_THREADS / 32];
   const int64_t q = blockIdx.x;
@@ -340,10 +382,25 @@ knn_pilot1(const float* __restrict__ Xf, const float* __restrict__ nx, int64_t N
     c = __reduce_add_sync(0xffffffffu, cnt[bit & 1][lane]);
     if (c < m) b = mid + 1u;
   }
+  const float edge = __uint_as_float((b << 15) | 0x7fffu);
+  if (CHECK) {
+    const float err2 = pilot_err2(errc, nq, *maxn2_bits);
+    const uint32_t b1 = b >> 8, past = pilot_past(b1, err2);
+    const uint32_t k = __float_as_uint(edge + err2) >> 15;
+    const uint32_t lim = past ? past << 8 : (k >> 8 == b1 ? k + 1u : (b1 + 1u) << 8);
+    int c = 0;
+#pragma unroll
+    for (int u = 0; u < T; ++u) c += bin[u] < lim ? 1 : 0;
+    c = __reduce_add_sync(0xffffffffu, c);
+    __syncthreads();
+    if (lane == 0) cnt[0][warp] = c;
+    __syncthreads();
+    c = __reduce_add_sync(0xffffffffu, cnt[0][lane]);
+    if (c > fit) m = 0;
+  }
   if (tid == 0) {
     const float inf = __int_as_float(0x7f800000);
-    const float thr = __uint_as_float((b << 15) | 0x7fffu);
-    thr_out[q] = (m == 0 || !(thr < inf)) ? inf : thr;
+    thr_out[q] = (m == 0 || !(edge < inf)) ? inf : edge;
   }
 }
 
@@ -859,6 +916,11 @@ cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
   const bool tc = knn_uses_tc(N, nc_max), pilot = knn_has_pilot(N, M, nc_max);
   const int64_t S = knn_sample(N);
   KnnEntry* kbuf = reinterpret_cast<KnnEntry*>(ws.knn_buf);
+  // buffers that are larger for the threshold's sake: what the tensor-core filter
+  // may admit to them, in sample rows
+  const bool check = tc && cap > knn_cap_least(nc_max);
+  const float errc = kt_err_factor(kt_ka(p));
+  const int fit = (int)((cap - 2 * LAGP_KNN_TILE) * S / N);
   cudaError_t err;
   int dev = 0, sms = 0;
   if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
@@ -874,12 +936,15 @@ cudaError_t launch_knn(const double* X, int64_t N, int p, int PP, int64_t Npad,
     if (pilot) {                                                                             \
       prof_begin("knn_pilot", s);                                                            \
       if (alone)                                                                             \
-        knn_pilot1<V><<<(unsigned)M, KNN_PILOT1_THREADS, 0, s>>>(                            \
-            ws.Xf, ws.nx, N, S, p, xref, M, ws.center, nc_max, nc_loc, cap, ws.knn_thr);     \
+        (check ? knn_pilot1<V, true> : knn_pilot1<V, false>)                                 \
+            <<<(unsigned)M, KNN_PILOT1_THREADS, 0, s>>>(ws.Xf, ws.nx, N, S, p, xref, M,      \
+                                                        ws.center, nc_max, nc_loc, cap,      \
+                                                        errc, fit, ws.maxn2, ws.knn_thr);    \
       else                                                                                   \
-        knn_pilot<V><<<grid, KNN_WARPS * 32, 0, s>>>(ws.Xf, ws.nx, N, S, p, xref, M,         \
-                                                     ws.center, nc_max, nc_loc, cap,         \
-                                                     ws.knn_thr);                            \
+        (check ? knn_pilot<V, true> : knn_pilot<V, false>)                                   \
+            <<<grid, KNN_WARPS * 32, 0, s>>>(ws.Xf, ws.nx, N, S, p, xref, M, ws.center,      \
+                                             nc_max, nc_loc, cap, errc, fit, ws.maxn2,       \
+                                             ws.knn_thr);                                    \
       prof_end(s);                                                                           \
     }                                                                                        \
     if (tc) {                                                                                \

@@ -11,6 +11,13 @@ struct __align__(8) KnnEntry {
   int32_t idx;
 };
 
+// K of the tensor-core filter's contraction, and the bound on its distances' error
+// as a multiple of (|a| + |b|)^2 (knn_tc.cu)
+__host__ __device__ __forceinline__ int kt_ka(int p) { return (p + 2 + 7) & ~7; }
+__host__ __device__ __forceinline__ float kt_err_factor(int KA) {
+  return (float)(KA + 16) * 0x1p-21f * 1.25f;
+}
+
 // ---------------------------------------------------------------------------
 // Warp radix select: the k-th smallest (1-based) of cnt non-negative float
 // keys in e[0..cnt), returned as its bit pattern.  hist: 256 words of this

@@ -66,8 +66,6 @@ namespace lagp {
 #define KT_STAGES 6
 #define KT_EPI_BAR 1      // named barrier of the epilogue warps
 
-__host__ __device__ __forceinline__ int kt_ka(int p) { return (p + 2 + 7) & ~7; }
-
 // byte offset of (row, k) in the canonical no-swizzle K-major layout: 8-row x
 // 16-byte core matrices; the KA/4 k-chunks of a row group are adjacent (128
 // bytes apart), row groups KA/4 * 128 bytes apart.
@@ -81,9 +79,7 @@ __device__ __forceinline__ float kt_tf32(float v) {
   return __uint_as_float(r);
 }
 
-__device__ __forceinline__ float kt_err(int KA, float r) {
-  return (float)(KA + 16) * 0x1p-21f * 1.25f * r * r;
-}
+__device__ __forceinline__ float kt_err(int KA, float r) { return kt_err_factor(KA) * r * r; }
 
 // Design tiles [tile][hi | lo][KT_N rows x KA] in canonical order from the
 // centred FP32 copy: row i = [Xf_i, 1, |Xf_i|^2, 0..]; rows past N are

@@ -87,3 +87,20 @@ def test_gridded_designs(lagp, tmp_path, sides, nc, M):
         np.testing.assert_array_equal(cand[q], oracle.knn(Xh, Xr[q], nc)[0])
         below = (((Xh - Xr[q]) ** 2).sum(1) <= thr[q]).sum()
         assert nc <= below <= min(16 * (m + 6 * math.sqrt(m) + 8), N), (q, below)
+
+
+@pytest.mark.parametrize("M", [5, 3000])
+def test_clusters_within_the_filter_s_error(lagp, tmp_path, M):
+    """20 clusters of 1,000 points in a box whose filter error spans a cluster:
+    a threshold would admit the cluster, more than the room of 512 entries, so
+    there is none; on a uniform design there is. The lists are the oracle's."""
+    rng = np.random.default_rng(M)
+    N, p, nc = 20_000, 4, 30
+    cap, = values(tmp_path, ["knn_cap(%d, %d)" % (nc, N)])
+    Xh = rng.random((20, p))[np.arange(N) % 20] + 0.002 * rng.standard_normal((N, p))
+    Xr = Xh[rng.integers(0, N, M)] + 0.001 * rng.standard_normal((M, p))
+    cand, thr = search(lagp, to_dev(Xh), to_dev(Xr), nc, cap)
+    assert np.isinf(thr).mean() > 0.9
+    for q in range(0, M, max(1, M // 40)):
+        np.testing.assert_array_equal(cand[q], oracle.knn(Xh, Xr[q], nc)[0])
+    assert np.isfinite(search(lagp, to_dev(rng.random((N, p))), to_dev(Xr), nc, cap)[1]).all()
