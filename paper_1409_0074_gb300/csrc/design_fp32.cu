@@ -38,7 +38,8 @@
 // 25.7 against 35.0 ms per 20,000 locations (8-d, n = 50, N' = 1000) with the
 // factor in global memory, one lane per row and column and 32-bit loads.  Four
 // CTAs of 256 threads per SM keep the slots' caches near the size of L2: five
-// ran 26.8 ms, five or seven of 128 threads 26.8 and 34.1 ms.
+// ran 26.8 ms, five or seven of 128 threads 26.8 and 34.1 ms.  Up to N' = 512, where
+// the caches are small, most calls take eight of 128 threads (d32_threads).
 // Scoring coordinates are FP32 and centred on the design's bounding box.
 #include <cstdint>
 
@@ -47,8 +48,7 @@
 
 namespace lagp {
 
-#define D32_THREADS 256
-#define D32_WARPS (D32_THREADS / 32)
+#define D32_WARPS 8        // of the largest block (d32_threads)
 // row stride of the correlation cache and of the per-candidate arrays: four
 // candidates at a time
 #define D32_LDC(nc) (((nc) + 3) & ~3)
@@ -159,6 +159,7 @@ __device__ __forceinline__ VI vi_merge_max(VI a, VI b) {
   }
   return r;
 }
+template <int WARPS>
 __device__ VI block_best(VI t, float* fs, int* is) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int o = 16; o > 0; o >>= 1) {
@@ -171,7 +172,7 @@ __device__ VI block_best(VI t, float* fs, int* is) {
   if (lane == 0) { fs[2 * warp] = t.v; fs[2 * warp + 1] = t.v2; is[warp] = t.i; }
   __syncthreads();
   VI r; r.v = fs[0]; r.v2 = fs[1]; r.i = is[0];
-  for (int w = 1; w < D32_WARPS; ++w) {
+  for (int w = 1; w < WARPS; ++w) {
     VI u; u.v = fs[2 * w]; u.v2 = fs[2 * w + 1]; u.i = is[w];
     r = vi_merge_max(r, u);
   }
@@ -189,13 +190,14 @@ __device__ __forceinline__ const float* cand_f(const D32Params& P, const float* 
 // `best` receives this thread's part of the next search: the ALC of every
 // unselected candidate the thread updates, from the running sums it has just
 // written (the same arithmetic and candidate order as a separate pass).
+template <int THREADS>
 __device__ bool add_point32(const D32Params& P, L32& L, const int32_t* cl, const float* crow,
                             int nc, int r, double* Lg, float* Kc_loc, VI* best) {
   const int tid = threadIdx.x, p = P.p, j = L.j, warp = tid >> 5;
   const double* c = P.X + (int64_t)cl[r] * p;
   if (tid < p) L.S64[j * p + tid] = c[tid];
   if (tid < P.PP) L.Sf[j * P.PP + tid] = cand_f(P, crow, r)[tid];
-  if (tid == D32_THREADS - 1) {
+  if (tid == THREADS - 1) {
     L.ys[j] = P.Y[cl[r]];
     L.sel[j] = r;
     L.used[r] = 1;
@@ -203,7 +205,7 @@ __device__ bool add_point32(const D32Params& P, L32& L, const int32_t* cl, const
   __syncthreads();
   const double nit64 = d32_nit64;
   // correlations of the new point with the design, and with x (thread j)
-  for (int i = tid; i <= j; i += blockDim.x) {
+  for (int i = tid; i <= j; i += THREADS) {
     const double kv = corr64_fast(i < j ? L.S64 + i * p : L.xq, L.S64 + j * p, p, nit64);
     if (i < j) L.kvec[i] = kv;
     else L.kx[j] = kv;
@@ -211,7 +213,7 @@ __device__ bool add_point32(const D32Params& P, L32& L, const int32_t* cl, const
   __syncthreads();
   // l = L_j^{-1} k_j(x_new): four lanes per row, one for each of dot64_ilp's
   // accumulators (the first also takes the remainder)
-  for (int i = tid >> 2; i < ((j + 7) & ~7); i += D32_THREADS / 4) {
+  for (int i = tid >> 2; i < ((j + 7) & ~7); i += THREADS / 4) {
     const int t = tid & 3, len = i + 1, len4 = len & ~3;
     const double* Li = Lg + d32_tri(i);
     double acc = 0.0;
@@ -241,7 +243,7 @@ __device__ bool add_point32(const D32Params& P, L32& L, const int32_t* cl, const
   // row_j . y_S: two lanes per column, one for its even rows and one for its
   // odd ones (the sum's two accumulators, in either order)
   double* Lj = Lg + d32_tri(j);
-  for (int k = tid >> 1; k < ((j + 16) & ~15); k += D32_THREADS / 2) {
+  for (int k = tid >> 1; k < ((j + 16) & ~15); k += THREADS / 2) {
     const int h = tid & 1;
     double acc = 0.0;
     if (k < j) {
@@ -283,7 +285,7 @@ __device__ bool add_point32(const D32Params& P, L32& L, const int32_t* cl, const
   const float zj = L.zf[j];
   VI b;
   b.v = -1.f; b.v2 = -1.f; b.i = -1;
-  for (int q = 4 * tid; q < nc; q += 4 * blockDim.x) {
+  for (int q = 4 * tid; q < nc; q += 4 * THREADS) {
     float kv[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -357,8 +359,9 @@ __device__ bool add_point32(const D32Params& P, L32& L, const int32_t* cl, const
 // ALC_c = (w_c . z - K(c, x))^2 / ((1 + g) - |w_c|^2) from the running sums;
 // the largest score wins, ties to the lower candidate rank.  Each thread's part
 // comes from the update loop of the last appended point (add_point32).
+template <int THREADS>
 __device__ int search_exh32(const L32& L, VI best, double* gap_out) {
-  VI b = block_best(best, L.red, L.ired);
+  VI b = block_best<THREADS / 32>(best, L.red, L.ired);
   *gap_out = (b.v > 0.f && b.v2 >= 0.f) ? (double)((b.v - b.v2) / b.v) : 0.0;
   return b.i;
 }
@@ -366,9 +369,9 @@ __device__ int search_exh32(const L32& L, VI best, double* gap_out) {
 // PROMOTE: with precision promotion (a separate instantiation, so that the
 // default one carries none of its code)
 // SFACTOR: the packed factor in shared memory (d32_smem_factor), else in the
-// slot's global scratch
-template <bool PROMOTE, bool SFACTOR>
-__global__ void __launch_bounds__(D32_THREADS, 4) design32(D32Params P) {
+// slot's global scratch.  THREADS: 256 or 128 (d32_threads), 1,024 per SM.
+template <bool PROMOTE, bool SFACTOR, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) design32(D32Params P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned s_item;
   const int tid = threadIdx.x, p = P.p, PP = P.PP, ld = P.n_max;
@@ -429,16 +432,16 @@ __global__ void __launch_bounds__(D32_THREADS, 4) design32(D32Params P) {
 
     if (tid < p) L.xq[tid] = P.xref[loc * p + tid];
     if (tid < PP) L.xf[tid] = tid < p ? (float)(P.xref[loc * p + tid] - P.center[tid]) : 0.f;
-    if (P.tie_gap) for (int i = tid; i < ld; i += blockDim.x) P.tie_gap[loc * ld + i] = 0.0;
-    if (P.nevals) for (int i = tid; i < ld; i += blockDim.x) P.nevals[loc * ld + i] = 0;
+    if (P.tie_gap) for (int i = tid; i < ld; i += THREADS) P.tie_gap[loc * ld + i] = 0.0;
+    if (P.nevals) for (int i = tid; i < ld; i += THREADS) P.nevals[loc * ld + i] = 0;
     // the candidates' FP32 rows, gathered once into the slot in rank order
-    for (int e = tid; e < nc * (PP >> 2); e += blockDim.x) {
+    for (int e = tid; e < nc * (PP >> 2); e += THREADS) {
       const int q = e / (PP >> 2), c4 = (e - q * (PP >> 2)) << 2;
       *reinterpret_cast<float4*>(crow + (int64_t)q * PP + c4) =
           *reinterpret_cast<const float4*>(P.Xf + (int64_t)cl[q] * PP + c4);
     }
     __syncthreads();
-    for (int r = tid; r < nc; r += blockDim.x) {
+    for (int r = tid; r < nc; r += THREADS) {
       L.used[r] = 0;
       L.vs[r] = 0.f;
       L.ns[r] = 0.f;
@@ -448,19 +451,19 @@ __global__ void __launch_bounds__(D32_THREADS, 4) design32(D32Params P) {
 
     bool ok = (n >= P.n0) && (n <= nc) && (n <= ld);
     VI part;
-    for (int r = 0; r < P.n0 && ok; ++r) ok = add_point32(P, L, cl, crow, nc, r, Lg, Kc_loc, &part);
+    for (int r = 0; r < P.n0 && ok; ++r) ok = add_point32<THREADS>(P, L, cl, crow, nc, r, Lg, Kc_loc, &part);
     for (int j = P.n0; j < n && ok; ++j) {
       double gap = 0.0;
       int ne = 0;
-      int r = search_exh32(L, part, &gap);
+      int r = search_exh32<THREADS>(L, part, &gap);
       if (tid == 0) {
         if (P.tie_gap) P.tie_gap[loc * ld + (j - P.n0)] = gap;
         if (P.nevals) P.nevals[loc * ld + (j - P.n0)] = ne;
       }
-      ok = (r >= 0) && add_point32(P, L, cl, crow, nc, r, Lg, Kc_loc, &part);
+      ok = (r >= 0) && add_point32<THREADS>(P, L, cl, crow, nc, r, Lg, Kc_loc, &part);
     }
     if (ok) {
-      for (int i = tid; i < L.j; i += blockDim.x) L.tz[i] = __dmul_rn(L.z[i], L.zy[i]);
+      for (int i = tid; i < L.j; i += THREADS) L.tz[i] = __dmul_rn(L.z[i], L.zy[i]);
       __syncthreads();
       if (tid < 32) {
         const double a = sum_vector32(L.tz, L.j), b = sum_squares32(L.zy, L.j);
@@ -476,7 +479,7 @@ __global__ void __launch_bounds__(D32_THREADS, 4) design32(D32Params P) {
       atomicOr(P.status, LAGP_DEV_BAD_UPDATE);
     }
     if (P.selected)
-      for (int i = tid; i < ld; i += blockDim.x)
+      for (int i = tid; i < ld; i += THREADS)
         P.selected[loc * ld + i] = (i < L.j) ? cl[L.sel[i]] : -1;
     if (PROMOTE && tid == 0) {
       // smallest binary64 pivot v of the design: the factor's diagonal holds
@@ -516,16 +519,25 @@ cudaError_t launch_exh32(const DesignArgs& a, cudaStream_t s) {
   P.promote_count = a.ws->status + 1;
   size_t sm = smem_design32(a.n_max, a.p, a.PP, a.nc_max);
   const bool sf = d32_smem_factor(a.n_max);
-  auto k = P.promote ? (sf ? design32<true, true> : design32<true, false>)
-                     : (sf ? design32<false, true> : design32<false, false>);
-  cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  int dev = 0, sms = 0;
+  cudaError_t err;
+  if ((err = cudaGetDevice(&dev)) != cudaSuccess ||
+      (err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+    return err;
+  const int threads = d32_threads(a.M, a.nc_max, sms);
+  auto pick = [&](auto k256, auto k128) { return threads == 256 ? k256 : k128; };
+  auto k = P.promote ? (sf ? pick(design32<true, true, 256>, design32<true, true, 128>)
+                           : pick(design32<true, false, 256>, design32<true, false, 128>))
+                     : (sf ? pick(design32<false, true, 256>, design32<false, true, 128>)
+                           : pick(design32<false, false, 256>, design32<false, false, 128>));
+  err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (err != cudaSuccess) return err;
-  const int64_t grid = persistent_grid(k, D32_THREADS, sm, a.M, exh_slots(a.ws->chunk), 1,
+  const int64_t grid = persistent_grid(k, threads, sm, a.M, exh_slots(a.ws->chunk), 1,
                                        a.tune.exh_occ);
   if (grid < 0) return cudaErrorInvalidValue;
   if ((err = cudaMemsetAsync(P.queue, 0, sizeof(unsigned), s)) != cudaSuccess) return err;
   prof_begin("design32_exhaustive", s);
-  k<<<(unsigned)grid, D32_THREADS, sm, s>>>(P);
+  k<<<(unsigned)grid, threads, sm, s>>>(P);
   prof_end(s);
   return cudaGetLastError();
 }

@@ -58,6 +58,17 @@ inline int warps_per_cta_for_residency(size_t warp_bytes, size_t smem_sm, size_t
 // locations 2.63 against 2.65 ms, at n = 33 3.19 against 3.37).
 inline int mle_threads(int n) { return n <= 24 ? 128 : 256; }
 
+// Threads of a block of the incremental exhaustive scorer, which has 1,024 per SM.
+// Four candidates per thread leave most of 256 threads idle for small N', and four
+// blocks per SM hide less of a step's latencies than eight: 20,000 locations (p = 4,
+// n = 50) take 6.2 with 128 threads and 8.9 ms with 256 at N' = 60, 13.6 and 18.5 at
+// 200, 15.6 and 20.4 at 512; 700 locations 0.69 and 0.92, 1.10 and 1.58, 1.36 and 1.86.
+// Batches that fit on the SMs either way: N' = 200 0.96 and 0.97 ms at 300 locations,
+// N' = 256 1.03 and 1.01, N' = 512 0.70 and 0.67 for one.
+inline int d32_threads(int64_t M, int nc_max, int64_t sms) {
+  return nc_max <= 200 || (nc_max <= 512 && M > 4 * sms) ? 128 : 256;
+}
+
 // Threads of a block of the exact ranking.  A short list is a chain of latencies
 // that more blocks per SM hide, and its network is short: 20,000 locations at p = 4
 // take 0.049 ms with 128 threads and 0.178 with 256 and a network of 256 at N' = 30,

@@ -44,3 +44,12 @@ def test_pilot_takes_a_block_per_location_where_that_was_faster(tmp_path):
              (152, 1250, 8): 1, (456, 6250, 8): 1, (1, 32768, 8): 1, (1024, 32768, 8): 1}
     got = values(tmp_path, ["knn_pilot_alone(%d, %d, %d, 152)" % k for k in sides])
     assert got == list(sides.values())
+
+
+def test_exhaustive_scorer_takes_small_blocks_for_few_candidates(tmp_path):
+    """(M, N'): four blocks of 256 threads per SM ran 700 locations at N' = 100 in
+    two waves, 1.33 times as long as six had in one."""
+    sides = {(700, 100): 128, (1, 60): 128, (20_000, 200): 128, (20_000, 512): 128, (700, 300): 128,
+             (300, 256): 256, (1, 512): 256, (20_000, 1000): 256, (700, 1000): 256}
+    got = values(tmp_path, ["d32_threads(%d, %d, 152)" % k for k in sides])
+    assert got == list(sides.values())
