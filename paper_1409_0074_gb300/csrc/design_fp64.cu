@@ -32,6 +32,7 @@
 #include "common.cuh"
 #include "kdtree.cuh"
 #include "lagp_internal.h"
+#include "launch_plan.h"
 #include "mul64.h"
 
 namespace lagp {
@@ -69,6 +70,7 @@ struct D64Params {
   const int32_t* list; // locations to solve (list[0 .. *count - 1]), or null: CTA b solves b
   const unsigned* count;
   double golden, tol3; // Brent: (3 - sqrt 5) / 2 and tol / 3
+  bool ints;           // exhaustive: products on the integer units (d64_ints)
   int full;            // ray snaps over all of X_N through the k-d tree
   KdView<double> kd;   // the tree in binary64 (full scope)
 };
@@ -235,6 +237,7 @@ __device__ int search_exhaustive(const D64Params& P, Loc& L, const int32_t* cl, 
                                  const double* Kc_loc, double* gap_out) {
   const int j = L.j, ld = P.n_max, p = P.p;
   const double onepg = __dadd_rn(1.0, P.g);
+  const bool fast = P.ints && L.fast;
   Top2 t;
   t.b1 = -1.0; t.b2 = -1.0; t.i1 = -1;
   for (int r = threadIdx.x; r < nc; r += blockDim.x) {
@@ -250,7 +253,7 @@ __device__ int search_exhaustive(const D64Params& P, Loc& L, const int32_t* cl, 
 #pragma unroll 2
       for (int k = 0; k < j; ++k, kc += P.nc_max) {
         const double b = *kc;
-        if (L.fast && safe64(b)) {
+        if (fast && safe64(b)) {
           const Mul64 bs = split_b(b);
 #pragma unroll
           for (int u = 0; u < 4; ++u)
@@ -767,9 +770,14 @@ cudaError_t launch_design_fp64(const DesignArgs& a, int search, cudaStream_t s,
   if (search == SEARCH_EXHAUSTIVE)
     warps = d64_small_batch(a, list != nullptr) ? D64_SMALL / 32 : D64_WARPS;
   size_t sm = smem_design64(a.n_max, a.p, a.nc_max, a.nrays, warps, a.full_scope != 0);
+  int dev = 0, sms = 0;
+  cudaError_t err;
+  if ((err = cudaGetDevice(&dev)) != cudaSuccess ||
+      (err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+    return err;
+  P.ints = list != nullptr || d64_ints(a.M, a.nc_max, sms);
   const int64_t grid = list ? (a.M < grid_cap ? a.M : grid_cap) : a.M;
   if (grid <= 0) return cudaSuccess;
-  cudaError_t err;
   void (*kern)(D64Params) = design64<SEARCH_RAY, D64_THREADS>;
   if (search == SEARCH_EXHAUSTIVE)
     kern = warps > D64_WARPS ? design64<SEARCH_EXHAUSTIVE, D64_SMALL>

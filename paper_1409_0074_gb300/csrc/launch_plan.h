@@ -58,6 +58,17 @@ inline int warps_per_cta_for_residency(size_t warp_bytes, size_t smem_sm, size_t
 // locations 2.63 against 2.65 ms, at n = 33 3.19 against 3.37).
 inline int mle_threads(int n) { return n <= 24 ? 128 : 256; }
 
+// Whether the binary64 exhaustive search forms its products on the integer units.
+// That halves what a term costs where the binary64 pipe is busy; where each of an SM's
+// four sub-partitions has candidates for one warp at most, a term costs its latency,
+// which is longer: with the pipe's products 100 locations (p = 4, n = 30) take 1.59
+// and with the integer units' 1.76 ms at N' = 60, 1.74 and 1.84 at 128, but 2.22 and
+// 2.00 at 200; 304 locations 1.76 and 1.96 at N' = 60, but 2.63 and 2.17 at 100.
+inline bool d64_ints(int64_t M, int nc_max, int64_t sms) {
+  const int64_t per_sm = (M + sms - 1) / sms;
+  return per_sm > 2 || per_sm * ((nc_max + 31) / 32) > 4;
+}
+
 // Threads of a block of the incremental exhaustive scorer, which has 1,024 per SM.
 // Four candidates per thread leave most of 256 threads idle for small N', and four
 // blocks per SM hide less of a step's latencies than eight: 20,000 locations (p = 4,

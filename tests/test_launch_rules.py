@@ -53,3 +53,12 @@ def test_exhaustive_scorer_takes_small_blocks_for_few_candidates(tmp_path):
              (300, 256): 256, (1, 512): 256, (20_000, 1000): 256, (700, 1000): 256}
     got = values(tmp_path, ["d32_threads(%d, %d, 152)" % k for k in sides])
     assert got == list(sides.values())
+
+
+def test_small_binary64_batches_use_the_pipe_s_products(tmp_path):
+    """(M, N'): one warp with candidates per sub-partition waits for the products,
+    which the integer units form later (1.25 and 1.38 ms of kernel at N' = 60)."""
+    sides = {(1, 60): 0, (152, 128): 0, (304, 60): 0, (100, 200): 1, (153, 100): 1, (456, 60): 1,
+             (2000, 30): 1, (1, 1000): 1}
+    got = values(tmp_path, ["d64_ints(%d, %d, 152)" % k for k in sides])
+    assert got == list(sides.values())
