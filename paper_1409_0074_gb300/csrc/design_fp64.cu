@@ -250,15 +250,27 @@ __device__ int search_exhaustive(const D64Params& P, Loc& L, const int32_t* cl, 
       const double* Ki = L.Kinv + i * ld;
       const double* kc = Kc_loc + r;
       double acc[4] = {0.0, 0.0, 0.0, 0.0};
+      if (fast) {
 #pragma unroll 2
-      for (int k = 0; k < j; ++k, kc += P.nc_max) {
-        const double b = *kc;
-        if (fast && safe64(b)) {
-          const Mul64 bs = split_b(b);
+        for (int k = 0; k < j; ++k, kc += P.nc_max) {
+          const double b = *kc;
+          if (safe64(b)) {
+            const Mul64 bs = split_b(b);
 #pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (u < nr) acc[u] = __dadd_rn(acc[u], mul_rn_int(Ki[u * ld + k], bs));
-        } else {
+            for (int u = 0; u < 4; ++u)
+              if (u < nr) acc[u] = __dadd_rn(acc[u], mul_rn_int(Ki[u * ld + k], bs));
+          } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (u < nr) acc[u] = __dadd_rn(acc[u], __dmul_rn(Ki[u * ld + k], b));
+          }
+        }
+      } else {
+        // four correlations in flight, for a lone warp waits for them (n = 100, N' = 128,
+        // one location: 31.1 ms, two in flight 39.2)
+#pragma unroll 4
+        for (int k = 0; k < j; ++k, kc += P.nc_max) {
+          const double b = *kc;
 #pragma unroll
           for (int u = 0; u < 4; ++u)
             if (u < nr) acc[u] = __dadd_rn(acc[u], __dmul_rn(Ki[u * ld + k], b));
@@ -765,16 +777,16 @@ cudaError_t launch_design_fp64(const DesignArgs& a, int search, cudaStream_t s,
   } else {
     std::memset(&P.kd, 0, sizeof(P.kd));
   }
-  // rays: a warp per ray, at least four for the steps the block shares
-  int warps = a.nrays < 4 ? 4 : (a.nrays < D64_WARPS ? a.nrays : D64_WARPS);
-  if (search == SEARCH_EXHAUSTIVE)
-    warps = d64_small_batch(a, list != nullptr) ? D64_SMALL / 32 : D64_WARPS;
-  size_t sm = smem_design64(a.n_max, a.p, a.nc_max, a.nrays, warps, a.full_scope != 0);
   int dev = 0, sms = 0;
   cudaError_t err;
   if ((err = cudaGetDevice(&dev)) != cudaSuccess ||
       (err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
     return err;
+  // rays: a warp per ray, at least four for the steps the block shares
+  int warps = a.nrays < 4 ? 4 : (a.nrays < D64_WARPS ? a.nrays : D64_WARPS);
+  if (search == SEARCH_EXHAUSTIVE)
+    warps = d64_small_batch(a, list != nullptr) ? D64_SMALL / 32 : d64_warps(a.M, a.n_max, a.nc_max, sms);
+  size_t sm = smem_design64(a.n_max, a.p, a.nc_max, a.nrays, warps, a.full_scope != 0);
   P.ints = list != nullptr || d64_ints(a.M, a.nc_max, sms);
   const int64_t grid = list ? (a.M < grid_cap ? a.M : grid_cap) : a.M;
   if (grid <= 0) return cudaSuccess;

@@ -58,6 +58,18 @@ inline int warps_per_cta_for_residency(size_t warp_bytes, size_t smem_sm, size_t
 // locations 2.63 against 2.65 ms, at n = 33 3.19 against 3.37).
 inline int mle_threads(int n) { return n <= 24 ? 128 : 256; }
 
+// Warps of a block of the binary64 exhaustive search (the few locations of a batch
+// that leaves at most one block per SM aside).  Candidates for four warps at most take
+// four, and twice the blocks fit: with four and with eight warps 2,000 locations take
+// 4.11 and 6.73 ms at n = N' = 30, 5.84 and 7.52 at N' = 60, n = 30, 342 and 347 at N' =
+// 128, n = 100; one location at N' = 60, n = 30 1.30 and 1.34.  Where the matrix update
+// is most of a step and the blocks are few, it wants the threads: 400 locations at N' =
+// 60, n = 50 7.29 and 6.27 ms (900 there 9.33 and 12.53), one at N' = 90, n = 60 8.39
+// and 6.67.
+inline int d64_warps(int64_t M, int n, int nc_max, int64_t sms) {
+  return nc_max <= 128 && (n <= 32 || M > 4 * sms) ? 4 : 8;
+}
+
 // Whether the binary64 exhaustive search forms its products on the integer units.
 // That halves what a term costs where the binary64 pipe is busy; where each of an SM's
 // four sub-partitions has candidates for one warp at most, a term costs its latency,

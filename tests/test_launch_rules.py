@@ -62,3 +62,12 @@ def test_small_binary64_batches_use_the_pipe_s_products(tmp_path):
              (2000, 30): 1, (1, 1000): 1}
     got = values(tmp_path, ["d64_ints(%d, %d, 152)" % k for k in sides])
     assert got == list(sides.values())
+
+
+def test_few_candidates_in_binary64_take_small_blocks(tmp_path):
+    """(M, n, N'): with eight warps whatever N', 1,300 locations at n = N' = 30 took
+    1.31 times as long as before their blocks needed more registers."""
+    sides = {(1300, 30, 30): 4, (1, 30, 60): 4, (2000, 100, 128): 4, (900, 50, 60): 4,
+             (400, 50, 60): 8, (1, 60, 90): 8, (2000, 50, 1000): 8, (2000, 20, 129): 8}
+    got = values(tmp_path, ["d64_warps(%d, %d, %d, 152)" % k for k in sides])
+    assert got == list(sides.values())
