@@ -8,7 +8,10 @@ n0 = 6, n = 50, N' = 1000, theta = 1, g = 1e-6, ray search with p = 8 rays,
 FP32 scoring and FP64 factor update.  Inputs are resident in HBM before the
 timed region; a 256 MB buffer is written before every step to flush L2.
 
-Prints one JSON line.  `value` is locations/sec over all ranks (weak scaling:
+Prints one JSON line on stdout: the headline (`LINE_KEYS`), about a kilobyte, so
+that a caller that keeps only the end of the output has all of it.  The complete
+record (per-kernel times, the other forms, serving) is one JSON line on stderr, or
+in the file of `--details`.  `value` is locations/sec over all ranks (weak scaling:
 every rank predicts its own M locations; there is no collective on the data
 path).  `--impl reference` times the FP64 CPU oracle instead, on a bounded
 sample per step.
@@ -63,6 +66,8 @@ def parse():
                     help="arrival window per rate of the serving form")
     ap.add_argument("--workload", default="sinusoid_8d", choices=["sinusoid_8d", "paper_2d"],
                     help="the timed workload: the 8-d headline or the 2-d grid of Sec 5.1")
+    ap.add_argument("--details", default=None,
+                    help="file for the complete record (default: one JSON line on stderr)")
     ap.add_argument("--mle-stages", type=int, default=0, choices=[0, 1, 2],
                     help="time designs coupled with local inference for theta (one or two "
                          "stages) instead of designs at a fixed theta")
@@ -858,6 +863,23 @@ def base_line(args, world, value, ms, w):
                        "parallelism": "locations sharded over %d rank(s)" % world}}
 
 
+# the headline line; of `roofline` and `cpu_baseline` the figures that it reports
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+             "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config", "clocks",
+             "gpu_launches", "e2e", "rmse")
+ROOFLINE_KEYS = ("kernel", "bound", "achieved", "peak", "unit", "frac")
+
+
+def headline(record):
+    line = {k: record[k] for k in LINE_KEYS if k in record}
+    if record.get("roofline"):
+        line["roofline"] = {k: record["roofline"][k] for k in ROOFLINE_KEYS
+                            if k in record["roofline"]}
+    if record.get("cpu_baseline"):
+        line["cpu_baseline"] = {k: record["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind")}
+    return line
+
+
 def main():
     args = parse()
     rank, world = dist_init(args)
@@ -920,7 +942,12 @@ def main():
     else:
         line["e2e"] = None
     if rank == 0:
-        print(json.dumps(line))
+        if args.details:
+            with open(args.details, "w") as fh:
+                json.dump(line, fh)
+        else:
+            print(json.dumps(line), file=sys.stderr)
+        print(json.dumps(headline(line)))
 
 
 if __name__ == "__main__":
