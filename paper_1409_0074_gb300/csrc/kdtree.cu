@@ -2,20 +2,23 @@
 //
 // Level L (0 .. D-1) orders the positions of every level-L node by the
 // node's split coordinate L mod p: one stable least-significant-digit radix
-// sort of the keys (node << 24 | coordinate in units of 2^-24 of the design's
-// box), 8 bits a pass, over all positions.  Sorting by node as the high digits
-// keeps every node's points in its own range, so after the last level each
-// node's children are the lower and upper halves of its range.  Ties in a key
-// keep the previous order, so the tree is deterministic; a query is exact for
-// any order, since every node keeps the exact box of its points (and 2^-24 of the
-// box is what the FP32 rows resolve away from its centre).  Then the tree-ordered
-// FP32 rows are gathered and the node boxes are formed from the leaves upwards.
+// sort of the keys (node << 32 | the coordinate's ordered bits), 8 bits a pass, over
+// all positions.  Sorting by node as the high digits keeps every node's points in
+// its own range, so after the last level each node's children are the lower and
+// upper halves of its range.  Ties in a key keep the previous order, so the tree is
+// deterministic.  A query is exact for any order, since every node keeps the exact
+// box of its points, but it takes a tree that separates them: with coordinates in
+// 2^-24 of the design's box (a pass less, 2.75 instead of 3.20 ms at N = 1e6, p = 8) a
+// design with half its points within 1e-8 of the box's centre had one key for all of
+// those, and the ray kernel's walks past them took 4.5 instead of 0.44 ms per 500
+// locations.  Then the tree-ordered FP32 rows are gathered and the node boxes are
+// formed from the leaves upwards.
 //
 // A pass (tile histograms, their scan, a stable scatter by one warp per tile) is
 // bound by the scatter's chain of dependent steps, so tiles are small (1,024
 // keys: about six warps per SM at N = 1e6), the next keys are loaded ahead, and
-// the scan takes a block per digit.  N = 1e6, p = 8: 2.75 ms; with tiles of 4,096,
-// 32-bit coordinates (a pass more per level) and one block for the scan, 10.6 ms.
+// the scan takes a block per digit.  N = 1e6, p = 8: 3.20 ms; with tiles of 4,096 and
+// one block for the scan, 10.6 ms.
 #include <cstdint>
 
 #include "kdtree.cuh"
@@ -57,14 +60,10 @@ void kd_carve(int64_t N, int p, int PP, char* base, KdTree* t) {
 }
 
 // keys of level `level`: the position's node (relative index within the level)
-// above 24 bits of coordinate `dim` (centred on the design's box, so within
-// half its extent of zero)
+// above the bits of coordinate `dim`, changed so that they order like the values
 __global__ void kd_keys(const int32_t* __restrict__ perm, const float* __restrict__ Xf, int64_t N,
-                        int PP, int level, int dim, int first, const double* __restrict__ lo_box,
-                        const double* __restrict__ hi_box, uint64_t* __restrict__ keys,
+                        int PP, int level, int dim, int first, uint64_t* __restrict__ keys,
                         int32_t* __restrict__ vals) {
-  const float ext = (float)(hi_box[dim] - lo_box[dim]);
-  const float unit = ext > 0.f ? 16777215.f / ext : 0.f, mid = 0.5f * ext;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t gi = first ? (int32_t)i : perm[i];
@@ -75,8 +74,8 @@ __global__ void kd_keys(const int32_t* __restrict__ perm, const float* __restric
       if (i < m) { hi = m; node = node << 1; }
       else { lo = m; node = (node << 1) | 1u; }
     }
-    const float u = (Xf[(int64_t)gi * PP + dim] + mid) * unit;
-    keys[i] = ((uint64_t)node << 24) | (uint32_t)fminf(fmaxf(u, 0.f), 16777215.f);
+    const uint32_t b = __float_as_uint(Xf[(int64_t)gi * PP + dim]);
+    keys[i] = ((uint64_t)node << 32) | (b ^ (b >> 31 ? 0xffffffffu : 0x80000000u));
     vals[i] = gi;
   }
 }
@@ -240,8 +239,8 @@ __global__ void kd_up(int level, int p, int PP, float* __restrict__ box32,
   }
 }
 
-cudaError_t launch_kd_build(const double* X, const float* Xf, const double* lo, const double* hi,
-                            int64_t N, int p, int PP, const KdTree& t, cudaStream_t s) {
+cudaError_t launch_kd_build(const double* X, const float* Xf, int64_t N, int p, int PP,
+                            const KdTree& t, cudaStream_t s) {
   const int D = t.D;
   if ((D + KD_FAN - 1) / KD_FAN > KD_STACK) return cudaErrorInvalidValue;
   const int nblk = rs_blocks(N);
@@ -250,12 +249,11 @@ cudaError_t launch_kd_build(const double* X, const float* Xf, const double* lo, 
   uint64_t* kb[2] = {t.keys, t.keys + N};
   for (int level = 0; level < D; ++level) {
     // keys into buffer 0 (values: the current order, identity at level 0)
-    kd_keys<<<g, 256, 0, s>>>(t.perm, Xf, N, PP, level, level % p, level == 0, lo, hi, kb[0],
-                              t.vals);
+    kd_keys<<<g, 256, 0, s>>>(t.perm, Xf, N, PP, level, level % p, level == 0, kb[0], t.vals);
     int cur = 0;                 // keys in kb[cur]; values in t.vals for cur = 0 at start
     int32_t* vcur = t.vals;
     int32_t* valt = t.perm;
-    const int passes = 3 + (level + 7) / 8;
+    const int passes = 4 + (level + 7) / 8;
     for (int ps = 0; ps < passes; ++ps) {
       const int shift = 8 * ps;
       rs_hist<<<nblk, 256, 0, s>>>(kb[cur], N, shift, t.hist);
@@ -269,7 +267,7 @@ cudaError_t launch_kd_build(const double* X, const float* Xf, const double* lo, 
     }
     if (vcur != t.perm) kd_copy<<<g, 256, 0, s>>>(vcur, t.perm, N);
   }
-  if (D == 0) kd_keys<<<g, 256, 0, s>>>(t.perm, Xf, N, PP, 0, 0, 1, lo, hi, kb[0], t.perm);
+  if (D == 0) kd_keys<<<g, 256, 0, s>>>(t.perm, Xf, N, PP, 0, 0, 1, kb[0], t.perm);
   kd_gather<<<g, 256, 0, s>>>(t.perm, Xf, N, PP, t.pts32);
   const int64_t nleaf = (int64_t)1 << D;
   kd_leaf_box<<<(unsigned)((nleaf * 32 + 255) / 256), 256, 0, s>>>(t.perm, t.pts32, X, N, p, PP,

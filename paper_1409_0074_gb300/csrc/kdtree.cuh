@@ -247,8 +247,7 @@ struct KdTree {
 
 size_t kd_bytes(int64_t N, int p, int PP);
 void kd_carve(int64_t N, int p, int PP, char* base, KdTree* t);
-// (lo, hi: the design's bounding box, the origin of Xf its centre)
-cudaError_t launch_kd_build(const double* X, const float* Xf, const double* lo, const double* hi,
-                            int64_t N, int p, int PP, const KdTree& t, cudaStream_t s);
+cudaError_t launch_kd_build(const double* X, const float* Xf, int64_t N, int p, int PP,
+                            const KdTree& t, cudaStream_t s);
 
 }  // namespace lagp
