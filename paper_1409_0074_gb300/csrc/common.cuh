@@ -158,35 +158,6 @@ __device__ __forceinline__ double dot64_ilp8(const double* u, const double* v, i
   return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
 }
 
-// sum_{i=k..j-1} u[i] * M[i * ld + k] (a column of a row-major matrix) in
-// binary64, eight accumulators as above
-__device__ __forceinline__ double coldot64_ilp8(const double* u, const double* M, int64_t ld, int k,
-                                                int j) {
-  double a[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  int i = k;
-  for (; i + 7 < j; i += 8) {
-#pragma unroll
-    for (int t = 0; t < 8; ++t) a[t] = fma(u[i + t], M[(int64_t)(i + t) * ld + k], a[t]);
-  }
-  for (; i < j; ++i) a[0] = fma(u[i], M[(int64_t)i * ld + k], a[0]);
-  return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-}
-
-// sum_{k=0..len-1} u[k] * v[k] in binary64 with four independent accumulators
-// (GB300's FP64 latency makes a single FMA chain the critical path).
-__device__ __forceinline__ double dot64_ilp(const double* u, const double* v, int len) {
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-  int k = 0;
-  for (; k + 3 < len; k += 4) {
-    a0 = fma(u[k], v[k], a0);
-    a1 = fma(u[k + 1], v[k + 1], a1);
-    a2 = fma(u[k + 2], v[k + 2], a2);
-    a3 = fma(u[k + 3], v[k + 3], a3);
-  }
-  for (; k < len; ++k) a0 = fma(u[k], v[k], a0);
-  return (a0 + a1) + (a2 + a3);
-}
-
 __device__ __forceinline__ double relgap64(double a, double b) {
   double m = fmax(fabs(a), fabs(b));
   if (m == 0.0) return 0.0;

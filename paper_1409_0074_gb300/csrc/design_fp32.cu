@@ -119,10 +119,6 @@ static __shared__ double d32_nit64;
 // start of row i of the packed inverse factor
 __device__ __host__ __forceinline__ int d32_tri(int i) { return i * (i + 1) / 2; }
 
-__device__ __forceinline__ float warp_sum(float v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 __device__ __forceinline__ double warp_sumd(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
@@ -211,8 +207,8 @@ __device__ bool add_point32(const D32Params& P, L32& L, const int32_t* cl, const
     else L.kx[j] = kv;
   }
   __syncthreads();
-  // l = L_j^{-1} k_j(x_new): four lanes per row, one for each of dot64_ilp's
-  // accumulators (the first also takes the remainder)
+  // l = L_j^{-1} k_j(x_new): four lanes per row, each with every fourth product (the
+  // first also with the remainder)
   for (int i = tid >> 2; i < ((j + 7) & ~7); i += THREADS / 4) {
     const int t = tid & 3, len = i + 1, len4 = len & ~3;
     const double* Li = Lg + d32_tri(i);

@@ -10,8 +10,8 @@
 // therefore reproducible bit for bit by any IEEE-754 implementation of the
 // same formulas in the same order.
 //
-// Both searches are bound by the binary64 pipe, which takes a warp's
-// instruction every 64 cycles per SM sub-partition.  The inner sums
+// Both searches are bound by the binary64 pipe, which takes a warp's addition or
+// product every 76 cycles per SM sub-partition.  The inner sums
 // acc = rn(acc + rn(K^{-1}_ik k_k)) therefore form their products on the
 // integer units (mul64.h, the same bits) while the pipe does the additions:
 // 95.6 against 165.2 ms for 777 exhaustive 4-d designs of 50 points (N' = 1000).
@@ -773,7 +773,7 @@ cudaError_t launch_design_fp64(const DesignArgs& a, int search, cudaStream_t s,
   if (P.full) {
     const KdTree& t = a.ws->kd;
     P.kd.box = t.box64; P.kd.stride = a.p; P.kd.p = a.p; P.kd.D = t.D; P.kd.N = a.N;
-    P.kd.perm = t.perm; P.kd.pts = a.X; P.kd.by_design = true;
+    P.kd.perm = t.perm; P.kd.pts = a.X;
   } else {
     std::memset(&P.kd, 0, sizeof(P.kd));
   }

@@ -140,7 +140,7 @@ __device__ __forceinline__ float xld1(uint32_t addr) {
 // row start of the packed factor
 __device__ __host__ __forceinline__ int xtri(int i) { return i * (i + 1) / 2; }
 
-// sum_{i=k..j-1} u[i] L_ik over the packed factor, in coldot64_ilp8's order
+// sum_{i=k..j-1} u[i] L_ik over the packed factor, in eight sums (as dot64_ilp8)
 __device__ __forceinline__ double xcoldot(const double* u, const double* L, int k, int j) {
   double a[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   int i = k;

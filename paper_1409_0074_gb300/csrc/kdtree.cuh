@@ -94,8 +94,7 @@ __device__ __forceinline__ KdTop<T> kd_warp_merge(KdTop<T> t) {
 }
 
 // A view of the tree for one arithmetic.  box: [kd_nodes(D)][2][stride] (lo
-// row, then hi row); point(pos, k): coordinate k of the point at tree
-// position pos; perm: tree position -> design index.
+// row, then hi row); perm: tree position -> design index.
 template <typename T>
 struct KdView {
   const T* box;
@@ -103,10 +102,6 @@ struct KdView {
   int64_t N;
   const int32_t* perm;
   const T* pts;        // FP32: tree-ordered rows [N][stride]; binary64: the design [N][p]
-  bool by_design;      // pts indexed by design index (binary64) or by position (FP32)
-  __device__ __forceinline__ T point(int64_t pos, int32_t gi, int k) const {
-    return by_design ? pts[(int64_t)gi * p + k] : pts[pos * stride + k];
-  }
 };
 
 // Squared distance from xs to the box of node c.

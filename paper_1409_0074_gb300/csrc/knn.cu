@@ -875,8 +875,9 @@ size_t knn_smem_stream(int PP) {
   return (size_t)2 * LAGP_KNN_TILE * PP * 4 + 2 * LAGP_KNN_TILE * 4 + KNN_WARPS * 256 * 4 + 16;
 }
 
-// Pilot thresholds pay where the design is large against N' and there is work
-// enough for the pilot's own 30 us.  Streams without and with them (pilot and
+// Pilot thresholds pay where the design is large against N' and the stream forms
+// distances enough to be worth the 30 us of the pilot and the empty redo; the line
+// lies between the sides measured.  Streams without and with them (pilot and
 // redo included): 5,000 locations at p = 8, N = 2 N' (4000) 321 us against 313,
 // N = 4 N' (4000) 567 against 240, N = 8 N' (1024) 128 against 104; at p = 4, 8
 // locations, N = 8 N': 60 against 69 us at 1024, 80 against 83 at 2000, 142

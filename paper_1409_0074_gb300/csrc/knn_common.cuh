@@ -87,6 +87,4 @@ __device__ __forceinline__ int warp_compact(KnnEntry* e, int cnt, float keep) {
   return out;
 }
 
-// squared FP32 distance of a design row to the 4 locations of a warp, in the
-// stream's form |q|^2 + |x|^2 - 2 q.x
 }  // namespace lagp

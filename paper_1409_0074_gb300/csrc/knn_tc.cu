@@ -1,6 +1,7 @@
 // knn_tc.cu -- kNN candidate filter with the distances on the tensor cores
 // (Gramacy & Haaland, Sec 2.2: the local search is restricted to the N'
-// nearest neighbours of x), used where the pilot thresholds apply (N >= 32 N').
+// nearest neighbours of x), used from N = 32 N' on, where few points pass the pilot's
+// threshold (knn.cu; a smaller design is streamed, from N = 4 N' on with a threshold too).
 //
 // Squared distances as one contraction.  With centred FP32 coordinates a
 // (location) and b (design point),
@@ -190,8 +191,7 @@ __device__ __forceinline__ void kt_put(float d, int32_t idx, KnnEntry* qb, int r
 }
 
 // The passes among four neighbouring distances; how many, and how many lie at
-// or below the pilot value.  Rare (some lane has two), and kept out of line: in
-// line it made the unrolled epilogue 40 KB of code.
+// or below the pilot value.  Rare: some lane has two.
 template <bool SPLIT>
 __device__ __forceinline__ int2 kt_put4(float4 d, float keep, float thr, int32_t idx, KnnEntry* qb,
                                      int room, int32_t* counter, int n) {

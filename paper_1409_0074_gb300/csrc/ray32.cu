@@ -29,7 +29,8 @@
 // point append and of Brent's step, loops left rolled unless their trip hides
 // a latency, and the k-d walk in an instantiation of its own (FULL), the
 // kernel's stalls for instructions fell from 1.3 to 0.6 per issue and its time
-// at the sizes above from 157 to 121.7 ms (143 ms before the register-held kz).
+// for 100,000 8-d locations (n = 50, N' = 1000, 8 rays) from 157 to 121.7 ms (143 ms
+// before the register-held kz).
 //
 // Scheduling.  The kernel is persistent: each warp takes the next location
 // from a device work counter until the queue is empty, optionally through a
@@ -263,7 +264,8 @@ __device__ __forceinline__ void warp_sum64_3(double& a, double& b, double& c) {
   c = __shfl_sync(0xffffffffu, s, 8);
 }
 
-// dot64_ilp with the next four loads in flight during four multiply-adds
+// sum_{k<len} u[k] v[k] in four sums (the first also takes the remainder), with the
+// next four loads in flight during four multiply-adds
 __device__ __forceinline__ double row_dot(const double* u, const double* v, int len) {
   double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
   double n0 = 0.0, n1 = 0.0, n2 = 0.0, n3 = 0.0;
@@ -871,7 +873,7 @@ cudaError_t launch_ray32(const DesignArgs& a, cudaStream_t s) {
   if (P.full) {
     const KdTree& t = a.ws->kd;
     P.kd.box = t.box32; P.kd.stride = a.PP; P.kd.p = a.p; P.kd.D = t.D; P.kd.N = a.N;
-    P.kd.perm = t.perm; P.kd.pts = t.pts32; P.kd.by_design = false;
+    P.kd.perm = t.perm; P.kd.pts = t.pts32;
   } else {
     std::memset(&P.kd, 0, sizeof(P.kd));
   }

@@ -19,8 +19,8 @@
 
 namespace lagp {
 
-// start of row i in the zero-padded FP32 row storage (rows of length
-// (i+1) rounded up to a multiple of 4)
+// start of row i if rows of i + 1 elements were only padded to quads: what the storage
+// below is measured against in the tests
 LAGP_HD int roff(int i) {
   const int a = i >> 2, b = i & 3;
   return 4 * (i + 2 * a * (a - 1) + a * b);
